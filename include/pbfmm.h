@@ -157,11 +157,8 @@ int pb_profile(pb_ctx* ctx, int enable);
  *                         per packed instruction (add/mul/fma .f32x2); 0: one
  *                         source per scalar instruction.  Same arithmetic per
  *                         pair, summation order of the partial sums differs.
- *   PB_OPT_M2L_TILE       row tile of the tensor-core M2L: 0 (default): 256
- *                         pairs per MMA on CTA pairs (tcgen05 cta_group::2)
- *                         where the operator size allows (n_pad >= 128), else
- *                         128; 1: 128 pairs per MMA, one CTA per operator
- *                         part.  A tile-shape knob of the autotuner (pb_tune).
+ *   PB_OPT_M2L_TILE       0 or 1: accepted for compatibility, without effect
+ *                         (the tensor-core M2L has one row tile, 128 pairs).
  *   PB_OPT_LIST_DIRECT    1 (default): in the FP32 applies without
  *                         target-normal derivatives (fmm_apply_pair and
  *                         fmm_apply on the packed kernels, PB_OPT_LEAF_PACKED
@@ -276,9 +273,10 @@ int fmm_tree_export_list(const fmm_tree* tree, int which, int64_t* off, int32_t*
  * buffers the call is asynchronous; with any host buffer it synchronises.
  * Operators for (kernel, kappa, p, tree size) are precomputed on first use
  * and cached in the tree.  With PB_MIXED and p in 2..6, 8 or 10 the M2L,
- * M2M, L2L and the check -> equivalent solves run on the tensor cores (TF32
- * split into hi + lo parts, three products per step; at p = 8 and 10 each
- * operator is split into parts that fit in shared memory); with p = 7 or 9
+ * M2M, L2L and the check -> equivalent solves run on the tensor cores (FP32
+ * operands split into hi + lo parts, scaled halves for the M2L and TF32 for
+ * the others, three products per step; at p = 8 and 10 each operator is
+ * split into parts that fit in shared memory); with p = 7 or 9
  * or PB_FP64 on the CUDA cores, the
  * M2L parallel over interaction pairs.  The M2L / M2M / L2L reductions make
  * the summation order run-dependent (~1e-7 in FP32, ~1e-16 in FP64);
@@ -467,12 +465,12 @@ int pb_tune_ncrit(pb_ctx* ctx, const float* xyz, int64_t n, int p, const int32_t
  * it builds the octree of xyz (host or device, float [n][3]) and times the
  * paired Laplace + Yukawa (kappa 0.125) single+double-layer apply
  * (fmm_apply_pair, mixed precision, order p; mean of 3 after a warm run,
- * CUDA events) with every combination of PB_OPT_LEAF_NT (2, 4) and
- * PB_OPT_M2L_TILE (0, 1).  On return the context's PB_OPT_LEAF_NT and
- * PB_OPT_M2L_TILE hold the fastest combination (on an error they keep their
- * values from before the call); *best_ncrit, *best_leaf_nt, *best_m2l_tile
- * and *best_ms (any of the last three may be NULL) receive it.  The tile
- * options change the summation order of partial sums only.  Synchronous. */
+ * CUDA events) with PB_OPT_LEAF_NT 2 and 4.  On return the context's
+ * PB_OPT_LEAF_NT holds the faster one and PB_OPT_M2L_TILE 0 (on an error
+ * both keep their values from before the call); *best_ncrit, *best_leaf_nt,
+ * *best_m2l_tile (0) and *best_ms (any of the last three may be NULL)
+ * receive the result.  The tile options change the summation order of
+ * partial sums only.  Synchronous. */
 int pb_tune(pb_ctx* ctx, const float* xyz, int64_t n, int p, const int32_t* candidates, int ncand, int* best_ncrit,
             int* best_leaf_nt, int* best_m2l_tile, double* best_ms);
 

@@ -46,18 +46,17 @@ void pbfmm_test_wait_limit(int64_t cycles);
 int pbfmm_test_radix_sort(const uint64_t* keys, const int32_t* vals, int64_t n, int bits, uint64_t* keys_out,
                           int32_t* vals_out);
 
-/* Kernel of the tensor-core M2L: mode 1 (the default) runs pairs of CTAs
- * (a cluster of two, whose MMAs of M = 256 take A rows and B columns from
- * both CTAs' shared memory) at n_pad >= 128, mode 0 one CTA per operator
- * part.  M2M, L2L and the check -> equivalent solves always use one CTA per
- * part.  Returns the previous mode.  Read at kernel launch. */
+/* Kernel that pbfmm_selftest_m2l_tc runs: mode 1 (the default) the M2L's
+ * (split halves, persistent CTAs), mode 0 that of M2M, L2L and the check ->
+ * equivalent solves (TF32, one CTA per item and operator part).  The applies
+ * are not affected.  Returns the previous mode. */
 int pbfmm_test_tc_pair(int mode);
 
-/* Launch properties of the CTA-pair kernel at npad 128, without launching
- * it: out[0] registers per thread, out[1] max threads per block, out[2]
- * static shared bytes, out[3] dynamic shared bytes of a launch, out[4] the
- * number of clusters of two such CTAs that can be resident at once (0: the
- * launch cannot run on this device).  PB_OK or PB_ECUDA. */
+/* Launch properties of the M2L kernel at npad 128, without launching it:
+ * out[0] registers per thread, out[1] max threads per block, out[2] static
+ * shared bytes, out[3] dynamic shared bytes of a launch, out[4] the number of
+ * CTAs that can be resident at once (0: the launch cannot run on this
+ * device).  PB_OK or PB_ECUDA. */
 int pbfmm_test_tc_pair_info(int* out);
 
 /* Eigendecomposition of a symmetric n x n matrix A (row-major, FP64) with
@@ -70,6 +69,11 @@ int pbfmm_test_sym_eig(int n, const double* A, double* w, double* V);
  * (host buffers: Q [nrows][npad], Op [npad][npad], D [nrows][npad]; npad in
  * {32, 64, 128, 160, 320, 512}).  PB_OK, PB_EINVAL or PB_ETIMEOUT. */
 int pbfmm_selftest_m2l_tc(int nrows, int npad, const float* Q, const float* Op, float* D);
+
+/* D[i][n ^ x_i] = sum_k Op[n][k] Q[i][k ^ x_i], x_i = xs[i] & 7, through the
+ * M2L kernel (host buffers as above): the reflected operators of even
+ * expansion orders.  PB_OK, PB_EINVAL or PB_ETIMEOUT. */
+int pbfmm_selftest_m2l_f16(int nrows, int npad, const float* Q, const float* Op, const int32_t* xs, float* D);
 
 #ifdef __cplusplus
 }

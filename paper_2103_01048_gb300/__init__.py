@@ -457,8 +457,8 @@ def _test_sym_eig(A):
 
 
 def _test_tc_pair_info():
-    """Launch properties of the CTA-pair kernel (npad 128): registers, max
-    threads per block, static and dynamic shared bytes, resident clusters."""
+    """Launch properties of the M2L kernel (npad 128): registers, max threads
+    per block, static and dynamic shared bytes, resident CTAs."""
     out = np.zeros(5, dtype=np.int32)
     rc = _lib.pbfmm_test_tc_pair_info(ptr(out))
     if rc != PB_OK:
@@ -467,8 +467,8 @@ def _test_tc_pair_info():
 
 
 def _test_tc_pair(mode):
-    """Select the tensor-core box-operator kernel (1: CTA pairs where
-    available, 0: one CTA per operator part); returns the previous mode."""
+    """Select the kernel of _selftest_m2l_tc (1: the M2L's, 0: the box
+    operators'); returns the previous mode."""
     return int(_lib.pbfmm_test_tc_pair(int(mode)))
 
 
@@ -495,6 +495,22 @@ def _selftest_m2l_tc(Q, Op):
     rc = _lib.pbfmm_selftest_m2l_tc(Q.shape[0], Q.shape[1], ptr(Q), ptr(Op), ptr(D))
     if rc != PB_OK:
         raise PBError(rc, "tensor-core M2L self-test failed")
+    return D
+
+
+_lib.pbfmm_selftest_m2l_f16.argtypes = [ctypes.c_int, ctypes.c_int, _P, _P, _P, _P]
+_lib.pbfmm_selftest_m2l_f16.restype = ctypes.c_int
+
+
+def _selftest_m2l_f16(Q, Op, xs):
+    """D[i, n ^ x] = sum_k Op[n, k] Q[i, k ^ x], x = xs[i], through the M2L kernel (float32 host arrays)."""
+    Q = np.ascontiguousarray(Q, np.float32)
+    Op = np.ascontiguousarray(Op, np.float32)
+    xs = np.ascontiguousarray(xs, np.int32)
+    D = np.zeros_like(Q)
+    rc = _lib.pbfmm_selftest_m2l_f16(Q.shape[0], Q.shape[1], ptr(Q), ptr(Op), ptr(xs), ptr(D))
+    if rc != PB_OK:
+        raise PBError(rc, "M2L self-test failed")
     return D
 
 

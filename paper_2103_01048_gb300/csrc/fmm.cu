@@ -15,14 +15,13 @@
 
 namespace pbfmm {
 
-bool m2l_tc_launch(const fmm_tree* T, const Operators& O, const float* Qu, float* Qd, int* err, cudaStream_t st);
+bool m2l_h_launch(const fmm_tree* T, const Operators& O, const Operators* O2, const float* Qu, float* Qd, float* tmp,
+                  const float* Qu2, float* Qd2, float* tmp2, int* err, cudaStream_t st);
 bool pc_tc_launch(const fmm_tree* T, const Operators& O, int child_level, bool up, float* Q, int* err,
                   cudaStream_t st);
 bool c2e_tc_launch(const fmm_tree* T, const Operators& O, bool up, const float* X, float* Y, float* tmp, int* err,
                    cudaStream_t st, bool xfar = false);
 // two operator sets (Laplace, Yukawa) in the same launches
-bool m2l_tc_launch2(const fmm_tree* T, const Operators& O, const Operators* O2, const float* Qu, float* Qd,
-                    const float* Qu2, float* Qd2, int* err, cudaStream_t st);
 bool pc_tc_launch2(const fmm_tree* T, const Operators& O, const Operators* O2, int child_level, bool up, float* Q,
                    float* Q2, int* err, cudaStream_t st);
 bool c2e_tc_launch2(const fmm_tree* T, const Operators& O, const Operators* O2, bool up, const float* X, float* Y,
@@ -1413,7 +1412,7 @@ template <typename T>
 struct Work {
     DBuf<typename V4<T>::type> sq, sm, tn;
     DBuf<T> Qu, Qd, chk, pot, dn;
-    DBuf<T> tmp;          // FP32 path: intermediate of the factored check -> equivalent solves
+    DBuf<T> tmp;          // FP32 path: intermediate of the factored check -> equivalent solves, M2L source rows
 };
 
 template <typename T, typename TO, int NPAD>
@@ -1590,8 +1589,9 @@ static void far_m2l(fmm_tree* Tr, const Operators& O, Work<T>& W) {
     pb_ctx* ctx = Tr->ctx;
     bool tc_done = false;
     if constexpr (std::is_same<T, float>::value) {
-        if (Tr->m2l_pairs.nitems > 0 && !ctx->deterministic)
-            tc_done = m2l_tc_launch(Tr, O, W.Qu.p, W.Qd.p, ctx->dev_err, ctx->stream);
+        if (!ctx->deterministic)
+            tc_done = m2l_h_launch(Tr, O, nullptr, W.Qu.p, W.Qd.p, W.tmp.p, nullptr, nullptr, nullptr, ctx->dev_err,
+                                   ctx->stream);
     }
     if (!tc_done && !ctx->deterministic && Tr->m2l_pairs.nitems32 > 0) {
         // one CTA per at most 32 V-list pairs of one (level, offset) group:
@@ -1683,8 +1683,8 @@ template <typename T>
 static void far_pair_m2l(fmm_tree* Tr, const Operators& OL, const Operators& OY, Work<T>& WL, Work<T>& WY) {
     pb_ctx* ctx = Tr->ctx;
     if constexpr (std::is_same<T, float>::value) {
-        if (Tr->m2l_pairs.nitems > 0 && !ctx->deterministic &&
-            m2l_tc_launch2(Tr, OL, &OY, WL.Qu.p, WL.Qd.p, WY.Qu.p, WY.Qd.p, ctx->dev_err, ctx->stream))
+        if (!ctx->deterministic && m2l_h_launch(Tr, OL, &OY, WL.Qu.p, WL.Qd.p, WL.tmp.p, WY.Qu.p, WY.Qd.p, WY.tmp.p,
+                                                ctx->dev_err, ctx->stream))
             return;
     }
     far_m2l(Tr, OL, WL);
@@ -1693,14 +1693,15 @@ static void far_pair_m2l(fmm_tree* Tr, const Operators& OL, const Operators& OY,
 
 // equivalent densities and check potentials of one kernel
 template <typename T>
-static void alloc_far(Work<T>& W, size_t nbox_npad, cudaStream_t st) {
+static void alloc_far(Work<T>& W, size_t nbox, int npad, cudaStream_t st) {
+    const size_t nbox_npad = nbox * npad;
     W.Qu.alloc(nbox_npad, st);
     W.Qd.alloc(nbox_npad, st);
     W.chk.alloc(nbox_npad, st);
     W.Qu.zero(st);
     W.Qd.zero(st);
     W.chk.zero(st);
-    if (std::is_same<T, float>::value) W.tmp.alloc(nbox_npad, st);
+    if (std::is_same<T, float>::value) W.tmp.alloc(nbox_npad + nbox, st);     // + a scale per box
 }
 
 template <typename T, typename In, bool YUK>
@@ -1718,7 +1719,7 @@ static void apply_t(fmm_tree* Tr, const Operators& O, double kappa_d, const In* 
     Work<T> W;
     W.sq.alloc(ns, st);
     if (DL) W.sm.alloc(ns, st);
-    alloc_far(W, (size_t)Tr->nbox * O.npad, st);
+    alloc_far(W, Tr->nbox, O.npad, st);
     W.pot.alloc(nt, st);
     if (DN) { W.dn.alloc(nt, st); W.tn.alloc(nt, st); }
     pb_ctx* ctx = Tr->ctx;
@@ -1880,8 +1881,8 @@ static void apply_pair_t(fmm_tree* Tr, const Operators& OL, const Operators& OY,
     Work<T> WL, WY;
     WL.sq.alloc(ns, st);
     WL.sm.alloc(ns, st);
-    alloc_far(WL, (size_t)Tr->nbox * OL.npad, st);
-    alloc_far(WY, (size_t)Tr->nbox * OY.npad, st);
+    alloc_far(WL, Tr->nbox, OL.npad, st);
+    alloc_far(WY, Tr->nbox, OY.npad, st);
     WL.pot.alloc(nt, st);
     WY.pot.alloc(nt, st);
     if (DN) { WL.dn.alloc(nt, st); WY.dn.alloc(nt, st); WL.tn.alloc(nt, st); }

@@ -27,15 +27,19 @@ struct Operators {
     DBuf<float> uc2ue_w1, uc2ue_w2, dc2de_w1, dc2de_w2;   // [nlev][npad^2]
     DBuf<float> m2m, l2l;         // [nlev][8][npad^2]  (child level index)
     DBuf<float> m2l;              // [nlev][343][npad^2]
-    // tensor-core M2L: per level and offset (Laplace: one level), the
-    // operator split into TF32 hi + lo parts, pre-swizzled (128B swizzle,
-    // K-major) per part of its rows and inner columns:
-    // [level][343][part][hi|lo][K blocks][rows of the part][128 B]
-    DBuf<float> m2l_tc;
-    DBuf<float> m2m_tc, l2l_tc;   // same packing, [level][8 octants]
+    // tensor-core M2L (m2l_f16.cu): per level (Laplace: one) and slot (even p:
+    // |offset|, 64; odd p: offset, 343) the operator as hi + lo halves and
+    // the inverse of its scale: [operator][part][K block][rows][128 B]
+    DBuf<uint8_t> m2l_h;
+    DBuf<float> m2l_h_inv;
+    int h_nslot = 0;
+    bool h_single = false;
+    // M2M / L2L per level and octant, split into TF32 hi + lo parts,
+    // pre-swizzled (128B swizzle, K-major) per part of its rows and inner
+    // columns: [level][8][part][hi|lo][K blocks][rows of the part][128 B]
+    DBuf<float> m2m_tc, l2l_tc;
     DBuf<float> uc2ue_w1_tc, uc2ue_w2_tc, dc2de_w1_tc, dc2de_w2_tc;   // same packing, [level]
     bool have_tc = false;
-    bool m2l_tc_single = false;   // Laplace: m2l_tc holds one level (the operators are level-invariant)
     // FP64 copies (all-FP64 path)
     DBuf<double> uc2ue_d, dc2de_d, m2m_d, l2l_d, m2l_d;
     bool have_d = false;

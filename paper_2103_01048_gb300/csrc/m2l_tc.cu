@@ -1,26 +1,25 @@
-// M2L on the 5th-generation tensor cores (tcgen05, TMEM accumulators).
+// Box-operator products on the 5th-generation tensor cores (tcgen05, TMEM
+// accumulators): M2M, L2L and the check -> equivalent solves; and the pair
+// lists of the tree passes (the M2L itself: m2l_f16.cu).
 //
-// The V-list pairs (Sec. "Fast multipole method": interaction list I(B)) are
-// grouped by (level, relative offset): all pairs of a group share one M2L
-// operator (with the DC2DE solve folded in, FP64-built, FP32-stored).  A CTA
-// owns one group chunk and one part of the operator: a block of its output
-// rows times a block of its inner columns (two row halves up to p = 6;
-// 4 x 2 parts at p = 8, 4 x 4 at p = 10), so that the part fits in shared
-// memory:
+// All pairs of an item share one operator (FP64-built, FP32-stored).  A CTA
+// owns one item and one part of the operator: a block of its output rows
+// times a block of its inner columns (two row halves up to p = 6; 4 x 2
+// parts at p = 8, 4 x 4 at p = 10), so that the part fits in shared memory:
 //   * the operator part, split into TF32 hi + lo parts and pre-swizzled in
 //     global memory (128B swizzle, K-major), is copied into shared memory
 //     once with cp.async.bulk and stays resident;
 //   * 128-pair row tiles stream through: the producer threads gather the
-//     source boxes' upward densities (the part's columns of the Qu rows),
-//     split them into TF32 hi + lo and write them swizzled into a ring of
-//     A stages;
+//     source rows (the part's columns), split them into TF32 hi + lo and
+//     write them swizzled into a ring of A stages;
 //   * one thread issues tcgen05.mma kind::tf32 (M = 128 pairs, N = the
 //     part's rows, K = 8 per instruction), three products per k-step
 //     (hi*hi + hi*lo + lo*hi: FP32-level accuracy), accumulating in TMEM;
 //   * the epilogue reads the accumulator with tcgen05.ld and adds each row
-//     into the target box's downward density with red.global.add.v4.f32
-//     (targets of one group are distinct; groups and inner parts overlap,
-//     hence the reduction).  Summation order across groups is not fixed.
+//     into the target row with red.global.add.v4.f32 (targets of one item
+//     are distinct; items and inner parts overlap, hence the reduction).
+// TF32 and not scaled halves: the factors of the check -> equivalent solves
+// span 14 decades, more than a common scale per row can hold.
 // Every wait is bounded (~1 s); on a timeout the kernel records an error
 // code, drains its own MMAs, frees TMEM and returns.
 #include "fmm.cuh"
@@ -29,7 +28,6 @@
 #include <algorithm>
 #include <atomic>
 #include <cstdio>
-#include <memory>
 
 namespace pbfmm {
 
@@ -37,9 +35,9 @@ void radix_sort_pairs(const unsigned* keys_in, const int* vals_in, unsigned* key
                       int bits, cudaStream_t st);
 
 constexpr int kTcRows = 128;           // pairs per row tile (MMA M)
-constexpr int kTcItemPairs = 2048;     // pairs per M2L work item (one operator load each)
+constexpr int kM2LSegBoxes = 8192;     // target boxes of one segment of the M2L pair list
+constexpr int kTcItemPairs = 2048;     // pairs per self-test item
 constexpr int kTcSmallItemPairs = 512; // M2M / L2L / check->equivalent items: fewer pairs per operator, more CTAs
-constexpr int kTcOffItemPairs = 8192;  // items of a level-invariant M2L set (one offset, all levels)
 
 // Operator split per padded size: NS parts of the output rows (MMA N =
 // npad / NS) times KS parts of the inner dimension (npad / KS columns,
@@ -95,16 +93,9 @@ static void pack_tc(int npad, long long nmat, const float* src, DBuf<float>& dst
     PB_CHECK_LAUNCH();
 }
 
-// Laplace M2L operators (the down-check -> down-equivalent solve folded in)
-// do not depend on the level: the 1/r kernel scales as 2^l with the box
-// size and the regularised pseudo-inverse as 2^-l.  Their tensor-core copy
-// keeps one level (the first with interaction lists), indexed by offset.
-void pack_m2l_tc(Operators& O, cudaStream_t st) {
+void pack_box_ops_tc(Operators& O, cudaStream_t st) {
     int ns = 0, ks = 0;
     if (!tc_split(O.npad, ns, ks)) { O.have_tc = false; return; }
-    O.m2l_tc_single = O.kernel == FMM_LAPLACE && O.nlev > 2;
-    if (O.m2l_tc_single) pack_tc(O.npad, kNumOffsets, O.m2l.p + 2LL * kNumOffsets * O.npad * O.npad, O.m2l_tc, st);
-    else pack_tc(O.npad, (long long)O.nlev * kNumOffsets, O.m2l.p, O.m2l_tc, st);
     if (O.m2m.p) pack_tc(O.npad, (long long)O.nlev * 8, O.m2m.p, O.m2m_tc, st);
     if (O.l2l.p) pack_tc(O.npad, (long long)O.nlev * 8, O.l2l.p, O.l2l_tc, st);
     if (O.uc2ue_w1.p) {
@@ -127,17 +118,24 @@ __global__ void k_pairs_emit(int nbox, const int* V, const int* V_n, const int* 
     for (int i = 0; i < V_n[b]; ++i) {
         int s = V[(long long)b * kVCap + i];
         int4 as = anchor[s];
-        int o = (as.x - ab.x + 3) * 49 + (as.y - ab.y + 3) * 7 + (as.z - ab.z + 3);
+        const int ox = as.x - ab.x, oy = as.y - ab.y, oz = as.z - ab.z;
+        const int slot = abs(ox) * 16 + abs(oy) * 4 + abs(oz);
+        const int sign = (ox < 0 ? 4 : 0) | (oy < 0 ? 2 : 0) | (oz < 0 ? 1 : 0);
         int e = V_off[b] + i;
-        key[e] = o * 32 + ab.w;            // offset-major, then level (< 22)
+        key[e] = (((b / kM2LSegBoxes) * 64 + slot) * 32 + ab.w) * 8 + sign;   // segment, |offset|, level (< 22), signs
         tgt[e] = b;
         src[e] = s;
     }
 }
 
-__global__ void k_gather_int(int n, const int* idx, const int* a, int* out) {
+__global__ void k_pairs_gather(int n, const int* idx, const int* key, const int* t, const int* s, int* tgt, int* src,
+                               int* srcx) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = a[idx[i]];
+    if (i >= n) return;
+    const int k = idx[i], sb = s[k];
+    tgt[i] = t[k];
+    src[i] = sb;
+    srcx[i] = sb | (key[i] & 7) << 28;
 }
 
 void build_m2l_pairs(fmm_tree* T) {
@@ -146,8 +144,9 @@ void build_m2l_pairs(fmm_tree* T) {
     const long long np = T->n_v;
     auto& P = T->m2l_pairs;
     P.npairs = np;
-    P.nitems = 0;
+    P.nitems32 = P.ntile_even = P.ntile_odd = P.nseg = 0;
     if (np == 0) return;
+    PB_REQUIRE(nb < (1 << 28), PB_EINVAL, "octree has too many boxes for the interaction pair lists");
     DBuf<int> voff, key, tgt, src, idx, key_s, idx_s;
     voff.alloc(nb + 1, st);
     {
@@ -164,57 +163,65 @@ void build_m2l_pairs(fmm_tree* T) {
     std::vector<int> hidx(np);
     for (long long i = 0; i < np; ++i) hidx[i] = (int)i;
     PB_CUDA(cudaMemcpyAsync(idx.p, hidx.data(), np * sizeof(int), cudaMemcpyHostToDevice, st));
-    // group by (offset, level) keeping each group in box order (stable sort;
-    // offset * 32 + level < 2^14)
-    radix_sort_pairs((const unsigned*)key.p, idx.p, (unsigned*)key_s.p, idx_s.p, np, 14, st);
+    // stable: each group keeps the box order
+    int bits = 14;
+    while ((nb - 1) / kM2LSegBoxes >> (bits - 14)) ++bits;
+    radix_sort_pairs((const unsigned*)key.p, idx.p, (unsigned*)key_s.p, idx_s.p, np, bits, st);
     P.tgt.alloc(np, st);
     P.src.alloc(np, st);
-    k_gather_int<<<div_up(np, 256), 256, 0, st>>>((int)np, idx_s.p, tgt.p, P.tgt.p);
-    k_gather_int<<<div_up(np, 256), 256, 0, st>>>((int)np, idx_s.p, src.p, P.src.p);
+    P.srcx.alloc(np, st);
+    k_pairs_gather<<<div_up(np, 256), 256, 0, st>>>((int)np, idx_s.p, key_s.p, tgt.p, src.p, P.tgt.p, P.src.p,
+                                                     P.srcx.p);
     PB_CHECK_LAUNCH();
     std::vector<int> hk(np);
     PB_CUDA(cudaMemcpyAsync(hk.data(), key_s.p, np * sizeof(int), cudaMemcpyDeviceToHost, st));
     PB_CUDA(cudaStreamSynchronize(st));
-    // work items: (first pair, pair count <= kTcItemPairs, operator index =
-    // level * 343 + offset, 0) per (offset, level) group; and per offset
-    // (all levels, <= kTcOffItemPairs pairs, operator index = offset) for a
-    // level-invariant operator set
-    std::vector<int4> items, items_off;
-    long long i = 0;
-    while (i < np) {
+    std::vector<int4> even, odd, items32;
+    std::vector<int> seg_even, seg_odd;
+    auto cut = [](std::vector<int4>& v, long long a, long long b, int step, int z) {
+        for (; a < b; a += step) v.push_back(make_int4((int)a, (int)std::min<long long>(step, b - a), z, 0));
+    };
+    for (long long i = 0; i < np;) {
+        // one (segment, |offset|, level): the runs of its signs, then the whole group
+        if (i == 0 || hk[i] >> 14 != hk[i - 1] >> 14) {
+            seg_even.push_back((int)even.size());
+            seg_odd.push_back((int)odd.size());
+        }
         long long j = i;
-        while (j < np && hk[j] == hk[i]) ++j;
-        const int off = hk[i] / 32, lvl = hk[i] % 32;
-        for (long long a = i; a < j; a += kTcItemPairs)
-            items.push_back(make_int4((int)a, (int)std::min<long long>(kTcItemPairs, j - a), lvl * kNumOffsets + off, 0));
+        while (j < np && hk[j] >> 3 == hk[i] >> 3) {
+            long long k = j;
+            while (k < np && hk[k] == hk[j]) ++k;
+            const int slot = (hk[j] >> 8) & 63, lev = (hk[j] >> 3) & 31, sg = hk[j] & 7;
+            const int o[3] = {slot >> 4, (slot >> 2) & 3, slot & 3};
+            const int off = ((sg & 4 ? -o[0] : o[0]) + 3) * 49 + ((sg & 2 ? -o[1] : o[1]) + 3) * 7 +
+                            ((sg & 1 ? -o[2] : o[2]) + 3);
+            cut(odd, j, k, 128, off * 32 + lev);
+            cut(items32, j, k, 32, lev * kNumOffsets + off);
+            j = k;
+        }
+        cut(even, i, j, 128, (hk[i] >> 3) & 2047);
         i = j;
     }
-    i = 0;
-    while (i < np) {
-        long long j = i;
-        while (j < np && hk[j] / 32 == hk[i] / 32) ++j;
-        for (long long a = i; a < j; a += kTcOffItemPairs)
-            items_off.push_back(make_int4((int)a, (int)std::min<long long>(kTcOffItemPairs, j - a), hk[i] / 32, 0));
-        i = j;
-    }
-    P.nitems_off = (int)items_off.size();
-    P.items_off.alloc(items_off.size(), st);
-    PB_CUDA(cudaMemcpyAsync(P.items_off.p, items_off.data(), items_off.size() * sizeof(int4), cudaMemcpyHostToDevice,
-                            st));
-    P.nitems = (int)items.size();
-    P.items.alloc(items.size(), st);
-    PB_CUDA(cudaMemcpyAsync(P.items.p, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
-    std::vector<int4> items32;
-    for (const int4& it : items)
-        for (int a = 0; a < it.y; a += 32) items32.push_back(make_int4(it.x + a, std::min(32, it.y - a), it.z, 0));
-    P.nitems32 = (int)items32.size();
-    P.items32.alloc(items32.size(), st);
-    PB_CUDA(cudaMemcpyAsync(P.items32.p, items32.data(), items32.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
+    P.nseg = (int)seg_even.size();
+    seg_even.push_back((int)even.size());
+    seg_odd.push_back((int)odd.size());
+    P.seg_even.alloc(seg_even.size(), st);
+    P.seg_odd.alloc(seg_odd.size(), st);
+    PB_CUDA(cudaMemcpyAsync(P.seg_even.p, seg_even.data(), seg_even.size() * sizeof(int), cudaMemcpyHostToDevice, st));
+    PB_CUDA(cudaMemcpyAsync(P.seg_odd.p, seg_odd.data(), seg_odd.size() * sizeof(int), cudaMemcpyHostToDevice, st));
+    auto up = [&](const std::vector<int4>& v, DBuf<int4>& d, int& n) {
+        n = (int)v.size();
+        d.alloc(v.size(), st);
+        PB_CUDA(cudaMemcpyAsync(d.p, v.data(), v.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
+    };
+    up(even, P.tiles_even, P.ntile_even);
+    up(odd, P.tiles_odd, P.ntile_odd);
+    up(items32, P.items32, P.nitems32);
     PB_CUDA(cudaStreamSynchronize(st));
 }
 
 // Items of the check -> equivalent solves on the tensor cores: the boxes of
-// each level (one row each) in chunks of at most kTcItemPairs.
+// each level (one row each) in chunks of at most kTcSmallItemPairs.
 static void level_items(const std::vector<int>& lvl_off, int nlev, DBuf<int4>& items, int& n, cudaStream_t st) {
     std::vector<int4> h;
     for (int l = 0; l < nlev; ++l)
@@ -328,21 +335,8 @@ struct TcSets {
     const float* ops[2];
     const float* X[2];
     float* Y[2];
-    int single[2];           // 1: the set holds one level of M2L operators, indexed by offset alone
     long long wait_limit;    // cycles a role waits on a barrier before giving up (set at launch)
-    int* trace;              // optional progress markers of the CTA-pair kernel (host-mapped), or null
-    int ncols;               // output columns that can be nonzero (n_e; the rest is padding); 0: all
 };
-
-// progress marker of the CTA-pair kernel (self-test diagnostics): slot k of
-// cluster rank r of the first cluster, written to host-mapped memory so it
-// stays readable after a failed launch
-__device__ __forceinline__ void tc_mark(int* trace, uint32_t rank, int k, int v) {
-    if (trace && blockIdx.y == 0 && blockIdx.x < 2 && blockIdx.z == 0) {
-        *(volatile int*)&trace[rank * 8 + k] = v;
-        __threadfence_system();
-    }
-}
 
 template <int NPAD>
 __global__ void __launch_bounds__(kTcThreads, 1) k_m2l_tc(const int4* __restrict__ items, const int* __restrict__ ptgt,
@@ -350,8 +344,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_m2l_tc(const int4* __restrict
                                                           int* __restrict__ err) {
     // Generic tensor-core box-operator product: for every pair p of the
     // item, Y[tgt[p]] += Op(item) X[src[p]] (Op resident for the CTA).
-    // Used for M2L (operator per level and offset), for M2M / L2L
-    // (operator per child level and octant) and for the factored
+    // Used for M2M / L2L (operator per child level and octant) and for the factored
     // check -> equivalent solves (operator per level).
     const float* __restrict__ ops = sets.ops[blockIdx.z];
     const float* __restrict__ Qu = sets.X[blockIdx.z];
@@ -378,7 +371,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_m2l_tc(const int4* __restrict
     const int part = blockIdx.y;                     // operator part: rows half, inner columns kpart
     const int half = part / KS, kpart = part % KS;
     const int first = it.x, npairs = it.y;
-    const int opi = sets.single[blockIdx.z] ? it.z % kNumOffsets : it.z;
+    const int opi = it.z;
     const int ntile = (npairs + kTcRows - 1) / kTcRows;
 
     if (tid == 0) {
@@ -547,313 +540,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_m2l_tc(const int4* __restrict
     if (warp == 0) tmem_dealloc(taddr, TCOLS);
 }
 
-// ---------------------------------------------------------------------------
-// CTA-pair variant (cluster of two CTAs, tcgen05 cta_group::2).  The two CTAs
-// of a cluster (consecutive along grid x: the pairs of tcgen05 cta_group::2
-// are formed along the cluster's x dimension) hold the two row parts
-// ns = 2 c and 2 c + 1 of the same inner
-// part and split every 256-pair row tile: CTA r gathers the tile's rows
-// r * 128 ... r * 128 + 127 into its own A stages.  The even CTA issues
-// MMAs of M = 256, N = 2 NH: A rows come from both CTAs' stages, B columns
-// from both CTAs' operator parts (the same shared-memory offsets in both),
-// and each CTA's tensor memory receives its own 128 rows x 2 NH columns.
-// Against the single-CTA kernel every source row is gathered once instead
-// of once per row part, and each A tile feeds twice the columns.
-//   producers and epilogues arrive (one per warp) on their own CTA's
-//   barriers; the odd CTA's warp 12 relays each completed event (operator
-//   part, full A stage, drained accumulator) to the even CTA's barrier with
-//   one cluster-scope arrival;
-//   MMA issuer (even CTA): commits to `empty` / `accf` of both CTAs.
-// Cluster barriers after the set-up and before the teardown keep every
-// remote arrival and MMA inside the lifetime of both CTAs.
-// ---------------------------------------------------------------------------
-template <int STAGES>
-struct TcPairSmem {
-    alignas(16) float epi[kTcEpiWarps][32][kTcEpiStride];
-    uint64_t barB, barBp, full[STAGES], empty[STAGES], accf[2], acce[2];
-    uint64_t pfull[STAGES], pacce[2];     // odd CTA: its warps' arrivals, relayed to the even CTA
-    uint32_t tmem_slot;
-    int failed;
-};
-
-// bounded wait on a barrier that threads of the other CTA arrive on
-__device__ __forceinline__ bool mbar_wait_cta_cl(uint64_t* bar, uint32_t parity, volatile int* failed,
-                                                 long long limit) {
-    long long t0 = clock64();
-    while (!mbar_try_wait_cluster(bar, parity)) {
-        if (*failed) return false;
-        if (clock64() - t0 > limit) {
-            *failed = 1;
-            return false;
-        }
-    }
-    return true;
-}
-
-template <int NPAD>
-__global__ void __launch_bounds__(kTcThreads, 1)
-    k_m2l_tc2(const int4* __restrict__ items, const int* __restrict__ ptgt, const int* __restrict__ psrc,
-              const TcSets sets, int* __restrict__ err) {
-    const float* __restrict__ ops = sets.ops[blockIdx.z];
-    const float* __restrict__ Qu = sets.X[blockIdx.z];
-    float* __restrict__ Qd = sets.Y[blockIdx.z];
-    const long long wl = sets.wait_limit;
-    constexpr int NS = TcCfg<NPAD>::NS, KS = TcCfg<NPAD>::KS, kTcStages = TcCfg<NPAD>::STAGES;
-    constexpr int NH = NPAD / NS;                    // operator rows held by this CTA
-    constexpr int NP = 2 * NH;                       // MMA N: the rows of the pair
-    constexpr int KC = NPAD / KS;                    // inner columns of this part
-    constexpr int KB = KC / 32;                      // K blocks of 32 tf32 (128 B)
-    constexpr int TILE = 2 * kTcRows;                // pairs per MMA row tile (M = 256)
-    static_assert(NS % 2 == 0 && NP % 16 == 0 && NP >= 32 && NP <= 256 && KC % 32 == 0, "CTA-pair split");
-    constexpr uint32_t B_SPLIT = KB * NH * 128;      // bytes of one of hi / lo
-    constexpr uint32_t A_SPLIT = kTcRows * 128;      // 16 KB
-    constexpr uint32_t ACOLS = NP <= 32 ? 32 : (NP <= 64 ? 64 : (NP <= 128 ? 128 : 256));
-    constexpr uint32_t TCOLS = 2 * ACOLS;
-    constexpr uint32_t IDESC = idesc_tf32_mn(256, NP);
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint8_t* sB = smem;                               // [hi|lo][KB][NH][128]
-    uint8_t* sA = smem + 2 * B_SPLIT;                 // [stage][hi|lo][128][128]
-    TcPairSmem<kTcStages>* S = (TcPairSmem<kTcStages>*)(sA + kTcStages * 2 * A_SPLIT);
-    volatile int* failed = &S->failed;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // grid (x: 2 x part pairs, y: items, z: operator sets), clusters of two along x
-    const uint32_t rank = cluster_ctarank();         // 0: issues the pair's MMAs
-    const int4 it = items[blockIdx.y];
-    const int c = blockIdx.x >> 1;                   // part pair: row-part pair nsp, inner part kpart
-    const int nsp = c / KS, kpart = c % KS;
-    const int part = (2 * nsp + (int)rank) * KS + kpart;
-    const int first = it.x, npairs = it.y;
-    const int opi = sets.single[blockIdx.z] ? it.z % kNumOffsets : it.z;
-    const int ntile = (npairs + TILE - 1) / TILE;
-    const int rofs = (int)rank * kTcRows;            // this CTA's rows of a tile
-    const int ncols = sets.ncols > 0 ? sets.ncols : NPAD;
-    static_assert(NP % (2 * kTcEpiLd) == 0, "epilogue chunks");
-
-    if (tid == 0) {
-        mbar_init(&S->barB, 1);
-        mbar_init(&S->barBp, 1);
-        // even CTA: its own warps arrive locally, the odd CTA's relay once
-        for (int q = 0; q < kTcStages; ++q) {
-            mbar_init(&S->full[q], kTcProdWarps + 1);
-            mbar_init(&S->empty[q], 1);
-            mbar_init(&S->pfull[q], kTcProdWarps);
-        }
-        for (int q = 0; q < 2; ++q) {
-            mbar_init(&S->accf[q], 1);
-            mbar_init(&S->acce[q], kTcEpiWarps + 1);
-            mbar_init(&S->pacce[q], kTcEpiWarps);
-        }
-        S->failed = 0;
-        fence_mbar_init();
-    }
-    if (warp == 0) {
-        tmem_alloc_pair(&S->tmem_slot, TCOLS);
-        tmem_relinquish_pair();
-    }
-    tc_fence_before();
-    __syncthreads();
-    cluster_sync_all();                              // both CTAs' barriers exist before any remote arrival
-    tc_fence_after();
-    const uint32_t taddr = S->tmem_slot;
-    if (tid == 0) {
-        tc_mark(sets.trace, rank, 0, 1);
-        tc_mark(sets.trace, rank, 1, (int)taddr);
-    }
-
-    // resident operator part: hi and lo, one bulk copy each
-    if (tid == 0) {
-        const uint8_t* gB = (const uint8_t*)ops + ((long long)opi * (NS * KS) + part) * (2LL * B_SPLIT);
-        mbar_arrive_expect_tx(&S->barB, 2 * B_SPLIT);
-        bulk_g2s(sB, gB, B_SPLIT, &S->barB);
-        bulk_g2s(sB + B_SPLIT, gB + B_SPLIT, B_SPLIT, &S->barB);
-    }
-
-    if (warp < kTcProdWarps) {
-        // ---- producers (as in the single-CTA kernel, on this CTA's rows)
-        const int l8 = lane & 7, rbase = warp * 4 + (lane >> 3);
-        auto src_of = [&](int tile, int i) -> int {
-            const int r = tile * TILE + rofs + i * 32 + rbase;
-            return (tile < ntile && r < npairs) ? psrc[first + r] : -1;
-        };
-        float4 v[KB][4];
-        int sn[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int s0 = src_of(0, i);
-            const float4* q4 = s0 >= 0 ? (const float4*)(Qu + (size_t)s0 * NPAD + kpart * KC) : nullptr;
-#pragma unroll
-            for (int kb = 0; kb < KB; ++kb) v[kb][i] = q4 ? q4[kb * 8 + l8] : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) sn[i] = src_of(1, i);
-        int g = 0;
-        for (int tile = 0; tile < ntile; ++tile) {
-#pragma unroll
-            for (int kb = 0; kb < KB; ++kb, ++g) {
-                const int s = g % kTcStages, n = g / kTcStages;
-                if (n > 0 && !mbar_wait_cta(&S->empty[s], (n - 1) & 1, failed, wl)) goto prod_done;
-                uint8_t* aHi = sA + (size_t)s * 2 * A_SPLIT;
-                uint8_t* aLo = aHi + A_SPLIT;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float4 x = v[kb][i];
-                    float4 h = make_float4(tf32_hi(x.x), tf32_hi(x.y), tf32_hi(x.z), tf32_hi(x.w));
-                    float4 l = make_float4(x.x - h.x, x.y - h.y, x.z - h.z, x.w - h.w);
-                    uint32_t off = sw128_off(i * 32 + rbase, l8 * 4);
-                    *(float4*)(aHi + off) = h;
-                    *(float4*)(aLo + off) = l;
-                }
-                fence_proxy_async();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(rank == 0 ? &S->full[s] : &S->pfull[s]);
-                if (tid == 0) tc_mark(sets.trace, rank, 5, g + 1);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float4* qn = sn[i] >= 0 ? (const float4*)(Qu + (size_t)sn[i] * NPAD + kpart * KC) : nullptr;
-                    v[kb][i] = qn ? qn[kb * 8 + l8] : make_float4(0.f, 0.f, 0.f, 0.f);
-                }
-            }
-#pragma unroll
-            for (int i = 0; i < 4; ++i) sn[i] = src_of(tile + 2, i);
-        }
-    prod_done:
-        __syncwarp();
-    } else if (warp < kTcProdWarps + kTcEpiWarps) {
-        // ---- epilogue: warp w reads TMEM lanes 32 (w % 4) ... + 31 of this CTA
-        const int q = warp & 3;
-        const int erow = q * 32 + lane;
-        for (int tile = 0; tile < ntile; ++tile) {
-            const int a = tile & 1, u = tile >> 1;
-            const int r = tile * TILE + rofs + erow;
-            const int t = r < npairs ? ptgt[first + r] : -1;
-            bool ok = mbar_wait_cta(&S->accf[a], u & 1, failed, wl);
-            if (!__all_sync(0xffffffffu, ok)) break;
-            tc_fence_after();
-            float (*buf)[kTcEpiStride] = S->epi[q];
-            const uint32_t tbase = taddr + ((uint32_t)(q * 32) << 16) + a * ACOLS;
-            // one 16-column chunk: transpose through shared memory so that a
-            // reduction instruction covers 8 rows x 64 B, skip padding columns
-            auto drain = [&](const uint32_t* r, int c0) {
-#pragma unroll
-                for (int cc = 0; cc < kTcEpiLd; cc += 4)
-                    *(float4*)&buf[lane][cc] = make_float4(__uint_as_float(r[cc]), __uint_as_float(r[cc + 1]),
-                                                           __uint_as_float(r[cc + 2]), __uint_as_float(r[cc + 3]));
-                __syncwarp();
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int rr = j * 8 + (lane >> 2), cc = (lane & 3) * 4;
-                    const float4 x = *(const float4*)&buf[rr][cc];
-                    const int tr = __shfl_sync(0xffffffffu, t, rr);
-                    const int col = nsp * NP + c0 + cc;
-                    if (tr >= 0 && col < ncols) red_add_v4(Qd + (size_t)tr * NPAD + col, x.x, x.y, x.z, x.w);
-                }
-                __syncwarp();
-            };
-            // the next chunk's TMEM load runs while the current one drains
-            uint32_t ra[kTcEpiLd], rb[kTcEpiLd];
-            tmem_ld16_issue(tbase, ra);
-            tmem_wait16(ra);
-#pragma unroll 1
-            for (int c0 = 0; c0 < NP; c0 += 2 * kTcEpiLd) {        // NP is a multiple of 32
-                tmem_ld16_issue(tbase + c0 + kTcEpiLd, rb);
-                drain(ra, c0);
-                tmem_wait16(rb);
-                if (c0 + 2 * kTcEpiLd < NP) tmem_ld16_issue(tbase + c0 + 2 * kTcEpiLd, ra);
-                drain(rb, c0 + kTcEpiLd);
-                if (c0 + 2 * kTcEpiLd < NP) tmem_wait16(ra);
-            }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(rank == 0 ? &S->acce[a] : &S->pacce[a]);
-            if (warp == kTcProdWarps && lane == 0) tc_mark(sets.trace, rank, 4, tile + 1);
-        }
-        __syncwarp();
-    } else if (rank == 0) {
-        // ---- MMA issuer of the pair
-        if (lane == 0) {
-            uint64_t* last = nullptr;
-            uint32_t last_par = 0;
-            int g = 0;
-            bool ok = mbar_wait_cta(&S->barB, 0, failed, wl) && mbar_wait_cta_cl(&S->barBp, 0, failed, wl);
-            tc_mark(sets.trace, rank, 2, ok ? 1 : -1);
-            for (int tile = 0; ok && tile < ntile; ++tile) {
-                const int a = tile & 1, u = tile >> 1;
-                if (u > 0 && !(ok = mbar_wait_cta_cl(&S->acce[a], (u - 1) & 1, failed, wl))) break;
-                const uint32_t dacc = taddr + a * ACOLS;
-                for (int kb = 0; kb < KB; ++kb, ++g) {
-                    const int s = g % kTcStages, n = g / kTcStages;
-                    if (!(ok = mbar_wait_cta_cl(&S->full[s], n & 1, failed, wl))) break;
-                    tc_fence_after();
-                    const uint32_t aH = smem_u32(sA + (size_t)s * 2 * A_SPLIT), aL = aH + A_SPLIT;
-                    const uint32_t bH = smem_u32(sB) + kb * NH * 128, bL = bH + B_SPLIT;
-#pragma unroll
-                    for (int ks = 0; ks < 4; ++ks) {
-                        const uint32_t acc0 = (kb > 0 || ks > 0) ? 1u : 0u;
-                        mma_tf32_pair(dacc, sw128_desc(aH + ks * 32), sw128_desc(bH + ks * 32), IDESC, acc0);
-                        mma_tf32_pair(dacc, sw128_desc(aH + ks * 32), sw128_desc(bL + ks * 32), IDESC, 1u);
-                        mma_tf32_pair(dacc, sw128_desc(aL + ks * 32), sw128_desc(bH + ks * 32), IDESC, 1u);
-                    }
-                    mma_commit_pair(&S->empty[s], 0x3);
-                    tc_mark(sets.trace, rank, 3, g + 1);
-                    last = &S->empty[s];
-                    last_par = n & 1;
-                }
-                if (!ok) break;
-                mma_commit_pair(&S->accf[a], 0x3);
-                last = &S->accf[a];
-                last_par = u & 1;
-            }
-            // after a failure: every MMA issued here has completed before TMEM is freed
-            if (!ok && last) mbar_wait(last, last_par);
-        }
-        __syncwarp();
-    } else {
-        // ---- odd CTA relays (one cluster-scope arrival per event instead
-        // of one per warp): lane 0 its operator part and its full A stages,
-        // lane 1 its drained accumulators, in the order the issuer needs them
-        if (lane == 0) {
-            bool ok = mbar_wait_cta(&S->barB, 0, failed, wl);
-            if (ok) mbar_arrive_cluster(mapa_shared(smem_u32(&S->barBp), 0));
-            tc_mark(sets.trace, rank, 2, ok ? 1 : -1);
-            for (int g = 0; ok && g < ntile * KB; ++g) {
-                const int s = g % kTcStages, n = g / kTcStages;
-                if ((ok = mbar_wait_cta(&S->pfull[s], n & 1, failed, wl)))
-                    mbar_arrive_cluster(mapa_shared(smem_u32(&S->full[s]), 0));
-            }
-        } else if (lane == 1) {
-            bool ok = true;
-            for (int tile = 0; ok && tile < ntile; ++tile) {
-                const int a = tile & 1, u = tile >> 1;
-                if ((ok = mbar_wait_cta(&S->pacce[a], u & 1, failed, wl)))
-                    mbar_arrive_cluster(mapa_shared(smem_u32(&S->acce[a]), 0));
-            }
-        }
-        __syncwarp();
-    }
-
-    tc_fence_before();
-    __syncthreads();
-    cluster_sync_all();                              // no remote arrival or MMA of the pair is pending
-    tc_fence_after();
-    if (tid == 0) {
-        tc_mark(sets.trace, rank, 7, S->failed);
-        tc_mark(sets.trace, rank, 6, 1);
-    }
-    if (tid == 0 && S->failed) {
-        atomicExch(err, 1);
-        mbar_wait(&S->barB, 0);         // the operator copy has landed before shared memory is released
-    }
-    if (warp == 0) tmem_dealloc_pair(taddr, TCOLS);
-}
-
-template <int NPAD>
-static constexpr size_t tc_pair_smem_bytes() {
-    using C = TcCfg<NPAD>;
-    return 1024 + 2 * (size_t)(NPAD / C::KS / 32) * (NPAD / C::NS) * 128 + C::STAGES * 2 * (size_t)kTcRows * 128 +
-           sizeof(TcPairSmem<C::STAGES>);
-}
-
 template <int NPAD>
 static constexpr size_t tc_smem_bytes() {
     using C = TcCfg<NPAD>;
@@ -862,15 +548,6 @@ static constexpr size_t tc_smem_bytes() {
 }
 static_assert(tc_smem_bytes<160>() <= 232448 && tc_smem_bytes<320>() <= 232448 && tc_smem_bytes<512>() <= 232448,
               "shared memory per CTA");
-static_assert(tc_pair_smem_bytes<160>() <= 232448 && tc_pair_smem_bytes<320>() <= 232448 &&
-                  tc_pair_smem_bytes<512>() <= 232448,
-              "shared memory per CTA");
-
-// Kernel choice: CTA pairs (k_m2l_tc2) where the operator size allows,
-// else one CTA per operator part (k_m2l_tc).
-static std::atomic<int> g_tc_pair{1};
-static bool tc_pair_for(int npad) { return g_tc_pair.load() != 0 && npad >= 128; }
-
 // opt in to the large shared-memory carve-out once per process, kernel and
 // device (not a stream operation, so it stays out of captured graphs)
 template <typename F>
@@ -885,35 +562,11 @@ static void smem_optin(F* kernel, size_t bytes, bool* done) {
 
 template <int NPAD>
 static void launch_tc_items(const int4* items, int nitems, const int* tgt, const int* src, const TcSets& sets,
-                            int nsets, int* err, cudaStream_t st, bool allow_pair) {
+                            int nsets, int* err, cudaStream_t st) {
     if (nitems <= 0) return;
     dim3 grid(nitems, TcCfg<NPAD>::NS * TcCfg<NPAD>::KS, nsets);
     TcSets s2 = sets;
     s2.wait_limit = g_wait_limit.load();
-    if constexpr (NPAD >= 128) {
-        if (allow_pair && tc_pair_for(NPAD)) {
-            static bool done[64] = {false};
-            const size_t sm = tc_pair_smem_bytes<NPAD>();
-            smem_optin(k_m2l_tc2<NPAD>, sm, done);
-            cudaLaunchAttribute attr[1];
-            attr[0].id = cudaLaunchAttributeClusterDimension;
-            attr[0].val.clusterDim.x = 2;                // the two row parts of a part pair
-            attr[0].val.clusterDim.y = 1;
-            attr[0].val.clusterDim.z = 1;
-            for (int i0 = 0; i0 < nitems; i0 += 65535) {  // items along grid y
-                cudaLaunchConfig_t cfg = {};
-                cfg.gridDim = dim3(TcCfg<NPAD>::NS * TcCfg<NPAD>::KS, std::min(65535, nitems - i0), nsets);
-                cfg.blockDim = dim3(kTcThreads);
-                cfg.dynamicSmemBytes = sm;
-                cfg.stream = st;
-                cfg.attrs = attr;
-                cfg.numAttrs = 1;
-                PB_CUDA(cudaLaunchKernelEx(&cfg, k_m2l_tc2<NPAD>, items + i0, tgt, src, s2, err));
-                PB_CHECK_LAUNCH();
-            }
-            return;
-        }
-    }
     static bool done[64] = {false};
     const size_t sm = tc_smem_bytes<NPAD>();
     smem_optin(k_m2l_tc<NPAD>, sm, done);
@@ -921,18 +574,15 @@ static void launch_tc_items(const int4* items, int nitems, const int* tgt, const
     PB_CHECK_LAUNCH();
 }
 
-// allow_pair: the launch may use the CTA-pair kernel (the M2L, whose work
-// items hold up to 2,048 pairs; the M2M / L2L / solve items are smaller and
-// keep one CTA per operator part)
 static bool tc_dispatch(int npad, const int4* items, int nitems, const int* tgt, const int* src, const TcSets& sets,
-                        int nsets, int* err, cudaStream_t st, bool allow_pair = false) {
+                        int nsets, int* err, cudaStream_t st) {
     switch (npad) {
-        case 32: launch_tc_items<32>(items, nitems, tgt, src, sets, nsets, err, st, allow_pair); return true;
-        case 64: launch_tc_items<64>(items, nitems, tgt, src, sets, nsets, err, st, allow_pair); return true;
-        case 128: launch_tc_items<128>(items, nitems, tgt, src, sets, nsets, err, st, allow_pair); return true;
-        case 160: launch_tc_items<160>(items, nitems, tgt, src, sets, nsets, err, st, allow_pair); return true;
-        case 320: launch_tc_items<320>(items, nitems, tgt, src, sets, nsets, err, st, allow_pair); return true;
-        case 512: launch_tc_items<512>(items, nitems, tgt, src, sets, nsets, err, st, allow_pair); return true;
+        case 32: launch_tc_items<32>(items, nitems, tgt, src, sets, nsets, err, st); return true;
+        case 64: launch_tc_items<64>(items, nitems, tgt, src, sets, nsets, err, st); return true;
+        case 128: launch_tc_items<128>(items, nitems, tgt, src, sets, nsets, err, st); return true;
+        case 160: launch_tc_items<160>(items, nitems, tgt, src, sets, nsets, err, st); return true;
+        case 320: launch_tc_items<320>(items, nitems, tgt, src, sets, nsets, err, st); return true;
+        case 512: launch_tc_items<512>(items, nitems, tgt, src, sets, nsets, err, st); return true;
         default: return false;
     }
 }
@@ -1031,73 +681,24 @@ bool c2e_tc_launch(const fmm_tree* T, const Operators& O, bool up, const float* 
     return c2e_tc_launch2(T, O, nullptr, up, X, Y, tmp, nullptr, nullptr, nullptr, err, st, xfar);
 }
 
-// M2L on the tensor cores for one or two operator sets; false when the
-// tensor-core path does not apply (caller uses the CUDA-core kernel)
-bool m2l_tc_launch2(const fmm_tree* T, const Operators& O, const Operators* O2, const float* Qu, float* Qd,
-                    const float* Qu2, float* Qd2, int* err, cudaStream_t st) {
-    if (!tc_ok(O) || (O2 && (!tc_ok(*O2) || O2->npad != O.npad))) return false;
-    if (T->m2l_pairs.nitems == 0) return true;
-    const auto& P = T->m2l_pairs;
-    const bool pair = T->ctx->m2l_tile == 0;       // PB_OPT_M2L_TILE: 256-pair tiles on CTA pairs
-    const bool single1 = O.m2l_tc_single, single2 = O2 && O2->m2l_tc_single;
-    if (!single1 && !single2) {
-        // both sets per (level, offset): one launch, grid z selects the set
-        TcSets sets{{O.m2l_tc.p, O2 ? O2->m2l_tc.p : nullptr}, {Qu, Qu2}, {Qd, Qd2}, {0, 0}, 0, nullptr, O.ne};
-        return tc_dispatch(O.npad, P.items.p, P.nitems, P.tgt.p, P.src.p, sets, O2 ? 2 : 1, err, st, pair);
-    }
-    // a level-invariant set takes the per-offset items (every level of an
-    // offset under one operator load); the other set its per-level items
-    auto one = [&](const Operators& o, const float* X, float* Y) {
-        TcSets sets{{o.m2l_tc.p, nullptr}, {X, nullptr}, {Y, nullptr}, {o.m2l_tc_single ? 1 : 0, 0}, 0, nullptr, o.ne};
-        if (o.m2l_tc_single && P.nitems_off > 0)
-            return tc_dispatch(o.npad, P.items_off.p, P.nitems_off, P.tgt.p, P.src.p, sets, 1, err, st, pair);
-        return tc_dispatch(o.npad, P.items.p, P.nitems, P.tgt.p, P.src.p, sets, 1, err, st, pair);
-    };
-    if (!one(O, Qu, Qd)) return false;
-    return O2 ? one(*O2, Qu2, Qd2) : true;
-}
-
-bool m2l_tc_launch(const fmm_tree* T, const Operators& O, const float* Qu, float* Qd, int* err, cudaStream_t st) {
-    return m2l_tc_launch2(T, O, nullptr, Qu, Qd, nullptr, nullptr, err, st);
-}
-
 }  // namespace pbfmm
 
 // ---------------------------------------------------------------------------
-// Self-test hook (not part of the documented ABI): D = Q Op^T for one
-// operator through the tensor-core M2L kernel, host buffers.
+// Self-test hooks (not part of the documented ABI)
 // ---------------------------------------------------------------------------
+namespace pbfmm {
+static std::atomic<int> g_selftest_h{1};
+bool m2l_h_supported(int npad);
+void m2l_h_selftest(int nrows, int npad, const float* Q, const float* Op, const int* xs, float* D, int* err,
+                    cudaStream_t st);
+void m2l_h_info(int* out);
+}  // namespace pbfmm
 using namespace pbfmm;
-extern "C" int pbfmm_test_tc_pair(int mode) { return g_tc_pair.exchange(mode ? 1 : 0); }
+extern "C" int pbfmm_test_tc_pair(int mode) { return g_selftest_h.exchange(mode ? 1 : 0); }
 
-// launch properties of the CTA-pair kernel at npad 128 (no launch):
-// out = {registers, max threads per block, static shared bytes, dynamic
-// shared bytes requested, max co-resident clusters of two for that launch}
 extern "C" int pbfmm_test_tc_pair_info(int* out) {
     try {
-        static bool done[64] = {false};
-        const size_t sm = tc_pair_smem_bytes<128>();
-        smem_optin(k_m2l_tc2<128>, sm, done);
-        cudaFuncAttributes fa;
-        PB_CUDA(cudaFuncGetAttributes(&fa, k_m2l_tc2<128>));
-        cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 2;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.gridDim = dim3(2, 1, 1);
-        cfg.blockDim = dim3(kTcThreads);
-        cfg.dynamicSmemBytes = sm;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        int nclusters = -1;
-        PB_CUDA(cudaOccupancyMaxActiveClusters(&nclusters, k_m2l_tc2<128>, &cfg));
-        out[0] = fa.numRegs;
-        out[1] = fa.maxThreadsPerBlock;
-        out[2] = (int)fa.sharedSizeBytes;
-        out[3] = (int)sm;
-        out[4] = nclusters;
+        m2l_h_info(out);
         return PB_OK;
     } catch (const Error& e) {
         std::fprintf(stderr, "pbfmm_test_tc_pair_info: %s\n", e.what());
@@ -1110,60 +711,41 @@ extern "C" int pbfmm_selftest_m2l_tc(int nrows, int npad, const float* Q, const 
         int ns_, ks_;
         if (nrows < 1 || !tc_split(npad, ns_, ks_)) return PB_EINVAL;
         cudaStream_t st = nullptr;
-        fmm_tree T;
-        Operators O;
-        O.npad = npad;
-        O.nlev = 1;
-        DBuf<float> m2l, q, d;
+        DBuf<float> op, q, d;
         DBuf<int> e;
-        m2l.alloc((size_t)kNumOffsets * npad * npad, st);
-        m2l.zero(st);
-        PB_CUDA(cudaMemcpyAsync(m2l.p, Op, (size_t)npad * npad * 4, cudaMemcpyHostToDevice, st));   // offset slot 0
-        O.m2l.p = m2l.p;
-        pack_m2l_tc(O, st);
-        O.m2l.p = nullptr;
+        op.alloc((size_t)npad * npad, st);
+        PB_CUDA(cudaMemcpyAsync(op.p, Op, (size_t)npad * npad * 4, cudaMemcpyHostToDevice, st));
         q.alloc((size_t)nrows * npad, st);
         d.alloc((size_t)nrows * npad, st);
         d.zero(st);
         e.alloc(1, st);
         e.zero(st);
         PB_CUDA(cudaMemcpyAsync(q.p, Q, (size_t)nrows * npad * 4, cudaMemcpyHostToDevice, st));
-        std::vector<int> id(nrows);
-        for (int i = 0; i < nrows; ++i) id[i] = i;
-        T.m2l_pairs.tgt.alloc(nrows, st);
-        T.m2l_pairs.src.alloc(nrows, st);
-        PB_CUDA(cudaMemcpyAsync(T.m2l_pairs.tgt.p, id.data(), nrows * 4, cudaMemcpyHostToDevice, st));
-        PB_CUDA(cudaMemcpyAsync(T.m2l_pairs.src.p, id.data(), nrows * 4, cudaMemcpyHostToDevice, st));
-        std::vector<int4> items;
-        for (int a = 0; a < nrows; a += kTcItemPairs) items.push_back(make_int4(a, std::min(kTcItemPairs, nrows - a), 0, 0));
-        // (operator index 0: level 0, offset slot 0)
-        T.m2l_pairs.nitems = (int)items.size();
-        T.m2l_pairs.items.alloc(items.size(), st);
-        PB_CUDA(cudaMemcpyAsync(T.m2l_pairs.items.p, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
-        // progress markers of the CTA-pair kernel in host-mapped memory
-        int* trace_h = nullptr;
-        int* trace_d = nullptr;
-        PB_CUDA(cudaHostAlloc((void**)&trace_h, 16 * sizeof(int), cudaHostAllocMapped));
-        std::unique_ptr<int, void (*)(int*)> trace_guard(trace_h, [](int* p) { cudaFreeHost(p); });
-        for (int i = 0; i < 16; ++i) trace_h[i] = 0;
-        PB_CUDA(cudaHostGetDevicePointer((void**)&trace_d, trace_h, 0));
-        try {
-            TcSets sets{{O.m2l_tc.p, nullptr}, {q.p, nullptr}, {d.p, nullptr}, {O.m2l_tc_single ? 1 : 0, 0}, 0,
-                        trace_d};
-            if (!tc_dispatch(O.npad, T.m2l_pairs.items.p, T.m2l_pairs.nitems, T.m2l_pairs.tgt.p, T.m2l_pairs.src.p,
-                             sets, 1, e.p, st, true))
-                return PB_EINVAL;
-            int herr = 0;
-            PB_CUDA(cudaMemcpyAsync(&herr, e.p, 4, cudaMemcpyDeviceToHost, st));
-            PB_CUDA(cudaMemcpyAsync(D, d.p, (size_t)nrows * npad * 4, cudaMemcpyDeviceToHost, st));
+        if (g_selftest_h.load() && m2l_h_supported(npad)) {
+            m2l_h_selftest(nrows, npad, q.p, op.p, nullptr, d.p, e.p, st);
+        } else {
+            DBuf<float> packed;
+            DBuf<int> ids;
+            DBuf<int4> ditems;
+            pack_tc(npad, 1, op.p, packed, st);
+            std::vector<int> id(nrows);
+            for (int i = 0; i < nrows; ++i) id[i] = i;
+            std::vector<int4> items;
+            for (int a = 0; a < nrows; a += kTcItemPairs)
+                items.push_back(make_int4(a, std::min(kTcItemPairs, nrows - a), 0, 0));
+            ids.alloc(nrows, st);
+            ditems.alloc(items.size(), st);
+            PB_CUDA(cudaMemcpyAsync(ids.p, id.data(), nrows * 4, cudaMemcpyHostToDevice, st));
+            PB_CUDA(cudaMemcpyAsync(ditems.p, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
+            TcSets sets{{packed.p, nullptr}, {q.p, nullptr}, {d.p, nullptr}, 0};
+            if (!tc_dispatch(npad, ditems.p, (int)items.size(), ids.p, ids.p, sets, 1, e.p, st)) return PB_EINVAL;
             PB_CUDA(cudaStreamSynchronize(st));
-            return herr ? PB_ETIMEOUT : PB_OK;
-        } catch (const Error& ex) {
-            std::fprintf(stderr, "pbfmm_selftest_m2l_tc: %s; pair-kernel markers:", ex.what());
-            for (int i = 0; i < 16; ++i) std::fprintf(stderr, " %d", ((volatile int*)trace_h)[i]);
-            std::fprintf(stderr, "\n");
-            throw;
         }
+        int herr = 0;
+        PB_CUDA(cudaMemcpyAsync(&herr, e.p, 4, cudaMemcpyDeviceToHost, st));
+        PB_CUDA(cudaMemcpyAsync(D, d.p, (size_t)nrows * npad * 4, cudaMemcpyDeviceToHost, st));
+        PB_CUDA(cudaStreamSynchronize(st));
+        return herr ? PB_ETIMEOUT : PB_OK;
     } catch (const Error& e) {
         return e.code;
     }

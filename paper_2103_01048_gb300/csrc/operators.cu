@@ -397,7 +397,8 @@ struct Builder {
 
 }  // namespace
 
-void pack_m2l_tc(Operators& O, cudaStream_t st);
+void pack_box_ops_tc(Operators& O, cudaStream_t st);
+void pack_m2l_h(Operators& O, cudaStream_t st);
 
 std::shared_ptr<Operators> get_operators(fmm_tree* T, int kernel, double kappa, int p, bool need_fp64) {
     auto key = std::make_tuple(kernel, kernel == FMM_YUKAWA ? kappa : 0.0, p, T->nlev);
@@ -424,17 +425,25 @@ std::shared_ptr<Operators> get_operators(fmm_tree* T, int kernel, double kappa, 
     O->npad = pad32(O->ne);
     O->nlev = T->nlev;
     const int n = O->ne, np = O->npad, L = T->nlev;
-    // unit surface: boundary points of the p x p x p grid on [-1, 1]^3
+    // unit surface: boundary points of the p x p x p grid on [-1, 1]^3.  Even
+    // p: orbits of the eight sign changes together, point 8 * orbit + sign
+    // bits (x: 4, y: 2, z: 1; 1 = negative), so that a reflection of the
+    // coordinates is an exclusive or of the point's number (m2l_f16.cu).
     std::vector<double> s;
     std::vector<float> sf;
-    for (int i = 0; i < p; ++i)
-        for (int j = 0; j < p; ++j)
-            for (int k = 0; k < p; ++k) {
-                if (i == 0 || j == 0 || k == 0 || i == p - 1 || j == p - 1 || k == p - 1) {
-                    double x = -1.0 + 2.0 * i / (p - 1), y = -1.0 + 2.0 * j / (p - 1), z = -1.0 + 2.0 * k / (p - 1);
-                    s.push_back(x); s.push_back(y); s.push_back(z);
-                    sf.push_back((float)x); sf.push_back((float)y); sf.push_back((float)z); sf.push_back(0.f);
-                }
+    auto put = [&](double x, double y, double z) {
+        s.push_back(x); s.push_back(y); s.push_back(z);
+        sf.push_back((float)x); sf.push_back((float)y); sf.push_back((float)z); sf.push_back(0.f);
+    };
+    const int i0 = p % 2 == 0 ? p / 2 : 0;
+    for (int i = i0; i < p; ++i)
+        for (int j = i0; j < p; ++j)
+            for (int k = i0; k < p; ++k) {
+                if (!(i == 0 || j == 0 || k == 0 || i == p - 1 || j == p - 1 || k == p - 1)) continue;
+                const double x = -1.0 + 2.0 * i / (p - 1), y = -1.0 + 2.0 * j / (p - 1), z = -1.0 + 2.0 * k / (p - 1);
+                if (i0 == 0) put(x, y, z);
+                else
+                    for (int m = 0; m < 8; ++m) put(m & 4 ? -x : x, m & 2 ? -y : y, m & 1 ? -z : z);
             }
     O->surf.alloc(s.size(), st);
     O->surf_f.alloc(sf.size(), st);
@@ -539,7 +548,8 @@ std::shared_ptr<Operators> get_operators(fmm_tree* T, int kernel, double kappa, 
         PB_CUDA(cudaMemcpyAsync(O->dc2de_w2.p, d2.data(), L * m2 * sizeof(float), cudaMemcpyHostToDevice, st));
         PB_CUDA(cudaStreamSynchronize(st));    // the host vectors go out of scope
     }
-    pack_m2l_tc(*O, st);
+    pack_box_ops_tc(*O, st);
+    pack_m2l_h(*O, st);
     PB_CUDA(cudaStreamSynchronize(st));
     T->ops[key] = O;
     auto& cache = T->ctx->op_cache;

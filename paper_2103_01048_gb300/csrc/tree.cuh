@@ -26,19 +26,21 @@ struct M2LSchedule {
     long long npairs = 0;              // total V-list pairs (algorithmic work)
 };
 
-// V-list pairs sorted by (level, offset) for the tensor-core M2L, cut into
-// work items (first pair, count <= 1024, level, offset).
+// V-list pairs sorted by (segment of 8,192 target boxes, |offset|, level,
+// signs of the offset), ascending target box inside a group.
 struct M2LPairs {
     DBuf<int> tgt, src;
-    DBuf<int4> items;
-    int nitems = 0;
+    DBuf<int> srcx;            // source box | sign bits of the offset << 28 (x: 4, y: 2, z: 1)
     long long npairs = 0;
-    DBuf<int4> items32;        // the same groups in chunks of at most 32 pairs (CUDA-core M2L)
+    DBuf<int4> items32;        // CUDA-core M2L: (first pair, count <= 32, level * 343 + offset, 0)
     int nitems32 = 0;
-    // items of a level-invariant operator set (Laplace): all levels of one
-    // offset together (the pairs are ordered by offset, then level)
-    DBuf<int4> items_off;
-    int nitems_off = 0;
+    // row tiles of the tensor-core M2L: (first pair, count <= 128, slot * 32
+    // + level, 0), slot = |offset| as 16 |x| + 4 |y| + |z| (even: one operator
+    // for the offsets that differ by signs) or the offset (odd)
+    DBuf<int4> tiles_even, tiles_odd;
+    int ntile_even = 0, ntile_odd = 0;
+    DBuf<int> seg_even, seg_odd;       // [nseg + 1] first tile of each segment
+    int nseg = 0;
 };
 
 // Parent-child pairs (children of level >= 3) grouped by (level, octant) for
