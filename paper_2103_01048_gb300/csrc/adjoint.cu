@@ -19,6 +19,7 @@
 // the same pairs, the transposed singular entries S^T, and the transposed
 // block preconditioner.
 #include "bem.cuh"
+#include "math64.cuh"
 #include <cmath>
 
 namespace pbfmm {
@@ -28,7 +29,7 @@ constexpr double kKcalA = 332.0637;
 
 template <typename T> __device__ __forceinline__ T rsqrt_a(T x);
 template <> __device__ __forceinline__ float rsqrt_a<float>(float x) { return rsqrtf(x); }
-template <> __device__ __forceinline__ double rsqrt_a<double>(double x) { return rsqrt(x); }
+template <> __device__ __forceinline__ double rsqrt_a<double>(double x) { return rsqrt64(x); }
 template <typename T> __device__ __forceinline__ T exp_a(T x);
 template <> __device__ __forceinline__ float exp_a<float>(float x) { return __expf(x); }
 template <> __device__ __forceinline__ double exp_a<double>(double x) { return exp(x); }
@@ -88,7 +89,7 @@ __global__ void k_adj_rhs(int nt, int nq, const double* __restrict__ qp, const d
                 double dx = s_a[k].x - x, dy = s_a[k].y - y, dz = s_a[k].z - z;
                 double r2 = dx * dx + dy * dy + dz * dz;
                 if (r2 <= 0) continue;
-                double ri = rsqrt(r2);
+                double ri = rsqrt64(r2);
                 sp += s_a[k].w * ri;
                 sd += s_a[k].w * (dx * nx + dy * ny + dz * nz) * ri * ri * ri;
             }
@@ -227,7 +228,7 @@ __global__ void k_atom_grad(int na, const double4* __restrict__ atoms, long long
             double dx = px - s_p[m][0], dy = py - s_p[m][1], dz = pz - s_p[m][2];
             double r2 = dx * dx + dy * dy + dz * dz;
             if (r2 <= 0) continue;
-            double ri = rsqrt(r2), ri3 = ri * ri * ri;
+            double ri = rsqrt64(r2), ri3 = ri * ri * ri;
             double mono = s_v[m][0] + s_v[m][2];          // monopole sources (reaction + adjoint)
             double dip = s_v[m][1];                       // dipole source of the reaction field
             double rn = dx * s_n[m][0] + dy * s_n[m][1] + dz * s_n[m][2];

@@ -13,6 +13,7 @@
 // on the device.  RHS (charge -> surface), reaction potential (Eq. phi_reac,
 // surface -> charge) and the FP64 energy sum (Eq. energy).
 #include "bem.cuh"
+#include "math64.cuh"
 #include "bem_quad.cuh"
 #include <cub/cub.cuh>
 #include <algorithm>
@@ -223,7 +224,7 @@ __global__ void k_p1(int nt, int nq, const double* __restrict__ x, const T* __re
 
 template <typename T> __device__ __forceinline__ T rsq(T x);
 template <> __device__ __forceinline__ float rsq<float>(float x) { return rsqrtf(x); }
-template <> __device__ __forceinline__ double rsq<double>(double x) { return rsqrt(x); }
+template <> __device__ __forceinline__ double rsq<double>(double x) { return rsqrt64(x); }
 template <typename T> __device__ __forceinline__ T ex(T x);
 template <> __device__ __forceinline__ float ex<float>(float x) { return __expf(x); }
 template <> __device__ __forceinline__ double ex<double>(double x) { return exp(x); }
@@ -309,7 +310,7 @@ __global__ void k_coulomb(long long np, const double* __restrict__ qp, int na, c
         for (int k = 0; k < cnt; ++k) {
             double dx = x - s[k].x, dy = y - s[k].y, dz = z - s[k].z;
             double r2 = dx * dx + dy * dy + dz * dz;
-            if (r2 > 0) acc += s[k].w * rsqrt(r2);
+            if (r2 > 0) acc += s[k].w * rsqrt64(r2);
         }
     }
     if (a < np) f[a] = acc * kInv4PiB * inv_eps;
@@ -372,7 +373,7 @@ __global__ void k_phi_reac(int na, const double4* __restrict__ atoms, long long 
         for (int m = 0; m < cnt; ++m) {
             double dx = px - s_p[m][0], dy = py - s_p[m][1], dz = pz - s_p[m][2];
             double r2 = dx * dx + dy * dy + dz * dz;
-            double rinv = r2 > 0 ? rsqrt(r2) : 0.0;
+            double rinv = r2 > 0 ? rsqrt64(r2) : 0.0;
             acc += rinv * s_p[m][3] + (dx * s_n[m][0] + dy * s_n[m][1] + dz * s_n[m][2]) * rinv * rinv * rinv;
         }
     }

@@ -8,6 +8,7 @@
 // and check potentials box-major [n_box][npad].  Everything here is templated
 // on the arithmetic type: float (mixed path) and double (all-FP64 path).
 #include "fmm.cuh"
+#include "math64.cuh"
 #include <algorithm>
 #include <climits>
 #include <memory>
@@ -32,6 +33,7 @@ void build_xbox_far(fmm_tree* T, int thrX);
 
 constexpr double kInv4PiD = 0.07957747154594767;
 constexpr double kLog2E = 1.4426950408889634;     // log2(e)
+constexpr int kC2EItemBoxes = 512;   // pairs of an item of the M2M / L2L and check -> equivalent lists, at most
 constexpr int kTC = 32;    // boxes per tile of the dense box-vector products (= kM2LTile)
 static_assert(kTC == kM2LTile, "M2L tile width");
 
@@ -48,39 +50,43 @@ template <> __device__ __forceinline__ float rsqrt_t<float>(float x) {
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-template <> __device__ __forceinline__ double rsqrt_t<double>(double x) { return rsqrt(x); }
-// 2^x
-template <typename T> __device__ __forceinline__ T exp2_t(T x);
-template <> __device__ __forceinline__ float exp2_t<float>(float x) {
+template <> __device__ __forceinline__ double rsqrt_t<double>(double x) { return rsqrt64(x); }
+// 2^x, x <= 0; tab: the table of exp2_64 (FP64 only)
+template <typename T> __device__ __forceinline__ T exp2_t(T x, const T* tab = nullptr);
+template <> __device__ __forceinline__ float exp2_t<float>(float x, const float*) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-template <> __device__ __forceinline__ double exp2_t<double>(double x) { return exp2(x); }
-template <typename T> __device__ __forceinline__ T exp_t(T x);
-template <> __device__ __forceinline__ float exp_t<float>(float x) { return exp2_t<float>(x * float(kLog2E)); }
-template <> __device__ __forceinline__ double exp_t<double>(double x) { return exp(x); }
+template <> __device__ __forceinline__ double exp2_t<double>(double x, const double* tab) { return exp2_64(x, tab); }
+// shared table of the FP64 kernels (one entry in FP32: unused)
+template <typename T> constexpr int kTabSize = sizeof(T) == 8 ? kExpTab : 1;
+template <typename T> __device__ __forceinline__ void fill_tab(T* tab) {
+    if constexpr (sizeof(T) == 8) exp2_64_table(tab);
+}
 
 // One source-target interaction, without the 1/(4 pi) factor:
 //   pot += g q + (d.m) f,   dn += -(d.n_t) f q,   d = x_t - y_s,
 //   g = e/r, f = e (1 + kappa r)/r^3, e = exp(-kappa r) (Yukawa) or 1.
 // GUARD: the pair may coincide (r = 0 contributes nothing).  Coincident
 // points share a Morton key, hence a leaf, so only a leaf's own box needs it.
+// Grouped as (e / r) (q + (d.m) c), c = (1 + kappa r) / r^2 = 1 / r^2 + kappa / r;
+// kl2 = -kappa log2(e), so that e = 2^(kl2 r).
 template <typename T, bool YUK, bool DL, bool DN, bool GUARD = true>
-__device__ __forceinline__ void interact(T dx, T dy, T dz, T q, T mx, T my, T mz, T nx, T ny, T nz, T kappa,
-                                         T& pot, T& dn) {
+__device__ __forceinline__ void interact(T dx, T dy, T dz, T q, T mx, T my, T mz, T nx, T ny, T nz, T kappa, T kl2,
+                                         const T* tab, T& pot, T& dn) {
     T r2 = dx * dx + dy * dy + dz * dz;
     T rinv = GUARD ? (r2 > T(0) ? rsqrt_t<T>(r2) : T(0)) : rsqrt_t<T>(r2);
-    T g = rinv, f = rinv * rinv * rinv;
-    if (YUK) {
-        T r = r2 * rinv;
-        T e = exp_t<T>(-kappa * r);
-        g *= e;
-        f *= e * (T(1) + kappa * r);
+    T g = rinv;
+    if (YUK) g *= exp2_t<T>(kl2 * (r2 * rinv), tab);
+    if (DL || DN) {
+        T c = rinv * rinv;
+        if (YUK) c += kappa * rinv;
+        pot += DL ? g * (q + (dx * mx + dy * my + dz * mz) * c) : g * q;
+        if (DN) dn -= (dx * nx + dy * ny + dz * nz) * c * (g * q);
+    } else {
+        pot += g * q;
     }
-    pot += g * q;
-    if (DL) pot += (dx * mx + dy * my + dz * mz) * f;
-    if (DN) dn -= (dx * nx + dy * ny + dz * nz) * f * q;
 }
 
 // The Laplace and the Yukawa interaction of one pair with the geometry
@@ -90,29 +96,28 @@ __device__ __forceinline__ void interact(T dx, T dy, T dz, T q, T mx, T my, T mz
 //   potY += e (g qY + (d.m) f (1 + kr)),  dnY -= e (1 + kr) (d.n) f qY,
 //   g = 1/r, f = 1/r^3, e = exp(-kappa r) (Sec. "Fast multipole method").
 // kl2 = -kappa log2(e), so that e = 2^(kl2 r).  Grouped as
-//   potL += (qL + (d.m) / r^2) / r,   potY += (e / r) (qY + (d.m)(1 + kr) / r^2).
+//   potL += (qL + (d.m) / r^2) / r,   potY += (e / r) (qY + (d.m)(1/r^2 + k/r)).
 template <typename T, bool DL, bool DN, bool GUARD>
 __device__ __forceinline__ void interact_pair(T dx, T dy, T dz, T qL, T qY, T mx, T my, T mz, T nx, T ny, T nz,
-                                              T kappa, T kl2, T& potL, T& potY, T& dnL, T& dnY) {
+                                              T kappa, T kl2, const T* tab, T& potL, T& potY, T& dnL, T& dnY) {
     T r2 = dx * dx + dy * dy + dz * dz;
     T rinv = GUARD ? (r2 > T(0) ? rsqrt_t<T>(r2) : T(0)) : rsqrt_t<T>(r2);
-    T r = r2 * rinv;
-    T er = exp2_t<T>(kl2 * r) * rinv;              // e^{-kr} / r
+    T er = exp2_t<T>(kl2 * (r2 * rinv), tab) * rinv;              // e^{-kr} / r
     if (DL || DN) {
         T rinv2 = rinv * rinv;
-        T u = kappa * r + T(1);
+        T c = kappa * rinv + rinv2;
         if (DL) {
-            T w = (dx * mx + dy * my + dz * mz) * rinv2;
-            potL += rinv * (w + qL);
-            potY += er * (w * u + qY);
+            T dm = dx * mx + dy * my + dz * mz;
+            potL += rinv * (dm * rinv2 + qL);
+            potY += er * (dm * c + qY);
         } else {
             potL += rinv * qL;
             potY += er * qY;
         }
         if (DN) {
-            T dn = (dx * nx + dy * ny + dz * nz) * rinv2;
-            dnL -= rinv * dn * qL;
-            dnY -= er * u * dn * qY;
+            T dn = dx * nx + dy * ny + dz * nz;
+            dnL -= dn * rinv2 * (rinv * qL);
+            dnY -= dn * c * (er * qY);
         }
     } else {
         potL += rinv * qL;
@@ -164,11 +169,15 @@ __global__ void k_gather_tn(long long n, const int* __restrict__ perm, const In*
     tn[k] = {(T)nrm[3 * i], (T)nrm[3 * i + 1], (T)nrm[3 * i + 2], T(0)};
 }
 
+// out[perm[k]] = sum of the nsplit partial results v[s][k], in order
 template <typename T, typename Out>
-__global__ void k_scatter(long long n, const int* __restrict__ perm, const T* __restrict__ v, Out* __restrict__ out) {
+__global__ void k_scatter(long long n, const int* __restrict__ perm, const T* __restrict__ v, Out* __restrict__ out,
+                          int nsplit = 1) {
     long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (k >= n) return;
-    out[perm[k]] = (Out)v[k];
+    T a = v[k];
+    for (int s = 1; s < nsplit; ++s) a += v[s * n + k];
+    out[perm[k]] = (Out)a;
 }
 
 // ---------------------------------------------------------------------------
@@ -192,6 +201,9 @@ __global__ void __launch_bounds__(256) k_p2check(int nbox, const int* __restrict
     using V = typename V4<T>::type;
     __shared__ V s_q[256];
     __shared__ V s_m[DL ? 256 : 1];
+    __shared__ T s_tab[kTabSize<T>];
+    if (YUK) fill_tab(s_tab);                    // (read after the first window's barriers)
+    const T kl2 = -kappa * T(kLog2E);
     const int CH = blockDim.x;
     int bi = blockIdx.x;
     if (bi >= nbox) return;
@@ -233,7 +245,7 @@ __global__ void __launch_bounds__(256) k_p2check(int nbox, const int* __restrict
 #pragma unroll
                 for (int m = 0; m < MAXP; ++m)
                     interact<T, YUK, DL, false>(px[m] - s.x, py[m] - s.y, pz[m] - s.z, s.w, mx, my, mz, 0, 0, 0,
-                                                kappa, acc[m], dummy);
+                                                kappa, kl2, s_tab, acc[m], dummy);
             }
         }
     }
@@ -276,6 +288,8 @@ __global__ void __launch_bounds__(256) k_p2check_pair(int nbox, const int* __res
     using V = typename V4<T>::type;
     __shared__ V s_q[256];
     __shared__ V s_m[256];
+    __shared__ T s_tab[kTabSize<T>];
+    fill_tab(s_tab);                             // (read after the first window's barriers)
     const int CH = blockDim.x;
     int bi = blockIdx.x;
     if (bi >= nbox) return;
@@ -301,15 +315,18 @@ __global__ void __launch_bounds__(256) k_p2check_pair(int nbox, const int* __res
     }
     T d0 = T(0), d1 = T(0);
     const T kl2 = -kappa * T(kLog2E);
-    int ui = 0, off = 0;
+    // grid y: windows taken in turn by gridDim.y CTAs, which add (the caller
+    // zeroes the check potentials)
+    int ui = 0, off = 0, win = 0;
     while (ui < nlist) {
+        const bool mine = win++ % gridDim.y == blockIdx.y;
         __syncthreads();
         int filled = 0;
         while (filled < CH && ui < nlist) {
             const int n = s_xn[ui];
             const int m = min(CH - filled, n - off);
             const int t = threadIdx.x - filled;
-            if (t >= 0 && t < m) {
+            if (mine && t >= 0 && t < m) {
                 const int j = s_xb[ui] + off + t;
                 V v = sq[j];
                 s_q[threadIdx.x] = {(T)((double)v.x - c.x), (T)((double)v.y - c.y), (T)((double)v.z - c.z), v.w};
@@ -320,19 +337,25 @@ __global__ void __launch_bounds__(256) k_p2check_pair(int nbox, const int* __res
             if (off >= n) { ++ui; off = 0; }
         }
         __syncthreads();
+        if (!mine) continue;
 #pragma unroll 4
         for (int t = 0; t < filled; ++t) {
             V s = s_q[t], mm = s_m[t];
 #pragma unroll
             for (int m = 0; m < MAXP; ++m)
                 interact_pair<T, DL, false, false>(px[m] - s.x, py[m] - s.y, pz[m] - s.z, s.w, mm.w, mm.x, mm.y,
-                                                   mm.z, 0, 0, 0, kappa, kl2, aL[m], aY[m], d0, d1);
+                                                   mm.z, 0, 0, 0, kappa, kl2, s_tab, aL[m], aY[m], d0, d1);
         }
     }
 #pragma unroll
     for (int m = 0; m < MAXP; ++m) {
         int i = threadIdx.x + m * CH;
-        if (i < npad) {
+        if (gridDim.y > 1) {
+            if (i < ne) {
+                atomicAdd(chkL + (long long)b * npad + i, aL[m] * T(kInv4PiD));
+                atomicAdd(chkY + (long long)b * npad + i, aY[m] * T(kInv4PiD));
+            }
+        } else if (i < npad) {
             chkL[(long long)b * npad + i] = (i < ne) ? aL[m] * T(kInv4PiD) : T(0);
             chkY[(long long)b * npad + i] = (i < ne) ? aY[m] * T(kInv4PiD) : T(0);
         }
@@ -506,6 +529,67 @@ __device__ __forceinline__ void box_gemm_body(const GemmArgs& a, const TO* __res
     }
 }
 
+// Box-operator products of the all-FP64 path: Y[tgt[p]] += Op(item) X[src[p]]
+// over the pairs of the items (M2L: <= 32 pairs of one (level, offset); M2M /
+// L2L: children of one (level, octant); check -> equivalent solves: boxes of
+// one level).  One CTA per eight pairs of an item: the FP64 pipe does two
+// fused multiply-adds per clock and SM, so a whole n_pad x 32 product keeps an
+// SM busy for 200 us and only an even spread over the SMs counts; operands
+// come from shared memory, which FP64 leaves idle.  Measured at 30,720 points,
+// p = 6: M2M + L2L 14.6 ms as one CTA per 32 parents, octants in turn.
+template <int NPAD>
+__global__ void __launch_bounds__(256) k_box_pairs64(const int4* __restrict__ items, const int* __restrict__ tgt,
+                                                     const int* __restrict__ src, const double* __restrict__ ops,
+                                                     const double* __restrict__ X, double* __restrict__ Y, int ne) {
+    constexpr int COLS = 8, RPT = NPAD / 32, KC = NPAD > 256 ? 8 : 16;
+    __shared__ double s_op[KC][NPAD + 1];
+    __shared__ double s_x[KC][COLS];
+    const int4 it = items[blockIdx.x];
+    const int p0 = blockIdx.y * COLS, cnt = min(COLS, it.y - p0);
+    if (cnt <= 0) return;
+    const int tid = threadIdx.x, c = tid % COLS, ty = tid / COLS;
+    const double* op = ops + (size_t)it.z * NPAD * NPAD;
+    const int pair = it.x + p0 + min(c, cnt - 1);
+    const double* xrow = X + (size_t)src[pair] * NPAD;
+    // rows ty + 32 r; the warp's rows of the last r may all be padding
+    const int nr = (ne - (ty & ~3) + 31) / 32;
+    double acc[RPT];
+#pragma unroll
+    for (int r = 0; r < RPT; ++r) acc[r] = 0.0;
+    for (int k0 = 0; k0 < ne; k0 += KC) {
+        __syncthreads();
+        for (int i = tid; i < NPAD * KC; i += 256) s_op[i % KC][i / KC] = op[(size_t)(i / KC) * NPAD + k0 + i % KC];
+        if (ty < KC) s_x[ty][c] = xrow[k0 + ty];
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < KC; ++k) {
+            const double x = s_x[k][c];
+#pragma unroll
+            for (int r = 0; r < RPT; ++r)
+                if (r < RPT - 1 || r < nr) acc[r] = fma(s_op[k][ty + 32 * r], x, acc[r]);
+        }
+    }
+    if (c >= cnt) return;
+    double* y = Y + (size_t)tgt[pair] * NPAD;
+#pragma unroll
+    for (int r = 0; r < RPT; ++r)
+        if (ty + 32 * r < ne) atomicAdd(y + ty + 32 * r, acc[r]);
+}
+
+static void box_pairs64(int npad, int ne, const int4* items, int nitems, int maxpairs, const int* tgt, const int* src,
+                        const double* ops, const double* X, double* Y, cudaStream_t st) {
+    if (nitems <= 0) return;
+    const dim3 grid(nitems, div_up(maxpairs, 8));
+#define PB_CASE(N) \
+    case N: k_box_pairs64<N><<<grid, 256, 0, st>>>(items, tgt, src, ops, X, Y, ne); break;
+    switch (npad) {
+        PB_CASE(32) PB_CASE(64) PB_CASE(128) PB_CASE(160) PB_CASE(224) PB_CASE(320) PB_CASE(416) PB_CASE(512)
+        default: throw Error(PB_EINVAL, "unsupported expansion order");
+    }
+#undef PB_CASE
+    PB_CHECK_LAUNCH();
+}
+
 // One kernel name per use so launch lists and profiles separate them.
 template <typename T, typename TO, int NPAD>
 __global__ void __launch_bounds__(256) k_m2l_simt(GemmArgs a, const TO* __restrict__ ops, const T* __restrict__ X,
@@ -554,6 +638,9 @@ __global__ void __launch_bounds__(128) k_leaf_eval(const int* __restrict__ leave
     __shared__ V s_q[CH];
     __shared__ V s_m[DL ? CH : 1];
     __shared__ T s_red[DN ? 2 : 1][NT * CH];
+    __shared__ T s_tab[kTabSize<T>];
+    if (YUK) fill_tab(s_tab);                    // (read after the first window's barriers)
+    const T kl2 = -kappa * T(kLog2E);
     int li = blockIdx.x;
     if (li >= nleaf) return;
     const int b = leaves[li];
@@ -598,7 +685,7 @@ __global__ void __launch_bounds__(128) k_leaf_eval(const int* __restrict__ leave
 #pragma unroll
                         for (int u = 0; u < NT; ++u)
                             interact<T, YUK, DL, DN, true>((T)xt[u].x - s.x, (T)xt[u].y - s.y, (T)xt[u].z - s.z, s.w,
-                                                           mx, my, mz, nx[u], ny[u], nz[u], kappa, pot[u], dn[u]);
+                                                           mx, my, mz, nx[u], ny[u], nz[u], kappa, kl2, s_tab, pot[u], dn[u]);
                     }
                 } else {
                     for (int k = g; g < G && k < cnt; k += G) {
@@ -608,7 +695,7 @@ __global__ void __launch_bounds__(128) k_leaf_eval(const int* __restrict__ leave
 #pragma unroll
                         for (int u = 0; u < NT; ++u)
                             interact<T, YUK, DL, DN, false>((T)xt[u].x - s.x, (T)xt[u].y - s.y, (T)xt[u].z - s.z,
-                                                            s.w, mx, my, mz, nx[u], ny[u], nz[u], kappa, pot[u], dn[u]);
+                                                            s.w, mx, my, mz, nx[u], ny[u], nz[u], kappa, kl2, s_tab, pot[u], dn[u]);
                     }
                 }
             }
@@ -640,7 +727,7 @@ __global__ void __launch_bounds__(128) k_leaf_eval(const int* __restrict__ leave
 #pragma unroll
                     for (int u = 0; u < NT; ++u)
                         interact<T, YUK, false, DN, false>(rx[u] - s.x, ry[u] - s.y, rz[u] - s.z, s.w, 0, 0, 0,
-                                                           nx[u], ny[u], nz[u], kappa, pot[u], dn[u]);
+                                                           nx[u], ny[u], nz[u], kappa, kl2, s_tab, pot[u], dn[u]);
                 }
             }
         }
@@ -730,7 +817,8 @@ __global__ void __launch_bounds__(128) k_leaf_pair(const int* __restrict__ leave
                                                    const T* __restrict__ QuY, const T* __restrict__ QdY,
                                                    const float4* __restrict__ surf, int ne, int npad, T kappa,
                                                    T* __restrict__ potL_out, T* __restrict__ potY_out,
-                                                   T* __restrict__ dnL_out, T* __restrict__ dnY_out) {
+                                                   T* __restrict__ dnL_out, T* __restrict__ dnY_out,
+                                                   long long part_stride) {
     using V = typename V4<T>::type;
     constexpr int CH = 128;
     constexpr int CAP = 16384 / (int)sizeof(V);     // points per window: 16 KB per array
@@ -738,11 +826,19 @@ __global__ void __launch_bounds__(128) k_leaf_pair(const int* __restrict__ leave
     static_assert(NR * NT * CH * (int)sizeof(T) <= CAP * (int)sizeof(V), "reduction fits the staging buffer");
     __shared__ __align__(16) V s_q[CAP];
     __shared__ __align__(16) V s_m[CAP];
+    __shared__ T s_tab[kTabSize<T>];
+    fill_tab(s_tab);                             // (read after the barriers below)
     __shared__ int s_self;
     T* s_red = reinterpret_cast<T*>(s_q);            // [NR][NT * CH], after the last window
     T* s_qy = reinterpret_cast<T*>(s_m);             // far windows: the Yukawa densities
     const int li = blockIdx.x;
     if (li >= nleaf) return;
+    // grid y: every window's points are split over gridDim.y CTAs, each with
+    // its own partial outputs (added in order by the scatter)
+    const int sp = blockIdx.y, S = gridDim.y;
+    potL_out += sp * part_stride;
+    potY_out += sp * part_stride;
+    if (DN) { dnL_out += sp * part_stride; dnY_out += sp * part_stride; }
     const int b = leaves[li];
     const int t0 = tb[b], t1 = te[b];
     const int slots = min(CH, max(4, (t1 - t0 + NT - 1) / NT));
@@ -786,22 +882,22 @@ __global__ void __launch_bounds__(128) k_leaf_pair(const int* __restrict__ leave
                 const int n = stage_near<V, true, CAP>(s_q, s_m, sq, sm, ul, nu, selfpos, sb, se, vi, off);   // sm.w: Yukawa monopole
                 __syncthreads();
                 const int selfhi = min(self_left, n);
-                int k = g;
-                for (; active && k < selfhi; k += G) {
+                int k = g + G * sp;
+                for (; active && k < selfhi; k += G * S) {
                     const V s = s_q[k], mm = s_m[k];
 #pragma unroll
                     for (int u = 0; u < NT; ++u)
                         interact_pair<T, DL, DN, true>(xt[u] - s.x, yt[u] - s.y, zt[u] - s.z, s.w, mm.w, mm.x, mm.y,
-                                                       mm.z, nx[u], ny[u], nz[u], kappa, kl2, pL[u], pY[u], dL[u],
+                                                       mm.z, nx[u], ny[u], nz[u], kappa, kl2, s_tab, pL[u], pY[u], dL[u],
                                                        dY[u]);
                 }
 #pragma unroll 4
-                for (; active && k < n; k += G) {
+                for (; active && k < n; k += G * S) {
                     const V s = s_q[k], mm = s_m[k];
 #pragma unroll
                     for (int u = 0; u < NT; ++u)
                         interact_pair<T, DL, DN, false>(xt[u] - s.x, yt[u] - s.y, zt[u] - s.z, s.w, mm.w, mm.x,
-                                                        mm.y, mm.z, nx[u], ny[u], nz[u], kappa, kl2, pL[u], pY[u],
+                                                        mm.y, mm.z, nx[u], ny[u], nz[u], kappa, kl2, s_tab, pL[u], pY[u],
                                                         dL[u], dY[u]);
                 }
                 __syncthreads();
@@ -837,13 +933,13 @@ __global__ void __launch_bounds__(128) k_leaf_pair(const int* __restrict__ leave
                 }
                 __syncthreads();
 #pragma unroll 4
-                for (int k = g; active && k < n; k += G) {
+                for (int k = g + G * sp; active && k < n; k += G * S) {
                     const V s = s_q[k];
                     const T qy = s_qy[k];
 #pragma unroll
                     for (int u = 0; u < NT; ++u)
                         interact_pair<T, false, DN, false>(rx[u] - s.x, ry[u] - s.y, rz[u] - s.z, s.w, qy, 0, 0, 0,
-                                                           nx[u], ny[u], nz[u], kappa, kl2, pL[u], pY[u], dL[u],
+                                                           nx[u], ny[u], nz[u], kappa, kl2, s_tab, pL[u], pY[u], dL[u],
                                                            dY[u]);
                 }
                 __syncthreads();
@@ -1462,24 +1558,23 @@ static void launch_p2check(cudaStream_t st, int nbox, const int* boxes, int mode
     PB_CHECK_LAUNCH();
 }
 
-// the two check -> equivalent conversions: the FP64 solve for the FP64
-// path; for the FP32 path the factored solve Y = W2 (W1 X), two FP32
-// passes through `tmp` (box-major like X and Y)
-template <typename T>
+// check -> equivalent conversion of the FP32 path on the CUDA cores: the
+// factored solve Y = W2 (W1 X), two passes through `tmp` (box-major like X
+// and Y)
 static void check2equiv(const Operators& O, int level, bool up, cudaStream_t st, GemmArgs ga, int ncols,
-                        const int* cols, const T* X, T* Y, T* tmp);
-template <>
-void check2equiv<float>(const Operators& O, int level, bool up, cudaStream_t st, GemmArgs ga, int ncols,
                         const int* cols, const float* X, float* Y, float* tmp) {
     ga.mode = G_DENSE; ga.ncols = ncols; ga.cols = cols; ga.col_base = 0; ga.level = level; ga.accumulate = 0;
     gemm_dispatch<float, float>(O.npad, st, div_up(ncols, kTC), ga, up ? O.uc2ue_w1.p : O.dc2de_w1.p, X, tmp);
     gemm_dispatch<float, float>(O.npad, st, div_up(ncols, kTC), ga, up ? O.uc2ue_w2.p : O.dc2de_w2.p, tmp, Y);
 }
-template <>
-void check2equiv<double>(const Operators& O, int level, bool up, cudaStream_t st, GemmArgs ga, int ncols,
-                         const int* cols, const double* X, double* Y, double*) {
-    ga.mode = G_DENSE; ga.ncols = ncols; ga.cols = cols; ga.col_base = 0; ga.level = level; ga.accumulate = 0;
-    gemm_dispatch<double, double>(O.npad, st, div_up(ncols, kTC), ga, up ? O.uc2ue_d.p : O.dc2de_d.p, X, Y);
+
+// CTAs that share a leaf's sources.  FP64: a leaf keeps an SM busy for half a
+// millisecond, and a few hundred of them leave the slowest SM with several
+// times the average, so about 24 CTAs per SM (30,720 points, p = 6: leaf
+// 10.1 -> 4.0 ms).
+static int leaf_split(const fmm_tree* Tr, bool fp64) {
+    if (!fp64 || Tr->n_tleaf <= 0) return 1;
+    return std::max(1, std::min(8, div_up(24LL * Tr->ctx->sm_count, Tr->n_tleaf)));
 }
 
 template <typename T, bool YUK, bool DL, bool DN>
@@ -1533,17 +1628,20 @@ static GemmArgs tree_gemm_args(const fmm_tree* Tr) {
     return ga;
 }
 
-// UC2UE at every leaf with sources (upward check potentials in W.chk)
+// UC2UE at every leaf with sources (upward check potentials in W.chk; Qu zero)
 template <typename T>
 static void far_uc2ue(fmm_tree* Tr, const Operators& O, Work<T>& W) {
-    if constexpr (std::is_same<T, float>::value) {
+    if constexpr (std::is_same<T, double>::value) {
+        box_pairs64(O.npad, O.ne, Tr->c2e_items_up.p, Tr->n_c2e_up, kC2EItemBoxes, Tr->sleaf_ids.p, Tr->sleaf_ids.p,
+                    O.uc2ue_d.p, W.chk.p, W.Qu.p, Tr->ctx->stream);
+    } else {
         if (c2e_tc_launch(Tr, O, true, W.chk.p, W.Qu.p, W.tmp.p, Tr->ctx->dev_err, Tr->ctx->stream)) return;
-    }
-    GemmArgs ga = tree_gemm_args<T>(Tr);
-    for (int l = 0; l < Tr->nlev; ++l) {
-        int a0 = Tr->sleaf_lvl_off[l], a1 = Tr->sleaf_lvl_off[l + 1];
-        if (a1 <= a0) continue;
-        check2equiv<T>(O, l, true, Tr->ctx->stream, ga, a1 - a0, Tr->sleaf_ids.p + a0, W.chk.p, W.Qu.p, W.tmp.p);
+        GemmArgs ga = tree_gemm_args<T>(Tr);
+        for (int l = 0; l < Tr->nlev; ++l) {
+            int a0 = Tr->sleaf_lvl_off[l], a1 = Tr->sleaf_lvl_off[l + 1];
+            if (a1 <= a0) continue;
+            check2equiv(O, l, true, Tr->ctx->stream, ga, a1 - a0, Tr->sleaf_ids.p + a0, W.chk.p, W.Qu.p, W.tmp.p);
+        }
     }
 }
 
@@ -1555,6 +1653,12 @@ static void m2m_level(fmm_tree* Tr, const Operators& O, Work<T>& W, int l) {
     cudaStream_t st = ctx->stream;
     if constexpr (std::is_same<T, float>::value) {
         if (!ctx->deterministic && pc_tc_launch(Tr, O, l + 1, true, W.Qu.p, ctx->dev_err, st)) return;
+    } else if (!ctx->deterministic) {
+        const auto& P = Tr->pc_pairs;
+        const int i0 = P.level_item_off[l + 1], i1 = P.level_item_off[l + 2];
+        box_pairs64(O.npad, O.ne, P.items.p + i0, i1 - i0, kC2EItemBoxes, P.parent.p, P.child.p, O.m2m_d.p, W.Qu.p, W.Qu.p,
+                    st);
+        return;
     }
     GemmArgs ga = tree_gemm_args<T>(Tr);
     int a0 = Tr->lvl_off[l], a1 = Tr->lvl_off[l + 1];
@@ -1568,18 +1672,21 @@ static void far_m2m(fmm_tree* Tr, const Operators& O, Work<T>& W) {
 }
 
 // DC2DE at every X-list box (downward check potentials of P2L in W.chk);
-// writes Qd of those boxes before the M2L accumulates
+// writes Qd (zero on entry) of those boxes before the M2L accumulates
 template <typename T>
 static void far_dc2de_x(fmm_tree* Tr, const Operators& O, Work<T>& W, bool xfar = false) {
-    if constexpr (std::is_same<T, float>::value) {
+    if constexpr (std::is_same<T, double>::value) {
+        box_pairs64(O.npad, O.ne, Tr->c2e_items_dn.p, Tr->n_c2e_dn, kC2EItemBoxes, Tr->xbox_ids.p, Tr->xbox_ids.p,
+                    O.dc2de_d.p, W.chk.p, W.Qd.p, Tr->ctx->stream);
+    } else {
         if (c2e_tc_launch(Tr, O, false, W.chk.p, W.Qd.p, W.tmp.p, Tr->ctx->dev_err, Tr->ctx->stream, xfar)) return;
-    }
-    PB_REQUIRE(!xfar, PB_EINVAL, "reduced X-box list without the tensor-core solve");
-    GemmArgs ga = tree_gemm_args<T>(Tr);
-    for (int l = 0; l < Tr->nlev; ++l) {
-        int a0 = Tr->xbox_lvl_off[l], a1 = Tr->xbox_lvl_off[l + 1];
-        if (a1 <= a0) continue;
-        check2equiv<T>(O, l, false, Tr->ctx->stream, ga, a1 - a0, Tr->xbox_ids.p + a0, W.chk.p, W.Qd.p, W.tmp.p);
+        PB_REQUIRE(!xfar, PB_EINVAL, "reduced X-box list without the tensor-core solve");
+        GemmArgs ga = tree_gemm_args<T>(Tr);
+        for (int l = 0; l < Tr->nlev; ++l) {
+            int a0 = Tr->xbox_lvl_off[l], a1 = Tr->xbox_lvl_off[l + 1];
+            if (a1 <= a0) continue;
+            check2equiv(O, l, false, Tr->ctx->stream, ga, a1 - a0, Tr->xbox_ids.p + a0, W.chk.p, W.Qd.p, W.tmp.p);
+        }
     }
 }
 
@@ -1592,6 +1699,14 @@ static void far_m2l(fmm_tree* Tr, const Operators& O, Work<T>& W) {
         if (!ctx->deterministic)
             tc_done = m2l_h_launch(Tr, O, nullptr, W.Qu.p, W.Qd.p, W.tmp.p, nullptr, nullptr, nullptr, ctx->dev_err,
                                    ctx->stream);
+    }
+    if constexpr (std::is_same<T, double>::value) {
+        if (!ctx->deterministic) {
+            const auto& P = Tr->m2l_pairs;
+            box_pairs64(O.npad, O.ne, P.items32.p, P.nitems32, 32, P.tgt.p, P.src.p, O.m2l_d.p, W.Qu.p, W.Qd.p,
+                        ctx->stream);
+            return;
+        }
     }
     if (!tc_done && !ctx->deterministic && Tr->m2l_pairs.nitems32 > 0) {
         // one CTA per at most 32 V-list pairs of one (level, offset) group:
@@ -1624,6 +1739,12 @@ static void l2l_level(fmm_tree* Tr, const Operators& O, Work<T>& W, int l) {
     cudaStream_t st = ctx->stream;
     if constexpr (std::is_same<T, float>::value) {
         if (!ctx->deterministic && pc_tc_launch(Tr, O, l, false, W.Qd.p, ctx->dev_err, st)) return;
+    } else if (!ctx->deterministic) {
+        const auto& P = Tr->pc_pairs;
+        const int i0 = P.level_item_off[l], i1 = P.level_item_off[l + 1];
+        box_pairs64(O.npad, O.ne, P.items.p + i0, i1 - i0, kC2EItemBoxes, P.child.p, P.parent.p, O.l2l_d.p, W.Qd.p, W.Qd.p,
+                    st);
+        return;
     }
     GemmArgs ga = tree_gemm_args<T>(Tr);
     int p0 = Tr->lvl_off[l - 1], p1 = Tr->lvl_off[l];
@@ -1806,8 +1927,15 @@ static void launch_p2check_pair(cudaStream_t st, int nbox, const int* boxes, int
         }
     }
     PB_REQUIRE(thrX < 0, PB_EINVAL, "direct X-list evaluation needs the packed check-potential kernel");
+    // FP64 P2L: X lists of up to 26 leaves, split like the leaves of
+    // apply_pair_t (1.84 -> 1.46 ms)
+    int split = 1;
+    if (std::is_same<T, double>::value && mode == 1 && !Tr->ctx->deterministic) {
+        split = std::max(1, std::min(8, div_up(24LL * Tr->ctx->sm_count, nbox)));
+        if (split > 1) { WL.chk.zero(st); WY.chk.zero(st); }
+    }
     if (O.npad <= 256)
-        k_p2check_pair<T, DL, 1><<<nbox, O.npad, 0, st>>>(nbox, boxes, mode, Tr->center.p, Tr->sb.p, Tr->se.p,
+        k_p2check_pair<T, DL, 1><<<dim3(nbox, split), O.npad, 0, st>>>(nbox, boxes, mode, Tr->center.p, Tr->sb.p, Tr->se.p,
                                                           Tr->X.p, Tr->X_n.p, WL.sq.p, WL.sm.p,
                                                           (const float4*)O.surf_f.p, O.ne, O.npad, kappa, WL.chk.p,
                                                           WY.chk.p);
@@ -1815,7 +1943,7 @@ static void launch_p2check_pair(cudaStream_t st, int nbox, const int* boxes, int
         // two check points per thread, the threads rounded up from n_pad / 2
         // (p = 8: 160 threads for 296 points; a fixed 256 left 42% of the
         // slots idle: P2M 2.12 -> 1.63 ms at 4M)
-        k_p2check_pair<T, DL, 2><<<nbox, std::min(256, (O.npad / 2 + 31) / 32 * 32), 0, st>>>(
+        k_p2check_pair<T, DL, 2><<<dim3(nbox, split), std::min(256, (O.npad / 2 + 31) / 32 * 32), 0, st>>>(
                                                        nbox, boxes, mode, Tr->center.p, Tr->sb.p, Tr->se.p,
                                                        Tr->X.p, Tr->X_n.p, WL.sq.p, WL.sm.p,
                                                        (const float4*)O.surf_f.p, O.ne, O.npad, kappa, WL.chk.p,
@@ -1825,7 +1953,7 @@ static void launch_p2check_pair(cudaStream_t st, int nbox, const int* boxes, int
 
 template <typename T, bool DL, bool DN, int PART>
 static void launch_leaf_pair(cudaStream_t st, fmm_tree* Tr, Work<T>& WL, Work<T>& WY, const Operators& O, T kappa,
-                             int thrW = -1, int thrX = -1) {
+                             int thrW = -1, int thrX = -1, int split = 1) {
     if (Tr->n_tleaf <= 0) return;
     const float4* tpos = Tr->same ? Tr->pos_s.p : Tr->pos_t.p;
     const int* tb = Tr->same ? Tr->sb.p : Tr->tb.p;
@@ -1847,10 +1975,11 @@ static void launch_leaf_pair(cudaStream_t st, fmm_tree* Tr, Work<T>& WL, Work<T>
     PB_REQUIRE(thrW < 0 && thrX < 0, PB_EINVAL, "direct W/X-list evaluation needs the packed leaf kernel");
     const int NT = nt_opt ? nt_opt : (sizeof(T) == 4 ? 4 : 2);
     auto k = NT == 4 ? k_leaf_pair<T, DL, DN, 4, PART> : k_leaf_pair<T, DL, DN, 2, PART>;
-    k<<<Tr->n_tleaf, 128, 0, st>>>(
+    k<<<dim3(Tr->n_tleaf, split), 128, 0, st>>>(
         Tr->leaf_ids.p, Tr->n_tleaf, tb, te, Tr->sb.p, Tr->se.p, Tr->U_off.p, Tr->U_ids.p, Tr->W_off.p, Tr->W_ids.p,
         Tr->level.p, Tr->center.p, tpos, WL.tn.p, WL.sq.p, WL.sm.p, WL.Qu.p, WL.Qd.p, WY.Qu.p, WY.Qd.p,
-        (const float4*)O.surf_f.p, O.ne, O.npad, kappa, WL.pot.p, WY.pot.p, WL.dn.p, WY.dn.p);
+        (const float4*)O.surf_f.p, O.ne, O.npad, kappa, WL.pot.p, WY.pot.p, WL.dn.p, WY.dn.p,
+        Tr->same ? Tr->ns : Tr->nt);
     PB_CHECK_LAUNCH();
 }
 
@@ -1883,9 +2012,10 @@ static void apply_pair_t(fmm_tree* Tr, const Operators& OL, const Operators& OY,
     WL.sm.alloc(ns, st);
     alloc_far(WL, Tr->nbox, OL.npad, st);
     alloc_far(WY, Tr->nbox, OY.npad, st);
-    WL.pot.alloc(nt, st);
-    WY.pot.alloc(nt, st);
-    if (DN) { WL.dn.alloc(nt, st); WY.dn.alloc(nt, st); WL.tn.alloc(nt, st); }
+    const int split = leaf_split(Tr, std::is_same<T, double>::value);
+    WL.pot.alloc(nt * split, st);
+    WY.pot.alloc(nt * split, st);
+    if (DN) { WL.dn.alloc(nt * split, st); WY.dn.alloc(nt * split, st); WL.tn.alloc(nt, st); }
     pb_ctx* ctx = Tr->ctx;
     auto ph = std::make_unique<PhaseTimer>(ctx, PB_PH_GATHER);
     k_gather_pair<T, In><<<div_up(ns, 256), 256, 0, st>>>(ns, Tr->perm_s.p, Tr->pos_s.p, qL, qY, dip, src_n, WL.sq.p,
@@ -1904,9 +2034,9 @@ static void apply_pair_t(fmm_tree* Tr, const Operators& OL, const Operators& OY,
         PB_CUDA(cudaStreamWaitEvent(ctx->aux, ctx->ev_fork, 0));
         {
             PhaseTimer phn(ctx, PB_PH_LEAF, ctx->aux);
-            if (DL) launch_leaf_pair<T, true, false, 1>(ctx->aux, Tr, WL, WY, OL, kappa, thrW, thrX);
-            else if (DN) launch_leaf_pair<T, false, true, 1>(ctx->aux, Tr, WL, WY, OL, kappa, thrW, thrX);
-            else launch_leaf_pair<T, false, false, 1>(ctx->aux, Tr, WL, WY, OL, kappa, thrW, thrX);
+            if (DL) launch_leaf_pair<T, true, false, 1>(ctx->aux, Tr, WL, WY, OL, kappa, thrW, thrX, split);
+            else if (DN) launch_leaf_pair<T, false, true, 1>(ctx->aux, Tr, WL, WY, OL, kappa, thrW, thrX, split);
+            else launch_leaf_pair<T, false, false, 1>(ctx->aux, Tr, WL, WY, OL, kappa, thrW, thrX, split);
         }
         PB_CUDA(cudaEventRecord(ctx->ev_join, ctx->aux));
     }
@@ -1937,24 +2067,24 @@ static void apply_pair_t(fmm_tree* Tr, const Operators& OL, const Operators& OY,
     if (fork) PB_CUDA(cudaStreamWaitEvent(st, ctx->ev_join, 0));
     ph.reset(); ph = std::make_unique<PhaseTimer>(ctx, PB_PH_LEAF);
     if (fork) {
-        if (DL) launch_leaf_pair<T, true, false, 2>(st, Tr, WL, WY, OL, kappa, thrW, thrX);
-        else if (DN) launch_leaf_pair<T, false, true, 2>(st, Tr, WL, WY, OL, kappa, thrW, thrX);
-        else launch_leaf_pair<T, false, false, 2>(st, Tr, WL, WY, OL, kappa, thrW, thrX);
+        if (DL) launch_leaf_pair<T, true, false, 2>(st, Tr, WL, WY, OL, kappa, thrW, thrX, split);
+        else if (DN) launch_leaf_pair<T, false, true, 2>(st, Tr, WL, WY, OL, kappa, thrW, thrX, split);
+        else launch_leaf_pair<T, false, false, 2>(st, Tr, WL, WY, OL, kappa, thrW, thrX, split);
     } else {
-        if (DL) launch_leaf_pair<T, true, false, 0>(st, Tr, WL, WY, OL, kappa, thrW, thrX);
-        else if (DN) launch_leaf_pair<T, false, true, 0>(st, Tr, WL, WY, OL, kappa, thrW, thrX);
-        else launch_leaf_pair<T, false, false, 0>(st, Tr, WL, WY, OL, kappa, thrW, thrX);
+        if (DL) launch_leaf_pair<T, true, false, 0>(st, Tr, WL, WY, OL, kappa, thrW, thrX, split);
+        else if (DN) launch_leaf_pair<T, false, true, 0>(st, Tr, WL, WY, OL, kappa, thrW, thrX, split);
+        else launch_leaf_pair<T, false, false, 0>(st, Tr, WL, WY, OL, kappa, thrW, thrX, split);
     }
     ph.reset(); ph = std::make_unique<PhaseTimer>(ctx, PB_PH_SCATTER);
     const int* pt = Tr->same ? Tr->perm_s.p : Tr->perm_t.p;
-    k_scatter<T, In><<<div_up(nt, 256), 256, 0, st>>>(nt, pt, WL.pot.p, outL);
+    k_scatter<T, In><<<div_up(nt, 256), 256, 0, st>>>(nt, pt, WL.pot.p, outL, split);
     PB_CHECK_LAUNCH();
-    k_scatter<T, In><<<div_up(nt, 256), 256, 0, st>>>(nt, pt, WY.pot.p, outY);
+    k_scatter<T, In><<<div_up(nt, 256), 256, 0, st>>>(nt, pt, WY.pot.p, outY, split);
     PB_CHECK_LAUNCH();
     if (DN) {
-        k_scatter<T, In><<<div_up(nt, 256), 256, 0, st>>>(nt, pt, WL.dn.p, dnL);
+        k_scatter<T, In><<<div_up(nt, 256), 256, 0, st>>>(nt, pt, WL.dn.p, dnL, split);
         PB_CHECK_LAUNCH();
-        k_scatter<T, In><<<div_up(nt, 256), 256, 0, st>>>(nt, pt, WY.dn.p, dnY);
+        k_scatter<T, In><<<div_up(nt, 256), 256, 0, st>>>(nt, pt, WY.dn.p, dnY, split);
         PB_CHECK_LAUNCH();
     }
     ph.reset();

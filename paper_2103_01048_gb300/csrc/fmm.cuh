@@ -22,7 +22,7 @@ struct Operators {
     int p = 0, ne = 0, npad = 0, nlev = 0;
     DBuf<double> surf;            // [ne][3] unit surface points
     DBuf<float> surf_f;           // [ne][4] float copy (x, y, z, 0)
-    // FP32 copies
+    // FP32 operators (the sets of the FP32 path hold only these)
     // factored solves of the FP32 path: pinv = W2 W1 (W1 = D V^T K^T, W2 = V)
     DBuf<float> uc2ue_w1, uc2ue_w2, dc2de_w1, dc2de_w2;   // [nlev][npad^2]
     DBuf<float> m2m, l2l;         // [nlev][8][npad^2]  (child level index)
@@ -40,9 +40,8 @@ struct Operators {
     DBuf<float> m2m_tc, l2l_tc;
     DBuf<float> uc2ue_w1_tc, uc2ue_w2_tc, dc2de_w1_tc, dc2de_w2_tc;   // same packing, [level]
     bool have_tc = false;
-    // FP64 copies (all-FP64 path)
+    // FP64 operators (the sets of the all-FP64 path hold only these)
     DBuf<double> uc2ue_d, dc2de_d, m2m_d, l2l_d, m2l_d;
-    bool have_d = false;
 };
 
 std::shared_ptr<Operators> get_operators(fmm_tree* T, int kernel, double kappa, int p, bool need_fp64);

@@ -37,7 +37,7 @@ void radix_sort_pairs(const unsigned* keys_in, const int* vals_in, unsigned* key
 constexpr int kTcRows = 128;           // pairs per row tile (MMA M)
 constexpr int kM2LSegBoxes = 8192;     // target boxes of one segment of the M2L pair list
 constexpr int kTcItemPairs = 2048;     // pairs per self-test item
-constexpr int kTcSmallItemPairs = 512; // M2M / L2L / check->equivalent items: fewer pairs per operator, more CTAs
+constexpr int kTcSmallItemPairs = 512; // M2M / L2L / check->equivalent items: few pairs per operator, many CTAs
 
 // Operator split per padded size: NS parts of the output rows (MMA N =
 // npad / NS) times KS parts of the inner dimension (npad / KS columns,

@@ -12,6 +12,7 @@
 // one fixed scratch array that lives in this file for the life of the
 // process.  It has no counterpart in the paper.
 #include "bem.cuh"
+#include "math64.cuh"
 
 namespace pbfmm {
 
@@ -63,7 +64,7 @@ __global__ void k_phi_reac_scratch(int na, const double4* __restrict__ atoms, lo
         for (int m = 0; m < cnt; ++m) {
             double dx = px - s_p[m][0], dy = py - s_p[m][1], dz = pz - s_p[m][2];
             double r2 = dx * dx + dy * dy + dz * dz;
-            double rinv = r2 > 0 ? rsqrt(r2) : 0.0;
+            double rinv = r2 > 0 ? rsqrt64(r2) : 0.0;
             acc += rinv * s_p[m][3] + (dx * s_n[m][0] + dy * s_n[m][1] + dz * s_n[m][2]) * rinv * rinv * rinv;
         }
     }

@@ -283,8 +283,8 @@ __global__ void k_store_padded(int n, int npad, const double* __restrict__ src, 
 // octants) C_z = P K_z with P the level's pseudo-inverse (n x n, FP64) and
 // K_z[k][j] = g(t_z + ts u_k, s_z + ss u_j) generated on the fly from the
 // unit surface u.  Tiled FP64 GEMM: 64 x 64 outputs per CTA, 4 x 4 per thread,
-// 16-wide K steps through shared memory; written padded to npad x npad (FP32
-// and, if dst_d, FP64) at dst + z * npad^2.
+// 16-wide K steps through shared memory; written padded to npad x npad to
+// dst_f (FP32) or dst_d (FP64) at z * npad^2.
 enum { OPB_M2L = 0, OPB_M2M = 1, OPB_L2L = 2 };
 constexpr int kOpTile = 64, kOpK = 16;
 
@@ -350,7 +350,7 @@ __global__ void __launch_bounds__(256) k_build_ops(int n, int npad, int mode, in
         for (int v = 0; v < 4; ++v) {
             const int i = i0 + ty + 16 * u, j = j0 + tx + 16 * v;
             if (i < n && j < n) {
-                dst_f[(size_t)z * m2 + (size_t)i * npad + j] = (float)acc[u][v];
+                if (dst_f) dst_f[(size_t)z * m2 + (size_t)i * npad + j] = (float)acc[u][v];
                 if (dst_d) dst_d[(size_t)z * m2 + (size_t)i * npad + j] = acc[u][v];
             }
         }
@@ -401,16 +401,19 @@ void pack_box_ops_tc(Operators& O, cudaStream_t st);
 void pack_m2l_h(Operators& O, cudaStream_t st);
 
 std::shared_ptr<Operators> get_operators(fmm_tree* T, int kernel, double kappa, int p, bool need_fp64) {
-    auto key = std::make_tuple(kernel, kernel == FMM_YUKAWA ? kappa : 0.0, p, T->nlev);
+    // one set per precision: the FP64 set keeps the grid order of the surface
+    // points (its regularised solves amplify the rounding of another order to
+    // 1e-9 of the weakest fields), the FP32 set numbers them by reflections
+    auto key = std::make_tuple(kernel, kernel == FMM_YUKAWA ? kappa : 0.0, need_fp64 ? -p : p, T->nlev);
     auto it = T->ops.find(key);
-    if (it != T->ops.end() && (!need_fp64 || it->second->have_d)) return it->second;
+    if (it != T->ops.end()) return it->second;
     // another tree of the context with the same box sizes may hold the set
-    const auto gkey = std::make_tuple(kernel, kernel == FMM_YUKAWA ? kappa : 0.0, p, T->R, T->nlev);
+    const auto gkey = std::make_tuple(kernel, kernel == FMM_YUKAWA ? kappa : 0.0, need_fp64 ? -p : p, T->R, T->nlev);
     {
         auto g = T->ctx->op_cache.find(gkey);
         if (g != T->ctx->op_cache.end()) {
             auto sp = std::static_pointer_cast<Operators>(g->second.lock());
-            if (sp && (!need_fp64 || sp->have_d)) {
+            if (sp) {
                 T->ops[key] = sp;
                 return sp;
             }
@@ -425,8 +428,8 @@ std::shared_ptr<Operators> get_operators(fmm_tree* T, int kernel, double kappa, 
     O->npad = pad32(O->ne);
     O->nlev = T->nlev;
     const int n = O->ne, np = O->npad, L = T->nlev;
-    // unit surface: boundary points of the p x p x p grid on [-1, 1]^3.  Even
-    // p: orbits of the eight sign changes together, point 8 * orbit + sign
+    // unit surface: boundary points of the p x p x p grid on [-1, 1]^3.  FP32
+    // and even p: orbits of the eight sign changes together, point 8 * orbit + sign
     // bits (x: 4, y: 2, z: 1; 1 = negative), so that a reflection of the
     // coordinates is an exclusive or of the point's number (m2l_f16.cu).
     std::vector<double> s;
@@ -435,7 +438,7 @@ std::shared_ptr<Operators> get_operators(fmm_tree* T, int kernel, double kappa, 
         s.push_back(x); s.push_back(y); s.push_back(z);
         sf.push_back((float)x); sf.push_back((float)y); sf.push_back((float)z); sf.push_back(0.f);
     };
-    const int i0 = p % 2 == 0 ? p / 2 : 0;
+    const int i0 = !need_fp64 && p % 2 == 0 ? p / 2 : 0;
     for (int i = i0; i < p; ++i)
         for (int j = i0; j < p; ++j)
             for (int k = i0; k < p; ++k) {
@@ -450,15 +453,15 @@ std::shared_ptr<Operators> get_operators(fmm_tree* T, int kernel, double kappa, 
     PB_CUDA(cudaMemcpyAsync(O->surf.p, s.data(), s.size() * sizeof(double), cudaMemcpyHostToDevice, st));
     PB_CUDA(cudaMemcpyAsync(O->surf_f.p, sf.data(), sf.size() * sizeof(float), cudaMemcpyHostToDevice, st));
     const size_t m2 = (size_t)np * np;
-    O->uc2ue_d.alloc(L * m2, st); O->dc2de_d.alloc(L * m2, st);
-    O->m2m.alloc(L * 8 * m2, st); O->l2l.alloc(L * 8 * m2, st);
-    O->m2l.alloc(L * (size_t)kNumOffsets * m2, st);
-    O->m2m.zero(st); O->l2l.zero(st); O->m2l.zero(st);
-    if (need_fp64) {
+    if (!need_fp64) {
+        O->m2m.alloc(L * 8 * m2, st); O->l2l.alloc(L * 8 * m2, st);
+        O->m2l.alloc(L * (size_t)kNumOffsets * m2, st);
+        O->m2m.zero(st); O->l2l.zero(st); O->m2l.zero(st);
+    } else {
+        O->uc2ue_d.alloc(L * m2, st); O->dc2de_d.alloc(L * m2, st);
         O->m2m_d.alloc(L * 8 * m2, st); O->l2l_d.alloc(L * 8 * m2, st);
         O->m2l_d.alloc(L * (size_t)kNumOffsets * m2, st);
         O->m2m_d.zero(st); O->l2l_d.zero(st); O->m2l_d.zero(st);
-        O->have_d = true;
     }
     Builder Bd(st, n, kernel, kappa, O->surf.p);
     DBuf<double> uc2ue_prev, dc;
@@ -470,40 +473,41 @@ std::shared_ptr<Operators> get_operators(fmm_tree* T, int kernel, double kappa, 
         // UC2UE_l, DC2DE_l
         Bd.kmat(Bd.A.p, zero, kAlphaOuter * r, zero, kAlphaInner * r);
         Bd.pinv(Bd.A.p, Bd.B.p);
-        Bd.store(Bd.B.p, nullptr, O->uc2ue_d.p + l * m2, np);
+        if (need_fp64) Bd.store(Bd.B.p, nullptr, O->uc2ue_d.p + l * m2, np);
         // DC2DE_l (kept in Bd.G's sibling buffer `dc`)
         Bd.kmat(Bd.A.p, zero, kAlphaInner * r, zero, kAlphaOuter * r);
         Bd.pinv(Bd.A.p, dc.p);
-        Bd.store(dc.p, nullptr, O->dc2de_d.p + l * m2, np);
+        if (need_fp64) Bd.store(dc.p, nullptr, O->dc2de_d.p + l * m2, np);
         if (l > 0) {
             // M2M_l[c] = UC2UE_{l-1} K(parent uc, child-c ue); parent half-width 2r
+            const size_t o = (size_t)l * 8 * m2;
             build_ops(st, n, np, OPB_M2M, kernel, kappa, O->surf.p, uc2ue_prev.p, r, kAlphaOuter * 2 * r,
-                      kAlphaInner * r, O->m2m.p + (size_t)l * 8 * m2, need_fp64 ? O->m2m_d.p + (size_t)l * 8 * m2 : nullptr);
+                      kAlphaInner * r, need_fp64 ? nullptr : O->m2m.p + o, need_fp64 ? O->m2m_d.p + o : nullptr);
             // L2L_l[c] = DC2DE_l K(child-c dc, parent de)
             build_ops(st, n, np, OPB_L2L, kernel, kappa, O->surf.p, dc.p, r, kAlphaInner * r, kAlphaOuter * 2 * r,
-                      O->l2l.p + (size_t)l * 8 * m2, need_fp64 ? O->l2l_d.p + (size_t)l * 8 * m2 : nullptr);
+                      need_fp64 ? nullptr : O->l2l.p + o, need_fp64 ? O->l2l_d.p + o : nullptr);
         }
         PB_CUDA(cudaMemcpyAsync(uc2ue_prev.p, Bd.B.p, (size_t)n * n * sizeof(double), cudaMemcpyDeviceToDevice, st));
         // M2L_l[o] = DC2DE_l K(dc of B, ue of the box at offset o); the
         // Laplace operators do not depend on the level (1/r scales as 2^l,
         // the regularised pseudo-inverse as 2^-l): levels below take level 2's
+        const size_t blk = (size_t)kNumOffsets * m2;
         if (l > 2 && kernel == FMM_LAPLACE) {
-            const size_t blk = (size_t)kNumOffsets * m2;
-            PB_CUDA(cudaMemcpyAsync(O->m2l.p + l * blk, O->m2l.p + 2 * blk, blk * sizeof(float),
-                                    cudaMemcpyDeviceToDevice, st));
             if (need_fp64)
                 PB_CUDA(cudaMemcpyAsync(O->m2l_d.p + l * blk, O->m2l_d.p + 2 * blk, blk * sizeof(double),
                                         cudaMemcpyDeviceToDevice, st));
+            else
+                PB_CUDA(cudaMemcpyAsync(O->m2l.p + l * blk, O->m2l.p + 2 * blk, blk * sizeof(float),
+                                        cudaMemcpyDeviceToDevice, st));
         } else if (l >= 2) {
             build_ops(st, n, np, OPB_M2L, kernel, kappa, O->surf.p, dc.p, r, kAlphaInner * r, kAlphaInner * r,
-                      O->m2l.p + (size_t)l * kNumOffsets * m2,
-                      need_fp64 ? O->m2l_d.p + (size_t)l * kNumOffsets * m2 : nullptr);
+                      need_fp64 ? nullptr : O->m2l.p + l * blk, need_fp64 ? O->m2l_d.p + l * blk : nullptr);
         }
         PB_CHECK_LAUNCH();
     }
     // factored UC2UE / DC2DE for the FP32 path: one host job per level and
     // direction, spread over the host cores
-    {
+    if (!need_fp64) {
         std::vector<float> w1((size_t)2 * L * m2), w2((size_t)2 * L * m2);
         std::atomic<int> next(0);
         // Laplace: K scales as 2^l with the level, so the eigenvectors are the
@@ -548,8 +552,10 @@ std::shared_ptr<Operators> get_operators(fmm_tree* T, int kernel, double kappa, 
         PB_CUDA(cudaMemcpyAsync(O->dc2de_w2.p, d2.data(), L * m2 * sizeof(float), cudaMemcpyHostToDevice, st));
         PB_CUDA(cudaStreamSynchronize(st));    // the host vectors go out of scope
     }
-    pack_box_ops_tc(*O, st);
-    pack_m2l_h(*O, st);
+    if (!need_fp64) {
+        pack_box_ops_tc(*O, st);
+        pack_m2l_h(*O, st);
+    }
     PB_CUDA(cudaStreamSynchronize(st));
     T->ops[key] = O;
     auto& cache = T->ctx->op_cache;

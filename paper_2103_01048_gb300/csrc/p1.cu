@@ -24,6 +24,7 @@
 // then the identity terms (the P1 mass matrix) and the lumped-mass
 // preconditioner.
 #include "bem.cuh"
+#include "math64.cuh"
 #include "bem_quad.cuh"
 #include <algorithm>
 #include <cmath>
@@ -468,7 +469,7 @@ __global__ void k_coulomb_dn(long long np, const double* __restrict__ qp, const 
             const double dx = x - s[k].x, dy = y - s[k].y, dz = z - s[k].z;
             const double r2 = dx * dx + dy * dy + dz * dz;
             if (r2 > 0) {
-                const double ri = rsqrt(r2);
+                const double ri = rsqrt64(r2);
                 acc += s[k].w * ri;
                 accd -= s[k].w * (dx * nx + dy * ny + dz * nz) * ri * ri * ri;
             }
@@ -544,7 +545,7 @@ __global__ void k_phi_reac_pts(int na, const double4* __restrict__ atoms, long l
         for (int m = 0; m < cnt; ++m) {
             const double dx = px - s_p[m][0], dy = py - s_p[m][1], dz = pz - s_p[m][2];
             const double r2 = dx * dx + dy * dy + dz * dz;
-            const double rinv = r2 > 0 ? rsqrt(r2) : 0.0;
+            const double rinv = r2 > 0 ? rsqrt64(r2) : 0.0;
             acc += rinv * s_p[m][3] + (dx * s_n[m][0] + dy * s_n[m][1] + dz * s_n[m][2]) * rinv * rinv * rinv;
         }
     }
