@@ -34,18 +34,13 @@ __global__ void k_rhs(int nt, int nq, const double* __restrict__ f, const double
 __global__ void k_dots(long long n, const double* __restrict__ V, long long ld, int nk, const double* __restrict__ w,
                        double* __restrict__ partial, int kmax);
 __global__ void k_dots_reduce(int nblk, int nk, const double* __restrict__ partial, int kmax, double* __restrict__ h,
-                              int accumulate);
-__global__ void k_update(long long n, const double* __restrict__ V, long long ld, int nk, const double* __restrict__ h,
-                         double* __restrict__ w);
+                              int accumulate, double* __restrict__ hsum);
 __global__ void k_scale(long long n, const double* __restrict__ w, const double* __restrict__ nrm2,
                         double* __restrict__ out);
-__global__ void k_givens(int j, int kmax, const double* __restrict__ h, const double* __restrict__ nrm2, double* H,
-                         double* cs, double* sn, double* g, double* resid);
 __global__ void k_backsolve(int m, int kmax, const double* __restrict__ H, const double* __restrict__ g, double* y);
 __global__ void k_axpy_basis(long long n, const double* __restrict__ V, long long ld, int m,
                              const double* __restrict__ y, double* __restrict__ x);
 __global__ void k_set_g0(const double* nrm2, double* g);
-__global__ void k_vadd(int n, const double* a, double* b);
 
 constexpr int kDotBlocksB = 304;
 
@@ -73,35 +68,20 @@ __global__ void k_b_copy_in(long long n, const double* __restrict__ V, const Bat
 __global__ void k_b_dots(long long n, const double* __restrict__ V, long long ld, const double* __restrict__ w,
                          double* __restrict__ partial, int kmax, const BatchDev* __restrict__ d, int all) {
     if (d->done) return;
-    __shared__ double red[256];
-    const int nk = all ? d->j + 1 : 1;
-    const double* base = all ? V : w;
-    long long chunk = (n + gridDim.x - 1) / gridDim.x;
-    long long i0 = blockIdx.x * chunk, i1 = min(n, i0 + chunk);
-    for (int k = 0; k < nk; ++k) {
-        double s = 0.0;
-        const double* v = base + (long long)k * ld;
-        for (long long i = i0 + threadIdx.x; i < i1; i += blockDim.x) s += v[i] * w[i];
-        red[threadIdx.x] = s;
-        __syncthreads();
-        for (int o = 128; o > 0; o >>= 1) {
-            if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) partial[(long long)blockIdx.x * kmax + k] = red[0];
-        __syncthreads();
-    }
+    long long i0, i1;
+    block_rows(n, i0, i1);
+    block_dots(i0, i1, all ? V : w, ld, all ? d->j + 1 : 1, w, partial + (long long)blockIdx.x * kmax);
 }
 
+// one warp per k, four k per block
 __global__ void k_b_dots_reduce(int nblk, const double* __restrict__ partial, int kmax, double* __restrict__ h,
                                 const BatchDev* __restrict__ d, int all) {
     if (d->done) return;
     const int nk = all ? d->j + 1 : 1;
-    const int k = threadIdx.x + blockIdx.x * blockDim.x;
+    const int k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (k >= nk) return;
-    double s = 0.0;
-    for (int b = 0; b < nblk; ++b) s += partial[(long long)b * kmax + k];
-    h[k] = s;
+    const double s = warp_sum_partials(nblk, partial, kmax, k);
+    if ((threadIdx.x & 31) == 0) h[k] = s;
 }
 
 // w -= sum_k h[k] V[k], k <= j (h staged in shared memory, kmax + 1 doubles)
@@ -197,7 +177,7 @@ static void batch_dots(BatchSystem& S, const double* Vb, int nk, const double* v
     cudaStream_t st = S.sub.stream;
     k_dots<<<S.nb, 256, 0, st>>>(S.n, Vb, S.n, nk, vec, S.partial.p, S.kmax + 1);
     PB_CHECK_LAUNCH();
-    k_dots_reduce<<<div_up(nk, 128), 128, 0, st>>>(S.nb, nk, S.partial.p, S.kmax + 1, out, acc);
+    k_dots_reduce<<<div_up(nk, 4), 128, 0, st>>>(S.nb, nk, S.partial.p, S.kmax + 1, out, acc, nullptr);
     PB_CHECK_LAUNCH();
 }
 
@@ -349,8 +329,7 @@ void solve_batch(pb_ctx* ctx, pb_mesh* const* meshes, int nsys, pb_result** resu
                 for (int pass = 0; pass < 2; ++pass) {       // CGS2
                     double* hp = pass == 0 ? S.h.p : S.h2.p;
                     k_b_dots<<<S.nb, 256, 0, st>>>(S.n, S.V.p, S.n, S.xout.p, S.partial.p, S.kmax + 1, S.dev.p, 1);
-                    k_b_dots_reduce<<<div_up(S.kmax + 1, 128), 128, 0, st>>>(S.nb, S.partial.p, S.kmax + 1, hp,
-                                                                            S.dev.p, 1);
+                    k_b_dots_reduce<<<div_up(S.kmax + 1, 4), 128, 0, st>>>(S.nb, S.partial.p, S.kmax + 1, hp, S.dev.p, 1);
                     k_b_update<<<S.ub, 256, (S.kmax + 1) * sizeof(double), st>>>(S.n, S.V.p, S.n, hp, S.xout.p,
                                                                                 S.dev.p);
                     PB_CHECK_LAUNCH();

@@ -413,46 +413,44 @@ __global__ void k_energy(int na, const double4* __restrict__ atoms, const double
 constexpr int kDotBlocks = 304;
 
 // partial[blk][k] = sum over the block's rows of V[k][i] w[i], k < nk
-__global__ void k_dots(long long n, const double* __restrict__ V, long long ld, int nk, const double* __restrict__ w,
-                       double* __restrict__ partial, int kmax) {
-    __shared__ double red[256];
-    long long chunk = (n + gridDim.x - 1) / gridDim.x;
-    long long i0 = blockIdx.x * chunk, i1 = min(n, i0 + chunk);
-    for (int k = 0; k < nk; ++k) {
-        double s = 0.0;
-        const double* v = V + (long long)k * ld;
-        for (long long i = i0 + threadIdx.x; i < i1; i += blockDim.x) s += v[i] * w[i];
-        red[threadIdx.x] = s;
-        __syncthreads();
-        for (int o = 128; o > 0; o >>= 1) {
-            if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) partial[(long long)blockIdx.x * kmax + k] = red[0];
-        __syncthreads();
+__global__ void __launch_bounds__(256) k_dots(long long n, const double* __restrict__ V, long long ld, int nk,
+                                              const double* __restrict__ w, double* __restrict__ partial, int kmax) {
+    long long i0, i1;
+    block_rows(n, i0, i1);
+    block_dots(i0, i1, V, ld, nk, w, partial + (long long)blockIdx.x * kmax);
+}
+
+// h[k] = sum (or += with accumulate); one warp per k, 128 threads per block
+// of four k.  hsum, if not null, takes h[k] added to it.
+__global__ void k_dots_reduce(int nblk, int nk, const double* __restrict__ partial, int kmax, double* __restrict__ h,
+                              int accumulate, double* __restrict__ hsum) {
+    const int k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (k >= nk) return;
+    const double s = warp_sum_partials(nblk, partial, kmax, k);
+    if ((threadIdx.x & 31) == 0) {
+        h[k] = accumulate ? h[k] + s : s;
+        if (hsum) hsum[k] += s;
     }
 }
 
-__global__ void k_dots_reduce(int nblk, int nk, const double* __restrict__ partial, int kmax, double* __restrict__ h,
-                              int accumulate) {
-    int k = threadIdx.x + blockIdx.x * blockDim.x;
-    if (k >= nk) return;
-    double s = 0.0;
-    for (int b = 0; b < nblk; ++b) s += partial[(long long)b * kmax + k];
-    h[k] = accumulate ? h[k] + s : s;
-}
-
-// w -= sum_k h[k] V[k]
-__global__ void k_update(long long n, const double* __restrict__ V, long long ld, int nk, const double* __restrict__ h,
-                         double* __restrict__ w) {
+// w -= sum_k h[k] V[k] on the block's rows, then the partial dots of the new
+// w with the basis (self = 0: second Gram-Schmidt pass) or with itself (1)
+__global__ void __launch_bounds__(256) k_update_dots(long long n, const double* __restrict__ V, long long ld, int nk,
+                                                     const double* __restrict__ h, double* w,
+                                                     double* __restrict__ partial, int kmax, int self) {
     extern __shared__ double sh[];
     for (int k = threadIdx.x; k < nk; k += blockDim.x) sh[k] = h[k];
     __syncthreads();
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    long long i0, i1;
+    block_rows(n, i0, i1);
+    for (long long i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
         double s = w[i];
+#pragma unroll 8
         for (int k = 0; k < nk; ++k) s -= sh[k] * V[(long long)k * ld + i];
         w[i] = s;
     }
+    __syncthreads();
+    block_dots(i0, i1, self ? w : V, ld, self ? 1 : nk, w, partial + (long long)blockIdx.x * kmax);
 }
 
 // out = w / nrm  (nrm = sqrt(*nrm2)); used for V[j+1]
@@ -462,29 +460,48 @@ __global__ void k_scale(long long n, const double* __restrict__ w, const double*
         out[i] = w[i] * inv;
 }
 
-// Hessenberg column j (h[0..j], h[j+1] = ||w||^2 on input) -> Givens update.
+// ||w||^2 from the blocks' partial results, then Hessenberg column j (h[0..j],
+// ||w||) -> Givens update; one block of 128 threads, the column and the
+// rotations staged in shared memory (3 (j + 2) doubles) for the serial chain.
 // H is column-major [kmax+1][kmax]; g, cs, sn of length kmax+1.
-__global__ void k_givens(int j, int kmax, const double* __restrict__ h, const double* __restrict__ nrm2,
-                         double* H, double* cs, double* sn, double* g, double* resid) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double* col = H + (long long)j * (kmax + 1);
-    for (int k = 0; k <= j; ++k) col[k] = h[k];
-    col[j + 1] = sqrt(*nrm2);
-    for (int k = 0; k < j; ++k) {
-        double a = col[k], b = col[k + 1];
-        col[k] = cs[k] * a + sn[k] * b;
-        col[k + 1] = -sn[k] * a + cs[k] * b;
+__global__ void __launch_bounds__(128) k_norm_givens(int nblk, const double* __restrict__ partial, int j, int kmax,
+                                                     const double* __restrict__ h, double* nrm2, double* H, double* cs,
+                                                     double* sn, double* g, double* resid) {
+    extern __shared__ double sh[];
+    double *col = sh, *c0 = sh + j + 2, *s0 = c0 + j + 1;
+    for (int k = threadIdx.x; k <= j; k += blockDim.x) {
+        col[k] = h[k];
+        if (k < j) { c0[k] = cs[k]; s0[k] = sn[k]; }
     }
-    double a = col[j], b = col[j + 1];
-    double r = hypot(a, b);
-    double c = r > 0 ? a / r : 1.0, s = r > 0 ? b / r : 0.0;
-    cs[j] = c;
-    sn[j] = s;
-    col[j] = r;
-    col[j + 1] = 0.0;
-    g[j + 1] = -s * g[j];
-    g[j] = c * g[j];
-    resid[0] = fabs(g[j + 1]);
+    if (threadIdx.x < 32) {
+        const double s = warp_sum_partials(nblk, partial, kmax + 1, 0);
+        if (threadIdx.x == 0) {
+            nrm2[0] = s;
+            col[j + 1] = sqrt(s);
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double a = col[0];
+        for (int k = 0; k < j; ++k) {
+            const double b = col[k + 1];
+            col[k] = c0[k] * a + s0[k] * b;
+            a = -s0[k] * a + c0[k] * b;
+        }
+        const double b = col[j + 1];
+        const double r = hypot(a, b);
+        const double c = r > 0 ? a / r : 1.0, s = r > 0 ? b / r : 0.0;
+        cs[j] = c;
+        sn[j] = s;
+        col[j] = r;
+        col[j + 1] = 0.0;
+        g[j + 1] = -s * g[j];
+        g[j] = c * g[j];
+        resid[0] = fabs(g[j + 1]);
+    }
+    __syncthreads();
+    double* out = H + (long long)j * (kmax + 1);
+    for (int k = threadIdx.x; k <= j + 1; k += blockDim.x) out[k] = col[k];
 }
 
 __global__ void k_backsolve(int m, int kmax, const double* __restrict__ H, const double* __restrict__ g, double* y) {
@@ -510,11 +527,6 @@ __global__ void k_axpy_basis(long long n, const double* __restrict__ V, long lon
 }
 
 __global__ void k_set_g0(const double* nrm2, double* g) { g[0] = sqrt(*nrm2); }
-
-__global__ void k_vadd(int n, const double* a, double* b) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) b[i] += a[i];
-}
 
 // ---------------------------------------------------------------------------
 // host side
@@ -711,15 +723,15 @@ int gmres(pb_mesh* M, const std::function<void(const double*, double*)>& matvec,
     x.alloc(n, st);
     x.zero(st);
     const int nb = std::min<long long>(kDotBlocks, (n + 255) / 256);
-    auto dots = [&](const double* Vb, int nk, const double* vec, double* out, int acc) {
-        k_dots<<<nb, 256, 0, st>>>(n, Vb, n, nk, vec, partial.p, kmax + 1);
-        PB_CHECK_LAUNCH();
-        k_dots_reduce<<<div_up(nk, 128), 128, 0, st>>>(nb, nk, partial.p, kmax + 1, out, acc);
+    auto reduce = [&](int nk, double* out, double* sum) {
+        k_dots_reduce<<<div_up(nk, 4), 128, 0, st>>>(nb, nk, partial.p, kmax + 1, out, 0, sum);
         PB_CHECK_LAUNCH();
     };
     const int ub = std::min<long long>(4 * M->ctx->sm_count, (n + 255) / 256);
     // r0 = P^{-1} b (b is already preconditioned), beta = ||r0||
-    dots(b, 1, b, nrm2.p, 0);
+    k_dots<<<nb, 256, 0, st>>>(n, b, n, 1, b, partial.p, kmax + 1);
+    PB_CHECK_LAUNCH();
+    reduce(1, nrm2.p, nullptr);
     double beta = std::sqrt(read_scalar(nrm2.p, st));
     if (beta == 0.0) { *iterations = 0; *residual = 0.0; return PB_OK; }
     k_scale<<<ub, 256, 0, st>>>(n, b, nrm2.p, V.p);
@@ -731,17 +743,19 @@ int gmres(pb_mesh* M, const std::function<void(const double*, double*)>& matvec,
     for (j = 0; j < kmax; ++j) {
         matvec(V.p + (long long)j * n, w.p);
         PhaseTimer ph(M->ctx, PB_PH_GMRES);
-        // CGS2: two passes of classical Gram-Schmidt
-        dots(V.p, j + 1, w.p, h.p, 0);
-        k_update<<<ub, 256, (j + 1) * sizeof(double), st>>>(n, V.p, n, j + 1, h.p, w.p);
+        // CGS2: two passes of classical Gram-Schmidt, each update fused with
+        // the products that follow it
+        const size_t sm = (j + 1) * sizeof(double);
+        k_dots<<<nb, 256, 0, st>>>(n, V.p, n, j + 1, w.p, partial.p, kmax + 1);
         PB_CHECK_LAUNCH();
-        dots(V.p, j + 1, w.p, h2.p, 0);
-        k_update<<<ub, 256, (j + 1) * sizeof(double), st>>>(n, V.p, n, j + 1, h2.p, w.p);
+        reduce(j + 1, h.p, nullptr);
+        k_update_dots<<<nb, 256, sm, st>>>(n, V.p, n, j + 1, h.p, w.p, partial.p, kmax + 1, 0);
         PB_CHECK_LAUNCH();
-        k_vadd<<<div_up(j + 1, 128), 128, 0, st>>>(j + 1, h2.p, h.p);
+        reduce(j + 1, h2.p, h.p);
+        k_update_dots<<<nb, 256, sm, st>>>(n, V.p, n, j + 1, h2.p, w.p, partial.p, kmax + 1, 1);
         PB_CHECK_LAUNCH();
-        dots(w.p, 1, w.p, nrm2.p, 0);
-        k_givens<<<1, 1, 0, st>>>(j, kmax, h.p, nrm2.p, H.p, cs.p, sn.p, g.p, resid.p);
+        k_norm_givens<<<1, 128, 3 * (j + 2) * sizeof(double), st>>>(nb, partial.p, j, kmax, h.p, nrm2.p, H.p, cs.p, sn.p,
+                                                                     g.p, resid.p);
         PB_CHECK_LAUNCH();
         k_scale<<<ub, 256, 0, st>>>(n, w.p, nrm2.p, V.p + (long long)(j + 1) * n);
         PB_CHECK_LAUNCH();

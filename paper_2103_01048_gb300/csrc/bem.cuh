@@ -50,6 +50,51 @@ struct pb_mesh {
 };
 
 namespace pbfmm {
+// ---- Gram-Schmidt products of the GMRES kernels (bem.cu, batch.cu)
+// partial[k] = sum over the rows [i0, i1) of V[k][i] w[i], k < nk: one warp per
+// four vectors (one read of w for four products), no block barrier.  The
+// basis is read once per pass; at the sizes of a solve it stays in L2 and the
+// pass is bound by its latency (a barrier tree per vector took 1.5 us each).
+__device__ __forceinline__ void block_dots(long long i0, long long i1, const double* V, long long ld,
+                                           int nk, const double* w, double* __restrict__ partial) {
+    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    for (int k0 = (threadIdx.x >> 5) * 4; k0 < nk; k0 += nw * 4) {
+        double s[4] = {0.0, 0.0, 0.0, 0.0};
+        const int m = min(4, nk - k0);
+        const double* v = V + (long long)k0 * ld;
+        if (m == 4) {
+            for (long long i = i0 + lane; i < i1; i += 32) {
+                const double x = w[i];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) s[u] += v[u * ld + i] * x;
+            }
+        } else {
+            for (long long i = i0 + lane; i < i1; i += 32) {
+                const double x = w[i];
+                for (int u = 0; u < m; ++u) s[u] += v[u * ld + i] * x;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            for (int o = 16; o > 0; o >>= 1) s[u] += __shfl_xor_sync(0xffffffffu, s[u], o);
+            if (lane == 0 && u < m) partial[k0 + u] = s[u];
+        }
+    }
+}
+__device__ __forceinline__ void block_rows(long long n, long long& i0, long long& i1) {
+    const long long chunk = (n + gridDim.x - 1) / gridDim.x;
+    i0 = min(n, blockIdx.x * chunk);
+    i1 = min(n, i0 + chunk);
+}
+
+// sum over the blocks' partial results of one k, by a warp (fixed order)
+__device__ __forceinline__ double warp_sum_partials(int nblk, const double* __restrict__ partial, int kmax, int k) {
+    double s = 0.0;
+    for (int b = threadIdx.x & 31; b < nblk; b += 32) s += partial[(long long)b * kmax + k];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+
 int gmres(pb_mesh* M, const std::function<void(const double*, double*)>& matvec, const double* b, DBuf<double>& x,
           double tol, int max_iter, int* iterations, double* residual);
 void ensure_singular_public(pb_mesh* M, double kappa);
