@@ -1043,33 +1043,39 @@ __device__ __forceinline__ f32x2 x2_exp2(f32x2 a) { return x2_pack(exp2_t<float>
 // A = {x, y}, B = {z, qL}, C = {mx, my}, D = {mz, qY}, each a pair.
 // KM: 3 both kernels; 1 Laplace only (density qL, sum pL); 2 Yukawa only
 // (density in the qL slot, sum pY).
-template <bool DL, bool GUARD, int KM = 3>
+// DN (monopoles only): dL, dY take the sums of -dg/dn_x q, n the target normal.
+template <bool DL, bool DN, bool GUARD, int KM = 3>
 __device__ __forceinline__ void interact_x2(f32x2 X, f32x2 Y, f32x2 Z, const ulonglong2& A, const ulonglong2& B,
                                             const ulonglong2& C, const ulonglong2& D, f32x2 kap, f32x2 kl2,
-                                            f32x2 one, f32x2& pL, f32x2& pY) {
+                                            f32x2& pL, f32x2& pY, f32x2 NX = 0, f32x2 NY = 0, f32x2 NZ = 0,
+                                            f32x2* dL = nullptr, f32x2* dY = nullptr) {
     const f32x2 dx = x2_sub(X, A.x), dy = x2_sub(Y, A.y), dz = x2_sub(Z, B.x);
     const f32x2 r2 = x2_fma(dx, dx, x2_fma(dy, dy, x2_mul(dz, dz)));
     const f32x2 rinv = x2_rsqrt<GUARD>(r2);
-    if (KM == 1) {
-        if (DL) {
-            const f32x2 w = x2_mul(x2_fma(dx, C.x, x2_fma(dy, C.y, x2_mul(dz, D.x))), x2_mul(rinv, rinv));
-            pL = x2_fma(rinv, x2_add(w, B.y), pL);
-        } else {
-            pL = x2_fma(rinv, B.y, pL);
-        }
-        return;
-    }
-    const f32x2 r = x2_mul(r2, rinv);
-    const f32x2 er = x2_mul(x2_exp2(x2_mul(kl2, r)), rinv);        // e^{-kr} / r
+    f32x2 er = 0;
+    if (KM & 2) er = x2_mul(x2_exp2(x2_mul(kl2, x2_mul(r2, rinv))), rinv);        // e^{-kr} / r
+    const f32x2 qY = KM == 3 ? D.y : B.y;
     if (DL) {
         const f32x2 rinv2 = x2_mul(rinv, rinv);
-        const f32x2 u = x2_fma(kap, r, one);
-        const f32x2 w = x2_mul(x2_fma(dx, C.x, x2_fma(dy, C.y, x2_mul(dz, D.x))), rinv2);
-        if (KM == 3) pL = x2_fma(rinv, x2_add(w, B.y), pL);
-        pY = x2_fma(er, x2_fma(w, u, KM == 3 ? D.y : B.y), pY);
+        const f32x2 dm = x2_fma(dx, C.x, x2_fma(dy, C.y, x2_mul(dz, D.x)));
+        if (KM & 1) pL = x2_fma(rinv, x2_fma(dm, rinv2, B.y), pL);
+        if (KM & 2) pY = x2_fma(er, x2_fma(dm, x2_fma(kap, rinv, rinv2), qY), pY);   // (1 + kr) / r^2 = 1/r^2 + k/r
+    } else if (DN) {
+        const f32x2 rinv2 = x2_mul(rinv, rinv);
+        const f32x2 dn = x2_fma(dx, NX, x2_fma(dy, NY, x2_mul(dz, NZ)));
+        if (KM & 1) {
+            const f32x2 g = x2_mul(rinv, B.y);
+            pL = x2_add(pL, g);
+            *dL = x2_fma(x2_mul(dn, rinv2), g, *dL);
+        }
+        if (KM & 2) {
+            const f32x2 g = x2_mul(er, qY);
+            pY = x2_add(pY, g);
+            *dY = x2_fma(x2_mul(dn, x2_fma(kap, rinv, rinv2)), g, *dY);
+        }
     } else {
-        if (KM == 3) pL = x2_fma(rinv, B.y, pL);
-        pY = x2_fma(er, KM == 3 ? D.y : B.y, pY);
+        if (KM & 1) pL = x2_fma(rinv, B.y, pL);
+        if (KM & 2) pY = x2_fma(er, qY, pY);
     }
 }
 
@@ -1120,15 +1126,17 @@ __device__ __forceinline__ void put_src_x2(ulonglong2* sA, ulonglong2* sB, ulong
     d[h] = mz; d[2 + h] = qY;
 }
 
-// The paired leaf kernel in packed FP32 (no target-normal derivatives): the
-// work split of k_leaf_pair (NT targets per thread, G groups, the near field
+// The paired leaf kernel in packed FP32: the work split of k_leaf_pair (NT targets per thread, G groups, the near field
 // in windows of the concatenated U-list sources, the leaf itself first, then
 // the far field in windows of generated equivalent points), with each window
 // stored as pairs of points, every value pair one 64-bit half of a 16-byte
 // vector, so that group g takes the pairs g, g + G, ... and one packed
 // instruction serves two sources.  An odd window is padded with a point of
 // zero weight 1e10 away (its terms are exactly 0).
-template <bool DL, int NT, int PART, int KM = 3>
+// Grid y: the windows are dealt out to S = gridDim.y CTAs (windows of 1,024 / S
+// points), each with its own partial outputs, added in order by the scatter:
+// trees of a few hundred leaves fill the GPU (see leaf_split).
+template <bool DL, bool DN, int NT, int PART, int KM, bool SPLIT>
 __global__ void __launch_bounds__(128, 5) k_leaf_pair_x2(const int* __restrict__ leaves, int nleaf,
                                                       const int* __restrict__ tb, const int* __restrict__ te,
                                                       const int* __restrict__ sb, const int* __restrict__ se,
@@ -1142,11 +1150,15 @@ __global__ void __launch_bounds__(128, 5) k_leaf_pair_x2(const int* __restrict__
                                                       const float* __restrict__ QdY, const float4* __restrict__ surf,
                                                       int ne, int npad, float kappa, float* __restrict__ potL_out,
                                                       float* __restrict__ potY_out, const int* __restrict__ Xl,
-                                                      const int* __restrict__ Xn, int thrW, int thrX) {
+                                                      const int* __restrict__ Xn, int thrW, int thrX,
+                                                      const float4* __restrict__ tn, float* __restrict__ dnL_out,
+                                                      float* __restrict__ dnY_out, long long part_stride) {
     constexpr int CH = 128;
     constexpr int CAP = 1024;                    // points per window (512 pairs, 32 KB)
     constexpr int CP = CAP / 2;
-    static_assert(2 * NT * CH * 4 <= CP * 16, "reduction fits one staging array");
+    constexpr int NR = DN ? 4 : 2;
+    static_assert(NR * NT * CH * 4 <= CP * 16, "reduction fits one staging array");
+    static_assert(!(DL && DN), "no hypersingular kernel");
     __shared__ ulonglong2 sA[CP], sB[CP], sC[CP], sD[CP];
     __shared__ int s_self;
     constexpr int VC = 256;                      // near-list entries resolved per chunk
@@ -1160,6 +1172,11 @@ __global__ void __launch_bounds__(128, 5) k_leaf_pair_x2(const int* __restrict__
     float* s_red = reinterpret_cast<float*>(sA);
     const int li = blockIdx.x;
     if (li >= nleaf) return;
+    const int sp = SPLIT ? blockIdx.y : 0, S = SPLIT ? gridDim.y : 1, wcap = SPLIT ? CAP / S : CAP;
+    if (KM & 1) potL_out += sp * part_stride;
+    if (KM & 2) potY_out += sp * part_stride;
+    if (DN && (KM & 1)) dnL_out += sp * part_stride;
+    if (DN && (KM & 2)) dnY_out += sp * part_stride;
     const int b = leaves[li];
     const int t0 = tb[b], t1 = te[b];
     const int slots = min(CH, max(4, (t1 - t0 + NT - 1) / NT));
@@ -1177,7 +1194,7 @@ __global__ void __launch_bounds__(128, 5) k_leaf_pair_x2(const int* __restrict__
     const int* xl = Xl + (long long)b * kXCap;
     const double4 cb = center[b];
     const float kl2s = -kappa * float(kLog2E);
-    const f32x2 kap = x2_pack(kappa, kappa), kl2 = x2_pack(kl2s, kl2s), one = x2_pack(1.f, 1.f);
+    const f32x2 kap = x2_pack(kappa, kappa), kl2 = x2_pack(kl2s, kl2s);
     if (threadIdx.x == 0) s_self = -1;
     __syncthreads();
     for (int i = threadIdx.x; i < nu; i += CH)
@@ -1234,6 +1251,7 @@ __global__ void __launch_bounds__(128, 5) k_leaf_pair_x2(const int* __restrict__
         int ti[NT];
         bool vt[NT];
         f32x2 X[NT], Y[NT], Z[NT], pL[NT], pY[NT];
+        f32x2 NX[DN ? NT : 1], NY[DN ? NT : 1], NZ[DN ? NT : 1], dL[DN ? NT : 1], dY[DN ? NT : 1];
         float xs[NT], ys[NT], zs[NT];
 #pragma unroll
         for (int u = 0; u < NT; ++u) {
@@ -1243,13 +1261,19 @@ __global__ void __launch_bounds__(128, 5) k_leaf_pair_x2(const int* __restrict__
             xs[u] = x.x; ys[u] = x.y; zs[u] = x.z;
             X[u] = x2_pack(x.x, x.x); Y[u] = x2_pack(x.y, x.y); Z[u] = x2_pack(x.z, x.z);
             pL[u] = pY[u] = 0ull;
+            if (DN) {
+                const float4 m = vt[u] ? tn[ti[u]] : make_float4(0, 0, 0, 0);
+                NX[u] = x2_pack(m.x, m.x); NY[u] = x2_pack(m.y, m.y); NZ[u] = x2_pack(m.z, m.z);
+                dL[u] = dY[u] = 0ull;
+            }
         }
         if (PART != 2) {
-            int vi = 0, off = 0;
+            int vi = 0, off = 0, win = 0;
             while (vi < nvirt) {
+                const bool mine = !SPLIT || win++ % S == sp;
                 const int self_left = (selfpos >= 0 && vi == 0) ? nself - off : 0;
                 int filled = 0;
-                while (filled < CAP && vi < nvirt) {
+                while (filled < wcap && vi < nvirt) {
                     if (vi >= vbase + VC) {      // next chunk of resolved entries
                         __syncthreads();
                         vbase += VC;
@@ -1257,12 +1281,13 @@ __global__ void __launch_bounds__(128, 5) k_leaf_pair_x2(const int* __restrict__
                         __syncthreads();
                     }
                     const int j0 = s_vb[vi - vbase] + off, len = s_vn[vi - vbase] - off;
-                    const int take = min(len, CAP - filled);
-                    for (int e = threadIdx.x; e < take; e += CH)
+                    const int take = min(len, wcap - filled);
+                    for (int e = threadIdx.x; mine && e < take; e += CH)
                         copy_src_x2<DL, KM == 3>(sA, sB, sC, sD, filled + e, sq, sm, j0 + e);
                     filled += take;
                     if (take == len) { ++vi; off = 0; } else off += take;
                 }
+                if (!mine) continue;
                 if ((filled & 1) && threadIdx.x == 0)
                     put_src_x2(sA, sB, sC, sD, filled, 1e10f, 1e10f, 1e10f, 0.f, 0.f, 0.f, 0.f, 0.f);
                 cp_async_wait_all();
@@ -1274,14 +1299,18 @@ __global__ void __launch_bounds__(128, 5) k_leaf_pair_x2(const int* __restrict__
                     const ulonglong2 A = sA[k], B = sB[k], C = DL ? sC[k] : make_ulonglong2(0, 0), D = sD[k];
 #pragma unroll
                     for (int u = 0; u < NT; ++u)
-                        interact_x2<DL, true, KM>(X[u], Y[u], Z[u], A, B, C, D, kap, kl2, one, pL[u], pY[u]);
+                        interact_x2<DL, DN, true, KM>(X[u], Y[u], Z[u], A, B, C, D, kap, kl2, pL[u], pY[u],
+                                                          NX[DN ? u : 0], NY[DN ? u : 0], NZ[DN ? u : 0],
+                                                          &dL[DN ? u : 0], &dY[DN ? u : 0]);
                 }
 #pragma unroll 2
                 for (; active && k < np; k += G) {
                     const ulonglong2 A = sA[k], B = sB[k], C = DL ? sC[k] : make_ulonglong2(0, 0), D = sD[k];
 #pragma unroll
                     for (int u = 0; u < NT; ++u)
-                        interact_x2<DL, false, KM>(X[u], Y[u], Z[u], A, B, C, D, kap, kl2, one, pL[u], pY[u]);
+                        interact_x2<DL, DN, false, KM>(X[u], Y[u], Z[u], A, B, C, D, kap, kl2, pL[u], pY[u],
+                                                          NX[DN ? u : 0], NY[DN ? u : 0], NZ[DN ? u : 0],
+                                                          &dL[DN ? u : 0], &dY[DN ? u : 0]);
                 }
                 __syncthreads();
             }
@@ -1293,8 +1322,8 @@ __global__ void __launch_bounds__(128, 5) k_leaf_pair_x2(const int* __restrict__
                             rz = (float)((double)zs[u] - cb.z);
                 X[u] = x2_pack(rx, rx); Y[u] = x2_pack(ry, ry); Z[u] = x2_pack(rz, rz);
             }
-            const int nbw = CAP / ne;                    // whole boxes per window (ne <= CAP: host)
-            int fcur = 0;                                // next far candidate: W list, then the leaf's own
+            const int nbw = max(1, wcap / ne);           // whole boxes per window (ne <= CAP: host)
+            int fcur = 0, win = 0;                                // next far candidate: W list, then the leaf's own
             while (fcur < nsrcbox) {
                 if (fcur >= fbase + FC) {                // next chunk of resolved candidates
                     __syncthreads();
@@ -1329,6 +1358,10 @@ __global__ void __launch_bounds__(128, 5) k_leaf_pair_x2(const int* __restrict__
                 __syncthreads();
                 const int nb = s_nb, n = nb * ne;
                 fcur = s_fcur;
+                if (SPLIT && win++ % S != sp) {
+                    __syncthreads();                     // s_nb is read before the next pick
+                    continue;
+                }
                 for (int i = 0; i < nb; ++i) {
                     const int slot = s_sel[i];
                     const float4 bx = s_fb[slot];
@@ -1353,7 +1386,9 @@ __global__ void __launch_bounds__(128, 5) k_leaf_pair_x2(const int* __restrict__
                     const ulonglong2 A = sA[k], B = sB[k], D = sD[k];
 #pragma unroll
                     for (int u = 0; u < NT; ++u)
-                        interact_x2<false, false, KM>(X[u], Y[u], Z[u], A, B, C0, D, kap, kl2, one, pL[u], pY[u]);
+                        interact_x2<false, DN, false, KM>(X[u], Y[u], Z[u], A, B, C0, D, kap, kl2, pL[u], pY[u],
+                                                          NX[DN ? u : 0], NY[DN ? u : 0], NZ[DN ? u : 0],
+                                                          &dL[DN ? u : 0], &dY[DN ? u : 0]);
                 }
                 __syncthreads();
             }
@@ -1363,24 +1398,31 @@ __global__ void __launch_bounds__(128, 5) k_leaf_pair_x2(const int* __restrict__
         for (int u = 0; u < NT; ++u) {
             s_red[u * CH + threadIdx.x] = x2_lo(pL[u]) + x2_hi(pL[u]);
             s_red[(NT + u) * CH + threadIdx.x] = x2_lo(pY[u]) + x2_hi(pY[u]);
+            if (DN) {
+                s_red[((NR - 2) * NT + u) * CH + threadIdx.x] = x2_lo(dL[u]) + x2_hi(dL[u]);
+                s_red[((NR - 1) * NT + u) * CH + threadIdx.x] = x2_lo(dY[u]) + x2_hi(dY[u]);
+            }
         }
         __syncthreads();
         if (g == 0) {
 #pragma unroll
             for (int u = 0; u < NT; ++u) {
-                float a0 = 0.f, a1 = 0.f;
+                float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
                 for (int q = 0; q < G; ++q) {
-                    a0 += s_red[u * CH + tloc + q * slots];
-                    a1 += s_red[(NT + u) * CH + tloc + q * slots];
+                    const int o = u * CH + tloc + q * slots;
+                    a0 += s_red[o];
+                    a1 += s_red[NT * CH + o];
+                    if (DN) {
+                        a2 += s_red[(NR - 2) * NT * CH + o];
+                        a3 += s_red[(NR - 1) * NT * CH + o];
+                    }
                 }
                 if (vt[u]) {
-                    if (PART == 2) {
-                        if (KM & 1) potL_out[ti[u]] += a0 * float(kInv4PiD);
-                        if (KM & 2) potY_out[ti[u]] += a1 * float(kInv4PiD);
-                    } else {
-                        if (KM & 1) potL_out[ti[u]] = a0 * float(kInv4PiD);
-                        if (KM & 2) potY_out[ti[u]] = a1 * float(kInv4PiD);
-                    }
+                    const float c4 = float(kInv4PiD);            // (PART 2 adds to the near field)
+                    if (KM & 1) potL_out[ti[u]] = a0 * c4 + (PART == 2 ? potL_out[ti[u]] : 0.f);
+                    if (KM & 2) potY_out[ti[u]] = a1 * c4 + (PART == 2 ? potY_out[ti[u]] : 0.f);
+                    if (DN && (KM & 1)) dnL_out[ti[u]] = -a2 * c4 + (PART == 2 ? dnL_out[ti[u]] : 0.f);
+                    if (DN && (KM & 2)) dnY_out[ti[u]] = -a3 * c4 + (PART == 2 ? dnY_out[ti[u]] : 0.f);
                 }
             }
         }
@@ -1435,7 +1477,7 @@ __global__ void __launch_bounds__(128) k_p2check_pair_x2(int nbox, const int* __
     const int tloc = threadIdx.x % slots, g = threadIdx.x / slots;
     const bool active = g < G;
     const float kl2s = -kappa * float(kLog2E);
-    const f32x2 kap = x2_pack(kappa, kappa), kl2 = x2_pack(kl2s, kl2s), one = x2_pack(1.f, 1.f);
+    const f32x2 kap = x2_pack(kappa, kappa), kl2 = x2_pack(kl2s, kl2s);
     f32x2 PX[NP], PY[NP], PZ[NP], aL[NP], aY[NP];
 #pragma unroll
     for (int m = 0; m < NP; ++m) {
@@ -1470,7 +1512,7 @@ __global__ void __launch_bounds__(128) k_p2check_pair_x2(int nbox, const int* __
             const ulonglong2 A = sA[k], B = sB[k], C = DL ? sC[k] : make_ulonglong2(0, 0), D = sD[k];
 #pragma unroll
             for (int m = 0; m < NP; ++m)
-                interact_x2<DL, false>(PX[m], PY[m], PZ[m], A, B, C, D, kap, kl2, one, aL[m], aY[m]);
+                interact_x2<DL, false, false>(PX[m], PY[m], PZ[m], A, B, C, D, kap, kl2, aL[m], aY[m]);
         }
         __syncthreads();
     }
@@ -1568,39 +1610,45 @@ static void check2equiv(const Operators& O, int level, bool up, cudaStream_t st,
     gemm_dispatch<float, float>(O.npad, st, div_up(ncols, kTC), ga, up ? O.uc2ue_w2.p : O.dc2de_w2.p, tmp, Y);
 }
 
-// CTAs that share a leaf's sources.  FP64: a leaf keeps an SM busy for half a
-// millisecond, and a few hundred of them leave the slowest SM with several
-// times the average, so about 24 CTAs per SM (30,720 points, p = 6: leaf
-// 10.1 -> 4.0 ms).
+// CTAs that share a leaf's sources.  FP32: about 1,200 CTAs, 1.6 per resident
+// slot (five per SM).  FP64: a leaf keeps an SM busy for half a millisecond,
+// and a few hundred of them leave the slowest SM with several times the
+// average, so about 24 CTAs per SM (30,720 points, p = 6: leaf 10.1 -> 4.0 ms).
 static int leaf_split(const fmm_tree* Tr, bool fp64) {
-    if (!fp64 || Tr->n_tleaf <= 0) return 1;
-    return std::max(1, std::min(8, div_up(24LL * Tr->ctx->sm_count, Tr->n_tleaf)));
+    if (Tr->n_tleaf <= 0) return 1;
+    const long long want = fp64 ? 24LL * Tr->ctx->sm_count : 8LL * Tr->ctx->sm_count;
+    const int s = div_up(want, Tr->n_tleaf);
+    if (fp64) return std::max(1, std::min(8, s));
+    return s >= 4 ? 4 : (s >= 2 ? 2 : 1);
 }
 
 template <typename T, bool YUK, bool DL, bool DN>
 static void launch_leaf(cudaStream_t st, fmm_tree* Tr, Work<T>& W, const Operators& O, T kappa, int thrW = -1,
-                        int thrX = -1) {
+                        int thrX = -1, int split = 1) {
     if (Tr->n_tleaf <= 0) return;
     const float4* tpos = Tr->same ? Tr->pos_s.p : Tr->pos_t.p;
     const int* tb = Tr->same ? Tr->sb.p : Tr->tb.p;
     const int* te = Tr->same ? Tr->se.p : Tr->te.p;
-    if constexpr (std::is_same<T, float>::value && !DN) {
+    if constexpr (std::is_same<T, float>::value) {
         if (Tr->ctx->leaf_packed && O.ne <= 1024) {
             // the packed leaf kernel for one kernel (KM 1: Laplace, 2: Yukawa)
             constexpr int KM = YUK ? 2 : 1;
-            const int NT = Tr->ctx->leaf_nt ? Tr->ctx->leaf_nt : 4;
-            auto k = NT == 4 ? k_leaf_pair_x2<DL, 4, 0, KM> : k_leaf_pair_x2<DL, 2, 0, KM>;
-            k<<<Tr->n_tleaf, 128, 0, st>>>(Tr->leaf_ids.p, Tr->n_tleaf, tb, te, Tr->sb.p, Tr->se.p, Tr->U_off.p,
+            const int NT = Tr->ctx->leaf_nt ? Tr->ctx->leaf_nt : (DN ? 2 : 4);
+            auto k = split > 1 ? (NT == 4 ? k_leaf_pair_x2<DL, DN, 4, 0, KM, true> : k_leaf_pair_x2<DL, DN, 2, 0, KM, true>)
+                               : (NT == 4 ? k_leaf_pair_x2<DL, DN, 4, 0, KM, false> : k_leaf_pair_x2<DL, DN, 2, 0, KM, false>);
+            k<<<dim3(Tr->n_tleaf, split), 128, 0, st>>>(Tr->leaf_ids.p, Tr->n_tleaf, tb, te, Tr->sb.p, Tr->se.p, Tr->U_off.p,
                                            Tr->U_ids.p, Tr->W_off.p, Tr->W_ids.p, Tr->level.p, Tr->center.p, tpos,
                                            W.sq.p, W.sm.p, W.Qu.p, W.Qd.p, nullptr, nullptr,
                                            (const float4*)O.surf_f.p, O.ne, O.npad, kappa,
                                            YUK ? nullptr : W.pot.p, YUK ? W.pot.p : nullptr, Tr->X.p, Tr->X_n.p,
-                                           thrW, thrX);
+                                           thrW, thrX, W.tn.p, YUK ? nullptr : W.dn.p, YUK ? W.dn.p : nullptr,
+                                           Tr->same ? Tr->ns : Tr->nt);
             PB_CHECK_LAUNCH();
             return;
         }
     }
-    PB_REQUIRE(thrW < 0 && thrX < 0, PB_EINVAL, "direct W/X-list evaluation needs the packed leaf kernel");
+    PB_REQUIRE(thrW < 0 && thrX < 0 && split == 1, PB_EINVAL,
+               "direct W/X-list evaluation and split leaves need the packed leaf kernel");
     constexpr int NT = 2;     // 4 measured slower (register pressure)
     k_leaf_eval<T, YUK, DL, DN, NT><<<Tr->n_tleaf, 128, 0, st>>>(
         Tr->leaf_ids.p, Tr->n_tleaf, tb, te, Tr->sb.p, Tr->se.p, Tr->U_off.p, Tr->U_ids.p, Tr->W_off.p, Tr->W_ids.p,
@@ -1835,14 +1883,16 @@ static void apply_t(fmm_tree* Tr, const Operators& O, double kappa_d, const In* 
     if (DL && DN) throw Error(PB_EINVAL, "double layer with target-normal derivative is not provided");
     // small W boxes and small leaves' X lists summed directly (see list_direct)
     const int ldm = Tr->ctx->list_direct;
-    const bool ld = std::is_same<T, float>::value && !DN && Tr->ctx->leaf_packed && ldm != 0 && O.ne <= 1024;
+    const bool packed = std::is_same<T, float>::value && Tr->ctx->leaf_packed && O.ne <= 1024;
+    const bool ld = packed && ldm != 0;
+    const int split = packed ? leaf_split(Tr, false) : 1;
     const int thrW = ld && ldm != 2 ? O.ne / 2 : -1, thrX = ld && ldm != 3 ? O.ne : -1;
     Work<T> W;
     W.sq.alloc(ns, st);
     if (DL) W.sm.alloc(ns, st);
     alloc_far(W, Tr->nbox, O.npad, st);
-    W.pot.alloc(nt, st);
-    if (DN) { W.dn.alloc(nt, st); W.tn.alloc(nt, st); }
+    W.pot.alloc(nt * split, st);
+    if (DN) { W.dn.alloc(nt * split, st); W.tn.alloc(nt, st); }
     pb_ctx* ctx = Tr->ctx;
     auto ph = std::make_unique<PhaseTimer>(ctx, PB_PH_GATHER);
     k_gather_src<T, In><<<div_up(ns, 256), 256, 0, st>>>(ns, Tr->perm_s.p, Tr->pos_s.p, q, dip, src_n, W.sq.p,
@@ -1881,14 +1931,14 @@ static void apply_t(fmm_tree* Tr, const Operators& O, double kappa_d, const In* 
     far_l2l(Tr, O, W);
     ph.reset(); ph = std::make_unique<PhaseTimer>(ctx, PB_PH_LEAF);
     // ---- leaves: P2P + M2P + L2P
-    if (DL) launch_leaf<T, YUK, true, false>(st, Tr, W, O, kappa, thrW, thrX);
-    else if (DN) launch_leaf<T, YUK, false, true>(st, Tr, W, O, kappa, thrW, thrX);
-    else launch_leaf<T, YUK, false, false>(st, Tr, W, O, kappa, thrW, thrX);
+    if (DL) launch_leaf<T, YUK, true, false>(st, Tr, W, O, kappa, thrW, thrX, split);
+    else if (DN) launch_leaf<T, YUK, false, true>(st, Tr, W, O, kappa, thrW, thrX, split);
+    else launch_leaf<T, YUK, false, false>(st, Tr, W, O, kappa, thrW, thrX, split);
     ph.reset(); ph = std::make_unique<PhaseTimer>(ctx, PB_PH_SCATTER);
     const int* pt = Tr->same ? Tr->perm_s.p : Tr->perm_t.p;
-    k_scatter<T, In><<<div_up(nt, 256), 256, 0, st>>>(nt, pt, W.pot.p, out);
+    k_scatter<T, In><<<div_up(nt, 256), 256, 0, st>>>(nt, pt, W.pot.p, out, split);
     PB_CHECK_LAUNCH();
-    if (DN) k_scatter<T, In><<<div_up(nt, 256), 256, 0, st>>>(nt, pt, W.dn.p, out_dn);
+    if (DN) k_scatter<T, In><<<div_up(nt, 256), 256, 0, st>>>(nt, pt, W.dn.p, out_dn, split);
     if (DN) PB_CHECK_LAUNCH();
     ph.reset();
 }
@@ -1959,15 +2009,17 @@ static void launch_leaf_pair(cudaStream_t st, fmm_tree* Tr, Work<T>& WL, Work<T>
     const int* tb = Tr->same ? Tr->sb.p : Tr->tb.p;
     const int* te = Tr->same ? Tr->se.p : Tr->te.p;
     const int nt_opt = Tr->ctx->leaf_nt;
-    if constexpr (std::is_same<T, float>::value && !DN) {
+    if constexpr (std::is_same<T, float>::value) {
         if (Tr->ctx->leaf_packed && O.ne <= 1024) {
-            const int NT = nt_opt ? nt_opt : 4;
-            auto k = NT == 4 ? k_leaf_pair_x2<DL, 4, PART> : k_leaf_pair_x2<DL, 2, PART>;
-            k<<<Tr->n_tleaf, 128, 0, st>>>(Tr->leaf_ids.p, Tr->n_tleaf, tb, te, Tr->sb.p, Tr->se.p, Tr->U_off.p,
+            const int NT = nt_opt ? nt_opt : (DN ? 2 : 4);
+            auto k = split > 1 ? (NT == 4 ? k_leaf_pair_x2<DL, DN, 4, PART, 3, true> : k_leaf_pair_x2<DL, DN, 2, PART, 3, true>)
+                               : (NT == 4 ? k_leaf_pair_x2<DL, DN, 4, PART, 3, false> : k_leaf_pair_x2<DL, DN, 2, PART, 3, false>);
+            k<<<dim3(Tr->n_tleaf, split), 128, 0, st>>>(Tr->leaf_ids.p, Tr->n_tleaf, tb, te, Tr->sb.p, Tr->se.p, Tr->U_off.p,
                                            Tr->U_ids.p, Tr->W_off.p, Tr->W_ids.p, Tr->level.p, Tr->center.p, tpos,
                                            WL.sq.p, WL.sm.p, WL.Qu.p, WL.Qd.p, WY.Qu.p, WY.Qd.p,
                                            (const float4*)O.surf_f.p, O.ne, O.npad, kappa, WL.pot.p, WY.pot.p,
-                                           Tr->X.p, Tr->X_n.p, thrW, thrX);
+                                           Tr->X.p, Tr->X_n.p, thrW, thrX, WL.tn.p, WL.dn.p, WY.dn.p,
+                                           Tr->same ? Tr->ns : Tr->nt);
             PB_CHECK_LAUNCH();
             return;
         }
@@ -1989,9 +2041,9 @@ static void launch_leaf_pair(cudaStream_t st, fmm_tree* Tr, Work<T>& WL, Work<T>
 // direct pair with a dipole about twice one of them), and the X list of a
 // leaf of at most n_e targets (P2L would put the same sources on n_e check
 // points).  Returns the two thresholds, -1 when off.
-static void list_direct(const fmm_tree* Tr, const Operators& O, bool fp32, bool DN, int& thrW, int& thrX) {
+static void list_direct(const fmm_tree* Tr, const Operators& O, bool fp32, int& thrW, int& thrX) {
     const int mode = Tr->ctx->list_direct;         // 0 off, 1 W and X, 2 X only, 3 W only
-    const bool on = fp32 && !DN && Tr->ctx->leaf_packed && mode != 0 && O.ne <= 1024;
+    const bool on = fp32 && Tr->ctx->leaf_packed && mode != 0 && O.ne <= 1024;
     thrW = on && mode != 2 ? O.ne / 2 : -1;
     thrX = on && mode != 3 ? O.ne : -1;
 }
@@ -2006,7 +2058,7 @@ static void apply_pair_t(fmm_tree* Tr, const Operators& OL, const Operators& OY,
     const bool DL = dip != nullptr, DN = dnL != nullptr;
     if (DL && DN) throw Error(PB_EINVAL, "double layer with target-normal derivative is not provided");
     int thrW, thrX;
-    list_direct(Tr, OL, std::is_same<T, float>::value, DN, thrW, thrX);
+    list_direct(Tr, OL, std::is_same<T, float>::value, thrW, thrX);
     Work<T> WL, WY;
     WL.sq.alloc(ns, st);
     WL.sm.alloc(ns, st);
