@@ -925,6 +925,9 @@ static bool matvec_graph(pb_mesh* M, pb_result* R) {
     sub.coupling = ctx->coupling;
     sub.deterministic = ctx->deterministic;
     sub.singular = ctx->singular;
+    sub.leaf_nt = ctx->leaf_nt;
+    sub.leaf_packed = ctx->leaf_packed;
+    sub.list_direct = ctx->list_direct;
     sub.overlap = ctx->overlap;
     sub.aux = ctx->aux;                 // joins the capture through the fork event
     sub.ev_fork = ctx->ev_fork;

@@ -1126,6 +1126,127 @@ __device__ __forceinline__ void put_src_x2(ulonglong2* sA, ulonglong2* sB, ulong
     d[h] = mz; d[2 + h] = qY;
 }
 
+// ---------------------------------------------------------------------------
+// Source streams of the packed leaf kernel, one record per target leaf: the
+// leaf's near sources as ranges of the sorted points (its own first, then the
+// U list, the W boxes of at most thrW sources and, for leaves of at most thrX
+// targets, the X list; neighbouring ranges joined) and the far boxes (the
+// other W boxes and the leaf's own downward surface).  Built once per tree
+// and pair of thresholds, one warp per leaf; in the leaf kernel the lists
+// were seven dependent loads and a scan over every entry, 0.76 of 4.0 ms at
+// 4M points, p = 6.  Kept until the tree goes: captured graphs point to them.
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(128) k_leaf_stream(
+    int nleaf, const int* __restrict__ leaves, const int* __restrict__ tb, const int* __restrict__ te,
+    const int* __restrict__ sb, const int* __restrict__ se, const int* __restrict__ U_off, const int* __restrict__ U_ids,
+    const int* __restrict__ W_off, const int* __restrict__ W_ids, const int* __restrict__ Xl, const int* __restrict__ Xn,
+    const int* __restrict__ level, const double4* __restrict__ center, int thrW, int thrX,
+    LeafStream::Rec* __restrict__ recs, int2* __restrict__ near_l, float4* __restrict__ far_geo,
+    int* __restrict__ far_box) {
+    const int li = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (li >= nleaf) return;
+    const int b = leaves[li];
+    const double4 cb = center[b];
+    const int u0 = U_off[b], w0 = W_off[b], nu = U_off[b + 1] - u0, nw = W_off[b + 1] - w0;
+    const int s_own = sb[b], nself = se[b] - s_own, t0 = tb[b], t1 = te[b];
+    const int nx = thrX >= 0 && t1 - t0 <= thrX ? Xn[b] : 0;
+    const int near_off = u0 + w0 + kXCap * li, far_off = w0 + li;       // room for every list entry
+    int2* nl = near_l + near_off;
+    int n = 0, nf = 0;                                   // ranges and far boxes written
+    if (nself > 0) {
+        if (lane == 0) nl[0] = make_int2(s_own, nself);
+        n = 1;
+    }
+    int last0 = 0, last1 = -1;                           // the last joined range (the leaf's own stays alone)
+    auto put_far = [&](int k, int a, bool w) {
+        const double4 ca = center[a];
+        far_geo[far_off + k] = make_float4((float)(ca.x - cb.x), (float)(ca.y - cb.y), (float)(ca.z - cb.z),
+                                           float(w ? kAlphaInner : kAlphaOuter) * (float)ca.w);
+        far_box[far_off + k] = w ? a : -1 - a;
+    };
+    const unsigned below = (1u << lane) - 1u;
+    for (int v0 = 0; v0 < nu + nw + nx; v0 += 32) {
+        const int v = v0 + lane;
+        int a = -1, s0 = 0, s1 = 0;
+        bool far = false;
+        if (v < nu) {
+            a = U_ids[u0 + v];
+            if (a == b) a = -1;
+        } else if (v < nu + nw) {
+            a = W_ids[w0 + v - nu];
+        } else if (v < nu + nw + nx) {
+            a = Xl[(long long)b * kXCap + (v - nu - nw)];
+        }
+        if (a >= 0) {
+            s0 = sb[a];
+            s1 = se[a];
+            far = v >= nu && v < nu + nw && !(thrW >= 0 && s1 - s0 <= thrW);
+        }
+        const unsigned mf = __ballot_sync(0xffffffffu, far);
+        if (far) put_far(nf + __popc(mf & below), a, true);
+        nf += __popc(mf);
+        // ranges: an entry opens one unless it continues the entry before it
+        const bool in = a >= 0 && !far && s1 > s0;
+        const unsigned mi = __ballot_sync(0xffffffffu, in);
+        if (mi == 0) continue;
+        const int prev = 31 - __clz(mi & below);         // -1: none in this batch
+        const int pe = __shfl_sync(0xffffffffu, s1, prev < 0 ? 0 : prev);
+        const bool open = in && s0 != (prev < 0 ? last1 : pe);
+        const unsigned mo = __ballot_sync(0xffffffffu, open);
+        // end of the run that starts at this lane (or, for the entries before
+        // the first opening, of the range carried over)
+        const unsigned above = lane == 31 ? 0u : ~((2u << lane) - 1u);
+        const unsigned nxt = mo & above;
+        const unsigned run = mi & (nxt ? (1u << (__ffs(nxt) - 1)) - 1u : 0xffffffffu);
+        const int end = __shfl_sync(0xffffffffu, s1, 31 - __clz(run | 1u));
+        if (open) nl[n + __popc(mo & below)] = make_int2(s0, end - s0);
+        const unsigned lead = mo ? mi & ((1u << (__ffs(mo) - 1)) - 1u) : mi;
+        const int lead_end = __shfl_sync(0xffffffffu, s1, lead ? 31 - __clz(lead) : 0);
+        if (lead && lane == 0) nl[n - 1] = make_int2(last0, lead_end - last0);
+        n += __popc(mo);
+        const int lo = mo ? 31 - __clz(mo) : 0;          // the last opening becomes the range to continue
+        const int lo0 = __shfl_sync(0xffffffffu, s0, lo);
+        if (mo) last0 = lo0;
+        last1 = __shfl_sync(0xffffffffu, s1, 31 - __clz(mi));
+        __syncwarp();                                    // nl[n - 1] may be another lane's next
+    }
+    if (level[b] >= 2) {
+        if (lane == 0) put_far(nf, b, false);
+        ++nf;
+    }
+    if (lane == 0) {
+        LeafStream::Rec r;
+        r.t0 = t0; r.t1 = t1; r.nself = nself;
+        r.near_off = near_off; r.near_n = n;
+        r.far_off = far_off; r.far_n = nf;
+        r.pad = 0;
+        r.cx = cb.x; r.cy = cb.y; r.cz = cb.z;
+        recs[li] = r;
+    }
+}
+
+static const LeafStream& leaf_stream(fmm_tree* T, int thrW, int thrX) {
+    auto& p = T->leaf_streams[{thrW, thrX}];
+    if (p) return *p;
+    cudaStream_t st = T->ctx->stream;
+    cudaStreamCaptureStatus cap;
+    PB_CUDA(cudaStreamIsCapturing(st, &cap));
+    PB_REQUIRE(cap == cudaStreamCaptureStatusNone, PB_EINVAL, "leaf lists are not built yet (first apply is captured)");
+    auto L = std::make_unique<LeafStream>();
+    const int n = T->n_tleaf;
+    L->rec.alloc(n, st);
+    L->near.alloc(T->n_u + T->n_w + (long long)kXCap * n, st);
+    L->far_geo.alloc(T->n_w + n, st);
+    L->far_box.alloc(T->n_w + n, st);
+    k_leaf_stream<<<div_up(n, 4), 128, 0, st>>>(n, T->leaf_ids.p, T->same ? T->sb.p : T->tb.p,
+                                                T->same ? T->se.p : T->te.p, T->sb.p, T->se.p, T->U_off.p, T->U_ids.p,
+                                                T->W_off.p, T->W_ids.p, T->X.p, T->X_n.p, T->level.p, T->center.p, thrW,
+                                                thrX, L->rec.p, L->near.p, L->far_geo.p, L->far_box.p);
+    PB_CHECK_LAUNCH();
+    p = std::move(L);
+    return *p;
+}
+
 // The paired leaf kernel in packed FP32: the work split of k_leaf_pair (NT targets per thread, G groups, the near field
 // in windows of the concatenated U-list sources, the leaf itself first, then
 // the far field in windows of generated equivalent points), with each window
@@ -1137,22 +1258,18 @@ __device__ __forceinline__ void put_src_x2(ulonglong2* sA, ulonglong2* sB, ulong
 // points), each with its own partial outputs, added in order by the scatter:
 // trees of a few hundred leaves fill the GPU (see leaf_split).
 template <bool DL, bool DN, int NT, int PART, int KM, bool SPLIT>
-__global__ void __launch_bounds__(128, 5) k_leaf_pair_x2(const int* __restrict__ leaves, int nleaf,
-                                                      const int* __restrict__ tb, const int* __restrict__ te,
-                                                      const int* __restrict__ sb, const int* __restrict__ se,
-                                                      const int* __restrict__ U_off, const int* __restrict__ U_ids,
-                                                      const int* __restrict__ W_off, const int* __restrict__ W_ids,
-                                                      const int* __restrict__ level,
-                                                      const double4* __restrict__ center,
+__global__ void __launch_bounds__(128, 5) k_leaf_pair_x2(const LeafStream::Rec* __restrict__ recs,
+                                                      const int2* __restrict__ near_l,
+                                                      const float4* __restrict__ far_geo,
+                                                      const int* __restrict__ far_box,
                                                       const float4* __restrict__ tpos, const float4* __restrict__ sq,
                                                       const float4* __restrict__ sm, const float* __restrict__ QuL,
                                                       const float* __restrict__ QdL, const float* __restrict__ QuY,
                                                       const float* __restrict__ QdY, const float4* __restrict__ surf,
                                                       int ne, int npad, float kappa, float* __restrict__ potL_out,
-                                                      float* __restrict__ potY_out, const int* __restrict__ Xl,
-                                                      const int* __restrict__ Xn, int thrW, int thrX,
-                                                      const float4* __restrict__ tn, float* __restrict__ dnL_out,
-                                                      float* __restrict__ dnY_out, long long part_stride) {
+                                                      float* __restrict__ potY_out, const float4* __restrict__ tn,
+                                                      float* __restrict__ dnL_out, float* __restrict__ dnY_out,
+                                                      long long part_stride) {
     constexpr int CH = 128;
     constexpr int CAP = 1024;                    // points per window (512 pairs, 32 KB)
     constexpr int CP = CAP / 2;
@@ -1160,80 +1277,34 @@ __global__ void __launch_bounds__(128, 5) k_leaf_pair_x2(const int* __restrict__
     static_assert(NR * NT * CH * 4 <= CP * 16, "reduction fits one staging array");
     static_assert(!(DL && DN), "no hypersingular kernel");
     __shared__ ulonglong2 sA[CP], sB[CP], sC[CP], sD[CP];
-    __shared__ int s_self;
-    constexpr int VC = 256;                      // near-list entries resolved per chunk
-    constexpr int FC = CH;                       // far candidates resolved per chunk
-    constexpr int kSkip = INT_MIN;               // far candidate evaluated directly instead
-    __shared__ int s_vb[VC], s_vn[VC];           // near entry: first source, sources taken (0: none)
-    __shared__ float4 s_fb[FC];                  // far candidate: centre - the leaf's centre, radius
-    __shared__ int s_fc[FC];                     // box id (W list), -1 - id (own downward) or kSkip
-    __shared__ int s_sel[CH];                    // far window: the candidates it takes
-    __shared__ int s_nb, s_fcur;
+    constexpr int VC = 256;                      // near ranges held at a time
+    constexpr int FC = CH;                       // far boxes held at a time
+    __shared__ int2 s_v[VC];                     // first source, sources
+    __shared__ float4 s_fb[FC];                  // centre - the leaf's centre, radius of the surface
+    __shared__ int s_fc[FC];                     // box (W list, upward) or -1 - box (the leaf's own downward)
     float* s_red = reinterpret_cast<float*>(sA);
-    const int li = blockIdx.x;
-    if (li >= nleaf) return;
+    const LeafStream::Rec rec = recs[blockIdx.x];
     const int sp = SPLIT ? blockIdx.y : 0, S = SPLIT ? gridDim.y : 1, wcap = SPLIT ? CAP / S : CAP;
     if (KM & 1) potL_out += sp * part_stride;
     if (KM & 2) potY_out += sp * part_stride;
     if (DN && (KM & 1)) dnL_out += sp * part_stride;
     if (DN && (KM & 2)) dnY_out += sp * part_stride;
-    const int b = leaves[li];
-    const int t0 = tb[b], t1 = te[b];
+    const int t0 = rec.t0, t1 = rec.t1, nself = rec.nself;
     const int slots = min(CH, max(4, (t1 - t0 + NT - 1) / NT));
     const int G = CH / slots;
     const int tloc = threadIdx.x % slots, g = threadIdx.x / slots;
     const bool active = g < G;
-    const int* ul = U_ids + U_off[b];
-    const int nu = U_off[b + 1] - U_off[b];
-    const int nw = W_off[b + 1] - W_off[b];
-    const int nsrcbox = nw + (level[b] >= 2 ? 1 : 0);
-    // near stream: U list, then the W boxes of at most thrW sources, then the
-    // X list when the leaf has at most thrX targets (thr < 0: none)
-    const int nxd = (thrX >= 0 && t1 - t0 <= thrX) ? Xn[b] : 0;
-    const int nvirt = nu + (thrW >= 0 ? nw : 0) + nxd;
-    const int* xl = Xl + (long long)b * kXCap;
-    const double4 cb = center[b];
+    const int nvirt = rec.near_n, nfar = rec.far_n;
     const float kl2s = -kappa * float(kLog2E);
     const f32x2 kap = x2_pack(kappa, kappa), kl2 = x2_pack(kl2s, kl2s);
-    if (threadIdx.x == 0) s_self = -1;
-    __syncthreads();
-    for (int i = threadIdx.x; i < nu; i += CH)
-        if (ul[i] == b) s_self = i;
-    __syncthreads();
-    const int selfpos = s_self;
-    const int nself = selfpos >= 0 ? se[b] - sb[b] : 0;
-    // list entries resolved in parallel into shared memory (one round of
-    // dependent loads per chunk instead of one per box in the cursor loops)
     auto load_near = [&](int v0) {
-        for (int v = v0 + threadIdx.x; v < min(nvirt, v0 + VC); v += CH) {
-            int a;
-            bool inc = true;
-            if (v < nu) {
-                a = ul[u_at(v, selfpos)];
-            } else if (thrW >= 0 && v < nu + nw) {
-                a = W_ids[W_off[b] + (v - nu)];
-                inc = se[a] - sb[a] <= thrW;
-            } else {
-                a = xl[v - nu - (thrW >= 0 ? nw : 0)];
-            }
-            s_vb[v - v0] = sb[a];
-            s_vn[v - v0] = inc ? se[a] - sb[a] : 0;
-        }
+        for (int v = threadIdx.x; v < min(nvirt - v0, VC); v += CH) s_v[v] = near_l[rec.near_off + v0 + v];
     };
     auto load_far = [&](int f0) {
-        for (int i = f0 + threadIdx.x; i < min(nsrcbox, f0 + FC); i += CH) {
-            int code = -1 - b;
-            if (i < nw) {
-                const int a = W_ids[W_off[b] + i];
-                code = (thrW < 0 || se[a] - sb[a] > thrW) ? a : kSkip;
-            }
-            if (code != kSkip) {
-                const bool isw = code >= 0;
-                const double4 ca = center[isw ? code : -1 - code];
-                s_fb[i - f0] = make_float4((float)(ca.x - cb.x), (float)(ca.y - cb.y), (float)(ca.z - cb.z),
-                                           float(isw ? kAlphaInner : kAlphaOuter) * (float)ca.w);
-            }
-            s_fc[i - f0] = code;
+        const int i = threadIdx.x;
+        if (i < min(nfar - f0, FC)) {
+            s_fb[i] = far_geo[rec.far_off + f0 + i];
+            s_fc[i] = far_box[rec.far_off + f0 + i];
         }
     };
     int vbase = 0, fbase = 0;
@@ -1271,7 +1342,7 @@ __global__ void __launch_bounds__(128, 5) k_leaf_pair_x2(const int* __restrict__
             int vi = 0, off = 0, win = 0;
             while (vi < nvirt) {
                 const bool mine = !SPLIT || win++ % S == sp;
-                const int self_left = (selfpos >= 0 && vi == 0) ? nself - off : 0;
+                const int self_left = vi == 0 ? nself - off : 0;
                 int filled = 0;
                 while (filled < wcap && vi < nvirt) {
                     if (vi >= vbase + VC) {      // next chunk of resolved entries
@@ -1280,7 +1351,8 @@ __global__ void __launch_bounds__(128, 5) k_leaf_pair_x2(const int* __restrict__
                         load_near(vbase);
                         __syncthreads();
                     }
-                    const int j0 = s_vb[vi - vbase] + off, len = s_vn[vi - vbase] - off;
+                    const int2 v = s_v[vi - vbase];
+                    const int j0 = v.x + off, len = v.y - off;
                     const int take = min(len, wcap - filled);
                     for (int e = threadIdx.x; mine && e < take; e += CH)
                         copy_src_x2<DL, KM == 3>(sA, sB, sC, sD, filled + e, sq, sm, j0 + e);
@@ -1315,57 +1387,28 @@ __global__ void __launch_bounds__(128, 5) k_leaf_pair_x2(const int* __restrict__
                 __syncthreads();
             }
         }
-        if (PART != 1 && nsrcbox > 0) {
+        if (PART != 1 && nfar > 0) {
 #pragma unroll
             for (int u = 0; u < NT; ++u) {
-                const float rx = (float)((double)xs[u] - cb.x), ry = (float)((double)ys[u] - cb.y),
-                            rz = (float)((double)zs[u] - cb.z);
+                const float rx = (float)((double)xs[u] - rec.cx), ry = (float)((double)ys[u] - rec.cy),
+                            rz = (float)((double)zs[u] - rec.cz);
                 X[u] = x2_pack(rx, rx); Y[u] = x2_pack(ry, ry); Z[u] = x2_pack(rz, rz);
             }
             const int nbw = max(1, wcap / ne);           // whole boxes per window (ne <= CAP: host)
-            int fcur = 0, win = 0;                                // next far candidate: W list, then the leaf's own
-            while (fcur < nsrcbox) {
-                if (fcur >= fbase + FC) {                // next chunk of resolved candidates
+            int win = 0;
+            for (int f = 0; f < nfar;) {
+                if (f >= fbase + FC) {                   // next chunk of far boxes
                     __syncthreads();
                     fbase += FC;
                     load_far(fbase);
                     __syncthreads();
                 }
-                // warp 0 picks the window's boxes: up to nbw candidates of this
-                // chunk that are not evaluated directly
-                if (threadIdx.x < 32) {
-                    const int lane = threadIdx.x;
-                    const int cend = min(nsrcbox, fbase + FC);
-                    int nb = 0, c = fcur;
-                    while (nb < nbw && c < cend) {
-                        const int i = c + lane;
-                        const bool ok = i < cend && s_fc[i - fbase] != kSkip;
-                        const unsigned m = __ballot_sync(0xffffffffu, ok);
-                        const int rank = __popc(m & ((1u << lane) - 1u));
-                        const int want = nbw - nb, have = __popc(m);
-                        if (ok && rank < want) s_sel[nb + rank] = i - fbase;
-                        if (have <= want) {
-                            nb += have;
-                            c = min(c + 32, cend);
-                        } else {
-                            const unsigned last = __ballot_sync(0xffffffffu, ok && rank == want - 1);
-                            c += __ffs(last);            // one past the last box taken
-                            nb += want;
-                        }
-                    }
-                    if (lane == 0) { s_nb = nb; s_fcur = c; }
-                }
-                __syncthreads();
-                const int nb = s_nb, n = nb * ne;
-                fcur = s_fcur;
-                if (SPLIT && win++ % S != sp) {
-                    __syncthreads();                     // s_nb is read before the next pick
-                    continue;
-                }
+                const int nb = min(nbw, min(nfar, fbase + FC) - f), f0 = f - fbase, n = nb * ne;
+                f += nb;
+                if (SPLIT && win++ % S != sp) continue;
                 for (int i = 0; i < nb; ++i) {
-                    const int slot = s_sel[i];
-                    const float4 bx = s_fb[slot];
-                    const int code = s_fc[slot];
+                    const float4 bx = s_fb[f0 + i];
+                    const int code = s_fc[f0 + i];
                     const bool isw = code >= 0;
                     const size_t base = (size_t)(isw ? code : -1 - code) * npad;
                     const float* QL = isw ? QuL : QdL;
@@ -1636,13 +1679,13 @@ static void launch_leaf(cudaStream_t st, fmm_tree* Tr, Work<T>& W, const Operato
             const int NT = Tr->ctx->leaf_nt ? Tr->ctx->leaf_nt : (DN ? 2 : 4);
             auto k = split > 1 ? (NT == 4 ? k_leaf_pair_x2<DL, DN, 4, 0, KM, true> : k_leaf_pair_x2<DL, DN, 2, 0, KM, true>)
                                : (NT == 4 ? k_leaf_pair_x2<DL, DN, 4, 0, KM, false> : k_leaf_pair_x2<DL, DN, 2, 0, KM, false>);
-            k<<<dim3(Tr->n_tleaf, split), 128, 0, st>>>(Tr->leaf_ids.p, Tr->n_tleaf, tb, te, Tr->sb.p, Tr->se.p, Tr->U_off.p,
-                                           Tr->U_ids.p, Tr->W_off.p, Tr->W_ids.p, Tr->level.p, Tr->center.p, tpos,
-                                           W.sq.p, W.sm.p, W.Qu.p, W.Qd.p, nullptr, nullptr,
-                                           (const float4*)O.surf_f.p, O.ne, O.npad, kappa,
-                                           YUK ? nullptr : W.pot.p, YUK ? W.pot.p : nullptr, Tr->X.p, Tr->X_n.p,
-                                           thrW, thrX, W.tn.p, YUK ? nullptr : W.dn.p, YUK ? W.dn.p : nullptr,
-                                           Tr->same ? Tr->ns : Tr->nt);
+            const LeafStream& L = leaf_stream(Tr, thrW, thrX);
+            k<<<dim3(Tr->n_tleaf, split), 128, 0, st>>>(L.rec.p, L.near.p, L.far_geo.p, L.far_box.p, tpos, W.sq.p,
+                                                        W.sm.p, W.Qu.p, W.Qd.p, nullptr, nullptr,
+                                                        (const float4*)O.surf_f.p, O.ne, O.npad, kappa,
+                                                        YUK ? nullptr : W.pot.p, YUK ? W.pot.p : nullptr, W.tn.p,
+                                                        YUK ? nullptr : W.dn.p, YUK ? W.dn.p : nullptr,
+                                                        Tr->same ? Tr->ns : Tr->nt);
             PB_CHECK_LAUNCH();
             return;
         }
@@ -2014,12 +2057,12 @@ static void launch_leaf_pair(cudaStream_t st, fmm_tree* Tr, Work<T>& WL, Work<T>
             const int NT = nt_opt ? nt_opt : (DN ? 2 : 4);
             auto k = split > 1 ? (NT == 4 ? k_leaf_pair_x2<DL, DN, 4, PART, 3, true> : k_leaf_pair_x2<DL, DN, 2, PART, 3, true>)
                                : (NT == 4 ? k_leaf_pair_x2<DL, DN, 4, PART, 3, false> : k_leaf_pair_x2<DL, DN, 2, PART, 3, false>);
-            k<<<dim3(Tr->n_tleaf, split), 128, 0, st>>>(Tr->leaf_ids.p, Tr->n_tleaf, tb, te, Tr->sb.p, Tr->se.p, Tr->U_off.p,
-                                           Tr->U_ids.p, Tr->W_off.p, Tr->W_ids.p, Tr->level.p, Tr->center.p, tpos,
-                                           WL.sq.p, WL.sm.p, WL.Qu.p, WL.Qd.p, WY.Qu.p, WY.Qd.p,
-                                           (const float4*)O.surf_f.p, O.ne, O.npad, kappa, WL.pot.p, WY.pot.p,
-                                           Tr->X.p, Tr->X_n.p, thrW, thrX, WL.tn.p, WL.dn.p, WY.dn.p,
-                                           Tr->same ? Tr->ns : Tr->nt);
+            const LeafStream& L = leaf_stream(Tr, thrW, thrX);
+            k<<<dim3(Tr->n_tleaf, split), 128, 0, st>>>(L.rec.p, L.near.p, L.far_geo.p, L.far_box.p, tpos, WL.sq.p,
+                                                        WL.sm.p, WL.Qu.p, WL.Qd.p, WY.Qu.p, WY.Qd.p,
+                                                        (const float4*)O.surf_f.p, O.ne, O.npad, kappa, WL.pot.p,
+                                                        WY.pot.p, WL.tn.p, WL.dn.p, WY.dn.p,
+                                                        Tr->same ? Tr->ns : Tr->nt);
             PB_CHECK_LAUNCH();
             return;
         }

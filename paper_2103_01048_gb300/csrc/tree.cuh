@@ -53,6 +53,22 @@ struct PCPairs {
     int nitems = 0;
 };
 
+// Source streams of the packed leaf kernel (built in fmm.cu)
+struct LeafStream {
+    struct Rec {
+        int t0, t1;                // targets
+        int nself;                 // the leaf's own sources (its first near range; 0: no such range)
+        int near_off, near_n;      // near: (first source, count)
+        int far_off, far_n;
+        int pad;
+        double cx, cy, cz;         // centre of the leaf
+    };
+    DBuf<Rec> rec;
+    DBuf<int2> near;
+    DBuf<float4> far_geo;          // centre - the leaf's centre, radius of the surface
+    DBuf<int> far_box;             // box (upward densities) or -1 - box (downward)
+};
+
 }  // namespace pbfmm
 
 struct fmm_tree {
@@ -104,6 +120,9 @@ struct fmm_tree {
     int n_xfar = 0;
     pbfmm::DBuf<int4> c2e_items_xfar;
     int n_c2e_xfar = 0;
+
+    // by (W threshold, X threshold): at most four combinations of options per expansion order
+    std::map<std::pair<int, int>, std::unique_ptr<pbfmm::LeafStream>> leaf_streams;
 
     std::map<std::tuple<int, double, int, int>, std::shared_ptr<pbfmm::Operators>> ops;
 };

@@ -74,3 +74,43 @@ def test_one_leaf_direct(n, layer):
     for k, v in got.items():
         ref = sum(t.sum(1) for t in terms[k.lstrip("1")]) * c4
         assert np.all(np.abs(v - ref) <= tol * absum[k.lstrip("1")] + 1e-30), k
+
+
+@pytest.mark.parametrize("mode", [0, 1, 2, 3])
+@pytest.mark.parametrize("separate", [False, True])
+def test_long_lists(mode, separate):
+    """Clustered points and small leaves: lists of more than 32 entries, ranges
+    that join across them, targets without sources; every direct-list mode
+    against the direct sum, the scalar kernel beside it.  1e-5, the bound
+    of the FMM applies (here p = 8)."""
+    import paper_2103_01048_gb300 as pb
+    from oracle.kernels import LAPLACE, YUKAWA, direct_sum, rel_l2
+    rng = np.random.default_rng(17)
+    pts = lambda a, b: np.concatenate([rng.normal(0, 0.02, (a, 3)), rng.uniform(-1, 1, (b, 3))]).astype(np.float32)
+    x = pts(2500, 1500)
+    t = pts(500, 2500) if separate else None
+    n = len(x if t is None else t)
+    q, d = (rng.uniform(-1, 1, len(x)).astype(np.float32) for _ in range(2))
+    nrm = rng.standard_normal((len(x), 3))
+    nrm = (nrm / np.linalg.norm(nrm, axis=1, keepdims=True)).astype(np.float32)
+    dev = lambda a: torch.from_numpy(a).cuda()
+    ctx = pb.pb_create(0, None)
+    try:
+        pb.pb_set_option(ctx, pb.PB_OPT_LIST_DIRECT, mode)
+        tree = pb.fmm_tree_build(ctx, dev(x), 12, None if t is None else dev(t))
+        off, _ = pb.fmm_tree_export(ctx, tree)["U"]
+        assert np.diff(off).max() > 32
+        got = []
+        for packed in (1, 0):
+            pb.pb_set_option(ctx, pb.PB_OPT_LEAF_PACKED, packed)
+            oL, oY = torch.zeros(n, device="cuda"), torch.zeros(n, device="cuda")
+            pb.fmm_apply_pair(ctx, tree, 0.5, 8, oL, oY, q_lap=dev(q), q_yuk=dev(q), dip=dev(d), src_n=dev(nrm))
+            torch.cuda.synchronize()
+            got.append((oL.cpu().numpy(), oY.cpu().numpy()))
+        pb.fmm_tree_destroy(tree)
+    finally:
+        pb.pb_destroy(ctx)
+    ref = [direct_sum(k, kap, x, q=q, dip=d, src_n=nrm, tgt=t) for k, kap in ((LAPLACE, 0.0), (YUKAWA, 0.5))]
+    for o in got:
+        for v, r in zip(o, ref):
+            assert rel_l2(v, r) < 1e-5
