@@ -169,15 +169,25 @@ __global__ void k_gather_tn(long long n, const int* __restrict__ perm, const In*
     tn[k] = {(T)nrm[3 * i], (T)nrm[3 * i + 1], (T)nrm[3 * i + 2], T(0)};
 }
 
-// out[perm[k]] = sum of the nsplit partial results v[s][k], in order
+// out[y][perm[k]] = sum of the nsplit partial results v[y][s][k], in order,
+// for the nout outputs of an apply
 template <typename T, typename Out>
-__global__ void k_scatter(long long n, const int* __restrict__ perm, const T* __restrict__ v, Out* __restrict__ out,
-                          int nsplit = 1) {
+struct Scatter {
+    const T* v[4];
+    Out* out[4];
+};
+template <typename T, typename Out>
+__global__ void k_scatter(long long n, const int* __restrict__ perm, Scatter<T, Out> S, int nout, int nsplit) {
     long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (k >= n) return;
-    T a = v[k];
-    for (int s = 1; s < nsplit; ++s) a += v[s * n + k];
-    out[perm[k]] = (Out)a;
+    const long long i = perm[k];
+#pragma unroll
+    for (int y = 0; y < 4; ++y) {
+        if (y >= nout) break;
+        T a = S.v[y][k];
+        for (int s = 1; s < nsplit; ++s) a += S.v[y][s * n + k];
+        S.out[y][i] = (Out)a;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1591,8 +1601,11 @@ __global__ void __launch_bounds__(128) k_p2check_pair_x2(int nbox, const int* __
 // ---------------------------------------------------------------------------
 template <typename T>
 struct Work {
+    struct Rows { T* p = nullptr; };
     DBuf<typename V4<T>::type> sq, sm, tn;
-    DBuf<T> Qu, Qd, chk, pot, dn;
+    DBuf<T> q;            // Qu, Qd (of the paired apply's second kernel as well): one buffer, zeroed at once
+    Rows Qu, Qd;
+    DBuf<T> chk, pot, dn;
     DBuf<T> tmp;          // FP32 path: intermediate of the factored check -> equivalent solves, M2L source rows
 };
 
@@ -1903,17 +1916,20 @@ static void far_pair_m2l(fmm_tree* Tr, const Operators& OL, const Operators& OY,
     far_m2l(Tr, OY, WY);
 }
 
-// equivalent densities and check potentials of one kernel
+// equivalent densities (zeroed) and check potentials of one kernel or two
+// (the check potentials are written before they are read)
 template <typename T>
-static void alloc_far(Work<T>& W, size_t nbox, int npad, cudaStream_t st) {
-    const size_t nbox_npad = nbox * npad;
-    W.Qu.alloc(nbox_npad, st);
-    W.Qd.alloc(nbox_npad, st);
-    W.chk.alloc(nbox_npad, st);
-    W.Qu.zero(st);
-    W.Qd.zero(st);
-    W.chk.zero(st);
-    if (std::is_same<T, float>::value) W.tmp.alloc(nbox_npad + nbox, st);     // + a scale per box
+static void alloc_far(Work<T>& W, Work<T>* W2, size_t nbox, int npad, cudaStream_t st) {
+    const size_t n = nbox * npad;
+    W.q.alloc(n * (W2 ? 4 : 2), st);
+    W.q.zero(st);
+    Work<T>* ws[2] = {&W, W2};
+    for (int k = 0; k < 2 && ws[k]; ++k) {
+        ws[k]->Qu.p = W.q.p + 2 * k * n;
+        ws[k]->Qd.p = ws[k]->Qu.p + n;
+        ws[k]->chk.alloc(n, st);
+        if (std::is_same<T, float>::value) ws[k]->tmp.alloc(n + nbox, st);     // + a scale per box
+    }
 }
 
 template <typename T, typename In, bool YUK>
@@ -1933,7 +1949,7 @@ static void apply_t(fmm_tree* Tr, const Operators& O, double kappa_d, const In* 
     Work<T> W;
     W.sq.alloc(ns, st);
     if (DL) W.sm.alloc(ns, st);
-    alloc_far(W, Tr->nbox, O.npad, st);
+    alloc_far<T>(W, nullptr, Tr->nbox, O.npad, st);
     W.pot.alloc(nt * split, st);
     if (DN) { W.dn.alloc(nt * split, st); W.tn.alloc(nt, st); }
     pb_ctx* ctx = Tr->ctx;
@@ -1979,10 +1995,9 @@ static void apply_t(fmm_tree* Tr, const Operators& O, double kappa_d, const In* 
     else launch_leaf<T, YUK, false, false>(st, Tr, W, O, kappa, thrW, thrX, split);
     ph.reset(); ph = std::make_unique<PhaseTimer>(ctx, PB_PH_SCATTER);
     const int* pt = Tr->same ? Tr->perm_s.p : Tr->perm_t.p;
-    k_scatter<T, In><<<div_up(nt, 256), 256, 0, st>>>(nt, pt, W.pot.p, out, split);
+    const Scatter<T, In> sc{{W.pot.p, W.dn.p}, {out, out_dn}};
+    k_scatter<T, In><<<div_up(nt, 256), 256, 0, st>>>(nt, pt, sc, DN ? 2 : 1, split);
     PB_CHECK_LAUNCH();
-    if (DN) k_scatter<T, In><<<div_up(nt, 256), 256, 0, st>>>(nt, pt, W.dn.p, out_dn, split);
-    if (DN) PB_CHECK_LAUNCH();
     ph.reset();
 }
 
@@ -2105,8 +2120,7 @@ static void apply_pair_t(fmm_tree* Tr, const Operators& OL, const Operators& OY,
     Work<T> WL, WY;
     WL.sq.alloc(ns, st);
     WL.sm.alloc(ns, st);
-    alloc_far(WL, Tr->nbox, OL.npad, st);
-    alloc_far(WY, Tr->nbox, OY.npad, st);
+    alloc_far(WL, &WY, Tr->nbox, OL.npad, st);
     const int split = leaf_split(Tr, std::is_same<T, double>::value);
     WL.pot.alloc(nt * split, st);
     WY.pot.alloc(nt * split, st);
@@ -2172,16 +2186,9 @@ static void apply_pair_t(fmm_tree* Tr, const Operators& OL, const Operators& OY,
     }
     ph.reset(); ph = std::make_unique<PhaseTimer>(ctx, PB_PH_SCATTER);
     const int* pt = Tr->same ? Tr->perm_s.p : Tr->perm_t.p;
-    k_scatter<T, In><<<div_up(nt, 256), 256, 0, st>>>(nt, pt, WL.pot.p, outL, split);
+    const Scatter<T, In> sc{{WL.pot.p, WY.pot.p, WL.dn.p, WY.dn.p}, {outL, outY, dnL, dnY}};
+    k_scatter<T, In><<<div_up(nt, 256), 256, 0, st>>>(nt, pt, sc, DN ? 4 : 2, split);
     PB_CHECK_LAUNCH();
-    k_scatter<T, In><<<div_up(nt, 256), 256, 0, st>>>(nt, pt, WY.pot.p, outY, split);
-    PB_CHECK_LAUNCH();
-    if (DN) {
-        k_scatter<T, In><<<div_up(nt, 256), 256, 0, st>>>(nt, pt, WL.dn.p, dnL, split);
-        PB_CHECK_LAUNCH();
-        k_scatter<T, In><<<div_up(nt, 256), 256, 0, st>>>(nt, pt, WY.dn.p, dnY, split);
-        PB_CHECK_LAUNCH();
-    }
     ph.reset();
 }
 

@@ -336,6 +336,8 @@ struct TcSets {
     const float* X[2];
     float* Y[2];
     long long wait_limit;    // cycles a role waits on a barrier before giving up (set at launch)
+    int store;               // 1: every target row has one product and one inner part: store, do not add
+    int sub, chunk;          // an item's pairs are cut into `sub` pieces of `chunk` pairs, one CTA (and part) each (0: by the launch)
 };
 
 template <int NPAD>
@@ -367,7 +369,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_m2l_tc(const int4* __restrict
     TcSmem<kTcStages>* S = (TcSmem<kTcStages>*)(sA + kTcStages * 2 * A_SPLIT);
     volatile int* failed = &S->failed;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int4 it = items[blockIdx.x];
+    int4 it = items[blockIdx.x / sets.sub];
+    const int skip = (blockIdx.x % sets.sub) * sets.chunk;
+    it.x += skip;
+    it.y = min(it.y - skip, sets.chunk);
+    if (it.y <= 0) return;
     const int part = blockIdx.y;                     // operator part: rows half, inner columns kpart
     const int half = part / KS, kpart = part % KS;
     const int first = it.x, npairs = it.y;
@@ -483,7 +489,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_m2l_tc(const int4* __restrict
                     const int rr = j * 8 + (lane >> 2), cc = (lane & 3) * 4;
                     const float4 x = *(const float4*)&buf[rr][cc];
                     const int tr = __shfl_sync(0xffffffffu, t, rr);
-                    if (tr >= 0) red_add_v4(Qd + (size_t)tr * NPAD + half * NH + c0 + cc, x.x, x.y, x.z, x.w);
+                    float* y = Qd + (size_t)tr * NPAD + half * NH + c0 + cc;
+                    if (tr < 0) continue;
+                    if (KS == 1 && sets.store) *(float4*)y = x;
+                    else red_add_v4(y, x.x, x.y, x.z, x.w);
                 }
                 __syncwarp();
             }
@@ -560,13 +569,34 @@ static void smem_optin(F* kernel, size_t bytes, bool* done) {
     }
 }
 
+static int tc_sm_count() {
+    static std::atomic<int> n{0};
+    if (n.load() == 0) {
+        int dev = 0, v = 0;
+        PB_CUDA(cudaGetDevice(&dev));
+        PB_CUDA(cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev));
+        n.store(v);
+    }
+    return n.load();
+}
+
 template <int NPAD>
 static void launch_tc_items(const int4* items, int nitems, const int* tgt, const int* src, const TcSets& sets,
                             int nsets, int* err, cudaStream_t st) {
     if (nitems <= 0) return;
-    dim3 grid(nitems, TcCfg<NPAD>::NS * TcCfg<NPAD>::KS, nsets);
     TcSets s2 = sets;
     s2.wait_limit = g_wait_limit.load();
+    if (s2.sub == 0) {
+        // pieces of an item: whole (512 pairs, four row tiles, 17 to 21 us, mostly
+        // latency), or down to one row tile (9 us) where SMs would else have no CTA
+        int sub = 1;
+        while (sub < kTcSmallItemPairs / kTcRows &&
+               (long long)nitems * sub * TcCfg<NPAD>::NS * TcCfg<NPAD>::KS * nsets < tc_sm_count())
+            sub *= 2;
+        s2.sub = sub;
+        s2.chunk = kTcSmallItemPairs / sub;
+    }
+    dim3 grid(nitems * s2.sub, TcCfg<NPAD>::NS * TcCfg<NPAD>::KS, nsets);
     static bool done[64] = {false};
     const size_t sm = tc_smem_bytes<NPAD>();
     smem_optin(k_m2l_tc<NPAD>, sm, done);
@@ -617,10 +647,10 @@ bool pc_tc_launch(const fmm_tree* T, const Operators& O, int child_level, bool u
 }
 
 // Check -> equivalent solve Y = W2 (W1 X) at the upward (sleaf) or downward
-// (X-list) boxes on the tensor cores: two passes through `tmp`, which is
-// zeroed first (every row of a pass receives exactly one product, so the
-// result does not depend on the order of the reductions). Y rows of those
-// boxes must be zero on entry. One operator set, or two (O2, X2, Y2, tmp2)
+// (X-list) boxes on the tensor cores: two passes through `tmp`.  Every row of
+// a pass receives exactly one product; up to p = 6 it is stored, at p = 8 and
+// 10 the operator's inner parts add into tmp (zeroed first) and into Y, whose
+// rows of those boxes must be zero on entry. One operator set, or two (O2, X2, Y2, tmp2)
 // in the same launches. False when the tensor-core path does not apply.
 bool c2e_tc_ok(const Operators& O) { return tc_ok(O) && O.uc2ue_w1_tc.p; }
 
@@ -666,12 +696,16 @@ bool c2e_tc_launch2(const fmm_tree* T, const Operators& O, const Operators* O2, 
     const int* ids = up ? T->sleaf_ids.p : (far ? T->xfar_ids.p : T->xbox_ids.p);
     auto w1 = [&](const Operators& o) { return up ? o.uc2ue_w1_tc.p : o.dc2de_w1_tc.p; };
     auto w2 = [&](const Operators& o) { return up ? o.uc2ue_w2_tc.p : o.dc2de_w2_tc.p; };
-    const size_t bytes = (size_t)T->nbox * O.npad * sizeof(float);
-    PB_CUDA(cudaMemsetAsync(tmp, 0, bytes, st));
-    if (O2) PB_CUDA(cudaMemsetAsync(tmp2, 0, bytes, st));
+    int parts = 0, ks = 0;
+    tc_split(O.npad, parts, ks);
+    if (ks > 1) {                     // the inner parts add up
+        const size_t bytes = (size_t)T->nbox * O.npad * sizeof(float);
+        PB_CUDA(cudaMemsetAsync(tmp, 0, bytes, st));
+        if (O2) PB_CUDA(cudaMemsetAsync(tmp2, 0, bytes, st));
+    }
     const int ns = O2 ? 2 : 1;
-    TcSets p1{{w1(O), O2 ? w1(*O2) : nullptr}, {X, X2}, {tmp, tmp2}};
-    TcSets p2{{w2(O), O2 ? w2(*O2) : nullptr}, {tmp, tmp2}, {Y, Y2}};
+    TcSets p1{{w1(O), O2 ? w1(*O2) : nullptr}, {X, X2}, {tmp, tmp2}, 0, 1};
+    TcSets p2{{w2(O), O2 ? w2(*O2) : nullptr}, {tmp, tmp2}, {Y, Y2}, 0, 1};
     if (!tc_dispatch(O.npad, items, nitems, ids, ids, p1, ns, err, st)) return false;
     return tc_dispatch(O.npad, items, nitems, ids, ids, p2, ns, err, st);
 }
@@ -737,7 +771,7 @@ extern "C" int pbfmm_selftest_m2l_tc(int nrows, int npad, const float* Q, const 
             ditems.alloc(items.size(), st);
             PB_CUDA(cudaMemcpyAsync(ids.p, id.data(), nrows * 4, cudaMemcpyHostToDevice, st));
             PB_CUDA(cudaMemcpyAsync(ditems.p, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
-            TcSets sets{{packed.p, nullptr}, {q.p, nullptr}, {d.p, nullptr}, 0};
+            TcSets sets{{packed.p, nullptr}, {q.p, nullptr}, {d.p, nullptr}, 0, 0, 1, kTcItemPairs};
             if (!tc_dispatch(npad, ditems.p, (int)items.size(), ids.p, ids.p, sets, 1, e.p, st)) return PB_EINVAL;
             PB_CUDA(cudaStreamSynchronize(st));
         }
