@@ -30,6 +30,7 @@ bool c2e_tc_launch2(const fmm_tree* T, const Operators& O, const Operators* O2, 
 // X-list boxes that keep P2L when small leaves sum their X lists directly
 bool c2e_tc_ok(const Operators& O);
 void build_xbox_far(fmm_tree* T, int thrX);
+void build_m2l_schedule(fmm_tree* T);
 
 constexpr double kInv4PiD = 0.07957747154594767;
 constexpr double kLog2E = 1.4426950408889634;     // log2(e)
@@ -1824,6 +1825,7 @@ static void far_m2l(fmm_tree* Tr, const Operators& O, Work<T>& W) {
                             W.Qd.p);
         tc_done = true;
     }
+    if (!tc_done && Tr->n_v > 0) build_m2l_schedule(Tr);
     if (!tc_done && Tr->m2l.ntile > 0) {
         GemmArgs ga = tree_gemm_args<T>(Tr);
         ga.mode = G_M2L;

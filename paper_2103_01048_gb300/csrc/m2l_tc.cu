@@ -111,7 +111,7 @@ void pack_box_ops_tc(Operators& O, cudaStream_t st) {
 // V-list pairs grouped by (level, offset)
 // ---------------------------------------------------------------------------
 __global__ void k_pairs_emit(int nbox, const int* V, const int* V_n, const int* V_off, const int4* anchor,
-                             int* key, int* tgt, int* src) {
+                             int* key, int* tgt, int* src, int* idx) {
     int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= nbox) return;
     int4 ab = anchor[b];
@@ -125,7 +125,16 @@ __global__ void k_pairs_emit(int nbox, const int* V, const int* V_n, const int* 
         key[e] = (((b / kM2LSegBoxes) * 64 + slot) * 32 + ab.w) * 8 + sign;   // segment, |offset|, level (< 22), signs
         tgt[e] = b;
         src[e] = s;
+        idx[e] = e;
     }
+}
+
+// first pair and key of every run of equal keys
+__global__ void k_pair_runs(int n, const int* key, int cap, int2* runs, int* count) {
+    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n || (i > 0 && key[i] == key[i - 1])) return;
+    const int k = atomicAdd(count, 1);
+    if (k < cap) runs[k] = make_int2(i, key[i]);
 }
 
 __global__ void k_pairs_gather(int n, const int* idx, const int* key, const int* t, const int* s, int* tgt, int* src,
@@ -157,12 +166,10 @@ void build_m2l_pairs(fmm_tree* T) {
         cub::DeviceScan::ExclusiveSum(t.p, tmp, T->V_n.p, voff.p, nb, st);
     }
     key.alloc(np, st); tgt.alloc(np, st); src.alloc(np, st);
-    k_pairs_emit<<<div_up(nb, 128), 128, 0, st>>>(nb, T->V.p, T->V_n.p, voff.p, T->anchor.p, key.p, tgt.p, src.p);
-    PB_CHECK_LAUNCH();
     idx.alloc(np, st); key_s.alloc(np, st); idx_s.alloc(np, st);
-    std::vector<int> hidx(np);
-    for (long long i = 0; i < np; ++i) hidx[i] = (int)i;
-    PB_CUDA(cudaMemcpyAsync(idx.p, hidx.data(), np * sizeof(int), cudaMemcpyHostToDevice, st));
+    k_pairs_emit<<<div_up(nb, 128), 128, 0, st>>>(nb, T->V.p, T->V_n.p, voff.p, T->anchor.p, key.p, tgt.p, src.p,
+                                                  idx.p);
+    PB_CHECK_LAUNCH();
     // stable: each group keeps the box order
     int bits = 14;
     while ((nb - 1) / kM2LSegBoxes >> (bits - 14)) ++bits;
@@ -173,33 +180,49 @@ void build_m2l_pairs(fmm_tree* T) {
     k_pairs_gather<<<div_up(np, 256), 256, 0, st>>>((int)np, idx_s.p, key_s.p, tgt.p, src.p, P.tgt.p, P.src.p,
                                                      P.srcx.p);
     PB_CHECK_LAUNCH();
-    std::vector<int> hk(np);
-    PB_CUDA(cudaMemcpyAsync(hk.data(), key_s.p, np * sizeof(int), cudaMemcpyDeviceToHost, st));
-    PB_CUDA(cudaStreamSynchronize(st));
+    // the runs of equal keys: (first pair, key), in any order, then sorted
+    DBuf<int2> druns;
+    DBuf<int> dn;
+    int cap = 8192, nrun = 0;
+    std::vector<int2> runs;
+    for (;;) {
+        druns.alloc(cap, st);
+        dn.alloc(1, st);
+        dn.zero(st);
+        k_pair_runs<<<div_up(np, 256), 256, 0, st>>>((int)np, key_s.p, cap, druns.p, dn.p);
+        PB_CHECK_LAUNCH();
+        runs.resize(cap);
+        PB_CUDA(cudaMemcpyAsync(&nrun, dn.p, sizeof(int), cudaMemcpyDeviceToHost, st));
+        PB_CUDA(cudaMemcpyAsync(runs.data(), druns.p, cap * sizeof(int2), cudaMemcpyDeviceToHost, st));
+        PB_CUDA(cudaStreamSynchronize(st));
+        if (nrun <= cap) break;
+        cap = nrun;
+    }
+    runs.resize(nrun);
+    std::sort(runs.begin(), runs.end(), [](const int2& x, const int2& y) { return x.x < y.x; });
+    runs.push_back(make_int2((int)np, -1));
     std::vector<int4> even, odd, items32;
     std::vector<int> seg_even, seg_odd;
     auto cut = [](std::vector<int4>& v, long long a, long long b, int step, int z) {
         for (; a < b; a += step) v.push_back(make_int4((int)a, (int)std::min<long long>(step, b - a), z, 0));
     };
-    for (long long i = 0; i < np;) {
+    for (int i = 0; i < nrun;) {
         // one (segment, |offset|, level): the runs of its signs, then the whole group
-        if (i == 0 || hk[i] >> 14 != hk[i - 1] >> 14) {
+        const int k = runs[i].y;
+        if (i == 0 || k >> 14 != runs[i - 1].y >> 14) {
             seg_even.push_back((int)even.size());
             seg_odd.push_back((int)odd.size());
         }
-        long long j = i;
-        while (j < np && hk[j] >> 3 == hk[i] >> 3) {
-            long long k = j;
-            while (k < np && hk[k] == hk[j]) ++k;
-            const int slot = (hk[j] >> 8) & 63, lev = (hk[j] >> 3) & 31, sg = hk[j] & 7;
+        int j = i;
+        for (; j < nrun && runs[j].y >> 3 == k >> 3; ++j) {
+            const int kj = runs[j].y, slot = (kj >> 8) & 63, lev = (kj >> 3) & 31, sg = kj & 7;
             const int o[3] = {slot >> 4, (slot >> 2) & 3, slot & 3};
             const int off = ((sg & 4 ? -o[0] : o[0]) + 3) * 49 + ((sg & 2 ? -o[1] : o[1]) + 3) * 7 +
                             ((sg & 1 ? -o[2] : o[2]) + 3);
-            cut(odd, j, k, 128, off * 32 + lev);
-            cut(items32, j, k, 32, lev * kNumOffsets + off);
-            j = k;
+            cut(odd, runs[j].x, runs[j + 1].x, 128, off * 32 + lev);
+            cut(items32, runs[j].x, runs[j + 1].x, 32, lev * kNumOffsets + off);
         }
-        cut(even, i, j, 128, (hk[i] >> 3) & 2047);
+        cut(even, runs[i].x, runs[j].x, 128, (k >> 3) & 2047);
         i = j;
     }
     P.nseg = (int)seg_even.size();

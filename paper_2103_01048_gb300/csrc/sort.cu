@@ -97,6 +97,51 @@ __global__ void k_scan_add(int* __restrict__ out, long long m, const int* __rest
     if (i < m) out[i] += totals[i / kRsTile];
 }
 
+// the whole scan by one block of 1024 threads (few tiles: one launch for three)
+__global__ void __launch_bounds__(1024) k_scan_block(const int* __restrict__ in, int m, int* __restrict__ out) {
+    __shared__ int warp_tot[32];
+    __shared__ int carry;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) carry = 0;
+    __syncthreads();
+    for (int b0 = 0; b0 < m; b0 += 8192) {
+        const int base = b0 + threadIdx.x * 8;
+        int v[8], s = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            v[k] = base + k < m ? in[base + k] : 0;
+            s += v[k];
+        }
+        int incl = s;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        if (lane == 31) warp_tot[warp] = incl;
+        __syncthreads();
+        if (warp == 0) {
+            const int w = warp_tot[lane];
+            int wi = w;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int t = __shfl_up_sync(0xffffffffu, wi, o);
+                if (lane >= o) wi += t;
+            }
+            warp_tot[lane] = wi - w;
+        }
+        __syncthreads();
+        const int c0 = carry;
+        int run = c0 + warp_tot[warp] + incl - s;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            if (base + k < m) out[base + k] = run;
+            run += v[k];
+        }
+        __syncthreads();                       // every thread has read the carry
+        if (threadIdx.x == 1023) carry = run;
+        __syncthreads();
+    }
+}
+
 template <typename K, typename V>
 __global__ void __launch_bounds__(kRsThreads) k_rs_scatter(const K* __restrict__ kin, const V* __restrict__ vin,
                                                            long long n, int shift, int ntiles,
@@ -207,12 +252,17 @@ static void radix_sort_pairs_t(const K* keys_in, const V* vals_in, K* keys_out, 
         const int shift = 8 * p;
         k_rs_hist<K><<<ntiles, kRsThreads, 0, st>>>(ks, n, shift, ntiles, counts.p);
         PB_CHECK_LAUNCH();
-        k_scan_chunks<<<nchunk, kRsThreads, 0, st>>>(counts.p, m, offsets.p, totals.p);
-        PB_CHECK_LAUNCH();
-        k_scan_totals<<<1, kRsThreads, 0, st>>>(totals.p, nchunk);
-        PB_CHECK_LAUNCH();
-        k_scan_add<<<div_up(m, 256), 256, 0, st>>>(offsets.p, m, totals.p);
-        PB_CHECK_LAUNCH();
+        if (m <= 65536) {                      // 256 tiles, 524,288 pairs: 8 rounds of one block
+            k_scan_block<<<1, 1024, 0, st>>>(counts.p, (int)m, offsets.p);
+            PB_CHECK_LAUNCH();
+        } else {
+            k_scan_chunks<<<nchunk, kRsThreads, 0, st>>>(counts.p, m, offsets.p, totals.p);
+            PB_CHECK_LAUNCH();
+            k_scan_totals<<<1, kRsThreads, 0, st>>>(totals.p, nchunk);
+            PB_CHECK_LAUNCH();
+            k_scan_add<<<div_up(m, 256), 256, 0, st>>>(offsets.p, m, totals.p);
+            PB_CHECK_LAUNCH();
+        }
         k_rs_scatter<K, V><<<ntiles, kRsThreads, 0, st>>>(ks, vs, n, shift, ntiles, offsets.p, kd, vd);
         PB_CHECK_LAUNCH();
         ks = kd;

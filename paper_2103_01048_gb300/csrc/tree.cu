@@ -379,15 +379,13 @@ __global__ void k_compact_scatter(int n, const int* flag, const int* pos, int* o
 static void exclusive_scan(const int* in, int* out, int n, cudaStream_t st);
 template <typename T> static T read1(const T* d, cudaStream_t st);
 
-// compaction helper: indices i with flag[i] != 0, in order
-static int compact(const int* flag, int n, DBuf<int>& out, cudaStream_t st) {
-    DBuf<int> pos;
-    pos.alloc(n + 1, st);
+// compaction helper: indices i with flag[i] != 0, in order; flag and pos hold
+// n + 1 entries, pos[n] receives the count
+static void compact(const int* flag, int n, int* pos, DBuf<int>& out, cudaStream_t st) {
     out.alloc(std::max(n, 1), st);
-    exclusive_scan(flag, pos.p, n, st);
-    k_compact_scatter<<<div_up(n, 256), 256, 0, st>>>(n, flag, pos.p, out.p);
+    exclusive_scan(flag, pos, n + 1, st);
+    k_compact_scatter<<<div_up(n, 256), 256, 0, st>>>(n, flag, pos, out.p);
     PB_CHECK_LAUNCH();
-    return read1(pos.p + n - 1, st) + read1(flag + n - 1, st);
 }
 
 static void exclusive_scan(const int* in, int* out, int n, cudaStream_t st) {
@@ -405,6 +403,55 @@ static T read1(const T* d, cudaStream_t st) {
     PB_CUDA(cudaMemcpyAsync(&h, d, sizeof(T), cudaMemcpyDeviceToHost, st));
     PB_CUDA(cudaStreamSynchronize(st));
     return h;
+}
+
+// M2L tile schedule: boxes with a non-empty V list, per level, tiles of
+// kM2LTile.  Only the fixed-order M2L of PB_OPT_DETERMINISTIC uses it: built
+// at its first apply on the tree (0.4 of the 2.3 ms of a 120,000-point build).
+void build_m2l_schedule(fmm_tree* T) {
+    if (T->m2l_built) return;
+    cudaStream_t st = T->ctx->stream;
+    const int nb = T->nbox;
+    std::vector<int> vn(nb);
+    PB_CUDA(cudaMemcpyAsync(vn.data(), T->V_n.p, nb * sizeof(int), cudaMemcpyDeviceToHost, st));
+    PB_CUDA(cudaStreamSynchronize(st));
+    std::vector<int> tiles, tlev;
+    for (int l = 0; l < T->nlev; ++l) {
+        std::vector<int> cur;
+        for (int b = T->lvl_off[l]; b < T->lvl_off[l + 1]; ++b)
+            if (vn[b] > 0) cur.push_back(b);
+        for (size_t i = 0; i < cur.size(); i += kM2LTile) {
+            for (int c = 0; c < kM2LTile; ++c)
+                tiles.push_back(i + c < cur.size() ? cur[i + c] : -1);
+            tlev.push_back(l);
+        }
+    }
+    M2LSchedule& S = T->m2l;
+    S.ntile = (int)tlev.size();
+    S.tile_level_h = tlev;
+    S.npairs = T->n_v;
+    if (S.ntile > 0) {
+        S.tile_box.alloc(tiles.size(), st);
+        S.tile_level.alloc(S.ntile, st);
+        PB_CUDA(cudaMemcpyAsync(S.tile_box.p, tiles.data(), tiles.size() * sizeof(int), cudaMemcpyHostToDevice, st));
+        PB_CUDA(cudaMemcpyAsync(S.tile_level.p, tlev.data(), tlev.size() * sizeof(int), cudaMemcpyHostToDevice, st));
+        DBuf<int> cnt;
+        cnt.alloc(S.ntile + 1, st);
+        cnt.zero(st);
+        S.entry_off.alloc(S.ntile + 1, st);
+        k_m2l_schedule<<<S.ntile, 128, 0, st>>>(S.ntile, S.tile_box.p, T->anchor.p, T->V.p, T->V_n.p, nullptr,
+                                                cnt.p, nullptr, nullptr, 0);
+        PB_CHECK_LAUNCH();
+        exclusive_scan(cnt.p, S.entry_off.p, S.ntile + 1, st);
+        S.nentry = read1(S.entry_off.p + S.ntile, st);
+        S.entry_offset_idx.alloc(std::max<long long>(S.nentry, 1), st);
+        S.entry_src.alloc(std::max<long long>(S.nentry, 1) * kM2LTile, st);
+        k_m2l_schedule<<<S.ntile, 128, 0, st>>>(S.ntile, S.tile_box.p, T->anchor.p, T->V.p, T->V_n.p,
+                                                S.entry_off.p, nullptr, S.entry_offset_idx.p, S.entry_src.p, 1);
+        PB_CHECK_LAUNCH();
+    }
+    PB_CUDA(cudaStreamSynchronize(st));
+    T->m2l_built = true;
 }
 
 void build_m2l_pairs(fmm_tree* T);
@@ -497,11 +544,9 @@ void build_tree(fmm_tree* T, const float* src, const float* tgt) {
                                                            T->tb.p, T->te.p, T->keys_s.p, keys_t, T->nchild.p);
         PB_CHECK_LAUNCH();
         scan.alloc(nb + 1, st);
-        exclusive_scan(T->nchild.p + lo, scan.p, nb, st);
-        int last_scan = read1(scan.p + nb - 1, st);
-        int last_n = read1(T->nchild.p + hi - 1, st);
-        int total = last_scan + last_n;
-        growall((size_t)hi + total);
+        exclusive_scan(T->nchild.p + lo, scan.p, nb + 1, st);    // scan[nb]: the children of this level
+        const int total = read1(scan.p + nb, st);
+        growall((size_t)hi + total + 1);             // (the scan reads one entry past the level)
         k_write_children<<<div_up(nb, 128), 128, 0, st>>>(lo, hi, lev, hi, T->same, scan.p, T->nchild.p,
                                                            T->first_child.p, T->sb.p, T->se.p, T->tb.p, T->te.p,
                                                            T->level.p, T->parent.p, T->anchor.p, T->keys_s.p,
@@ -549,126 +594,82 @@ void build_tree(fmm_tree* T, const float* src, const float* tgt) {
     PB_CUDA(cudaMemsetAsync(wcnt.p + nb, 0, sizeof(int), st));
     exclusive_scan(ucnt.p, T->U_off.p, nb + 1, st);
     exclusive_scan(wcnt.p, T->W_off.p, nb + 1, st);
-    T->n_u = read1(T->U_off.p + nb, st);
-    T->n_w = read1(T->W_off.p + nb, st);
+    {
+        int nu = 0, nw = 0;
+        PB_CUDA(cudaMemcpyAsync(&nu, T->U_off.p + nb, sizeof(int), cudaMemcpyDeviceToHost, st));
+        PB_CUDA(cudaMemcpyAsync(&nw, T->W_off.p + nb, sizeof(int), cudaMemcpyDeviceToHost, st));
+        PB_CUDA(cudaStreamSynchronize(st));
+        T->n_u = nu;
+        T->n_w = nw;
+    }
     T->U_ids.alloc(std::max<long long>(T->n_u, 1), st);
     T->W_ids.alloc(std::max<long long>(T->n_w, 1), st);
     k_leaf_lists<<<div_up(nb, 128), 128, 0, st>>>(nb, 1, T->nchild.p, T->first_child.p, T->anchor.p, T->coll.p,
                                                   T->coll_n.p, T->cn.p, T->cn_n.p, nullptr, nullptr, T->U_off.p,
                                                   T->W_off.p, T->U_ids.p, T->W_ids.p, ovf.p);
     PB_CHECK_LAUNCH();
-    PB_REQUIRE(read1(ovf.p, st) == 0, PB_EINVAL, "octree too deep for the list search stack");
-
-    // list totals
+    // 7. list totals, work counters and the index sets used by the FMM passes;
+    // everything the host needs of them comes back in one synchronisation
+    DBuf<int> tot;
+    tot.alloc(2, st);
     {
-        DBuf<int> tot;
-        tot.alloc(1, st);
         size_t tmp = 0;
         cub::DeviceReduce::Sum(nullptr, tmp, T->V_n.p, tot.p, nb, st);
         DBuf<char> t;
         t.alloc(tmp, st);
         cub::DeviceReduce::Sum(t.p, tmp, T->V_n.p, tot.p, nb, st);
-        T->n_v = read1(tot.p, st);
-        cub::DeviceReduce::Sum(t.p, tmp, T->X_n.p, tot.p, nb, st);
-        T->n_x = read1(tot.p, st);
+        cub::DeviceReduce::Sum(t.p, tmp, T->X_n.p, tot.p + 1, nb, st);
     }
-
-    // work counters
-    {
-        DBuf<unsigned long long> w;
-        w.alloc(6, st);
-        w.zero(st);
-        const int* tbeg0 = T->same ? T->sb.p : T->tb.p;
-        const int* tend0 = T->same ? T->se.p : T->te.p;
-        k_work<<<div_up(nb, 128), 128, 0, st>>>(nb, T->nchild.p, T->level.p, T->sb.p, T->se.p, tbeg0, tend0,
-                                                T->U_off.p, T->U_ids.p, T->W_off.p, T->X.p, T->X_n.p, w.p);
-        PB_CHECK_LAUNCH();
-        unsigned long long hw[6];
-        PB_CUDA(cudaMemcpyAsync(hw, w.p, sizeof(hw), cudaMemcpyDeviceToHost, st));
-        PB_CUDA(cudaStreamSynchronize(st));
-        for (int i = 0; i < 6; ++i) T->work[i] = (long long)hw[i];
-    }
-
-    // 7. index sets used by the FMM passes
-    DBuf<int> flag;
-    flag.alloc(nb, st);
     const int* tbeg = T->same ? T->sb.p : T->tb.p;
     const int* tend = T->same ? T->se.p : T->te.p;
+    DBuf<unsigned long long> w;
+    w.alloc(6, st);
+    w.zero(st);
+    k_work<<<div_up(nb, 128), 128, 0, st>>>(nb, T->nchild.p, T->level.p, T->sb.p, T->se.p, tbeg, tend, T->U_off.p,
+                                            T->U_ids.p, T->W_off.p, T->X.p, T->X_n.p, w.p);
+    PB_CHECK_LAUNCH();
+    DBuf<int> flag, pos;
+    flag.alloc(nb + 1, st);
+    flag.zero(st);
+    pos.alloc(3 * (size_t)(nb + 1), st);
+    int* pos_k[3] = {pos.p, pos.p + (nb + 1), pos.p + 2 * (size_t)(nb + 1)};
     k_flag<<<div_up(nb, 256), 256, 0, st>>>(nb, T->nchild.p, flag.p, 0, tbeg, tend);
-    T->n_tleaf = compact(flag.p, nb, T->leaf_ids, st);
+    compact(flag.p, nb, pos_k[0], T->leaf_ids, st);
     k_flag<<<div_up(nb, 256), 256, 0, st>>>(nb, T->nchild.p, flag.p, 1, T->sb.p, T->se.p);
-    int nsl = compact(flag.p, nb, T->sleaf_ids, st);
-    // leaves with sources are in box order = level order: find level boundaries
-    {
-        std::vector<int> ids(std::max(nsl, 1));
-        if (nsl) PB_CUDA(cudaMemcpyAsync(ids.data(), T->sleaf_ids.p, nsl * sizeof(int), cudaMemcpyDeviceToHost, st));
-        PB_CUDA(cudaStreamSynchronize(st));
-        T->sleaf_lvl_off.assign(T->nlev + 1, 0);
-        for (int l = 0; l <= T->nlev; ++l)
-            T->sleaf_lvl_off[l] = (int)(std::lower_bound(ids.begin(), ids.begin() + nsl, T->lvl_off[l]) - ids.begin());
-    }
+    compact(flag.p, nb, pos_k[1], T->sleaf_ids, st);
     k_flag<<<div_up(nb, 256), 256, 0, st>>>(nb, T->X_n.p, flag.p, 2, nullptr, nullptr);
-    T->n_xbox = compact(flag.p, nb, T->xbox_ids, st);
+    compact(flag.p, nb, pos_k[2], T->xbox_ids, st);
     {
-        std::vector<int> ids(std::max(T->n_xbox, 1));
-        if (T->n_xbox)
-            PB_CUDA(cudaMemcpyAsync(ids.data(), T->xbox_ids.p, T->n_xbox * sizeof(int), cudaMemcpyDeviceToHost, st));
-        PB_CUDA(cudaStreamSynchronize(st));
-        T->xbox_lvl_off.assign(T->nlev + 1, 0);
-        for (int l = 0; l <= T->nlev; ++l)
-            T->xbox_lvl_off[l] =
-                (int)(std::lower_bound(ids.begin(), ids.begin() + T->n_xbox, T->lvl_off[l]) - ids.begin());
-    }
-    {
-        // number of leaves
-        std::vector<int> nch(nb);
+        int hovf = 0, htot[2] = {0, 0}, cnt[3] = {0, 0, 0};
+        unsigned long long hw[6];
+        std::vector<int> sid(nb), xid(nb), nch(nb);
+        PB_CUDA(cudaMemcpyAsync(&hovf, ovf.p, sizeof(int), cudaMemcpyDeviceToHost, st));
+        PB_CUDA(cudaMemcpyAsync(htot, tot.p, sizeof(htot), cudaMemcpyDeviceToHost, st));
+        PB_CUDA(cudaMemcpyAsync(hw, w.p, sizeof(hw), cudaMemcpyDeviceToHost, st));
+        for (int k = 0; k < 3; ++k)
+            PB_CUDA(cudaMemcpyAsync(cnt + k, pos_k[k] + nb, sizeof(int), cudaMemcpyDeviceToHost, st));
+        PB_CUDA(cudaMemcpyAsync(sid.data(), T->sleaf_ids.p, nb * sizeof(int), cudaMemcpyDeviceToHost, st));
+        PB_CUDA(cudaMemcpyAsync(xid.data(), T->xbox_ids.p, nb * sizeof(int), cudaMemcpyDeviceToHost, st));
         PB_CUDA(cudaMemcpyAsync(nch.data(), T->nchild.p, nb * sizeof(int), cudaMemcpyDeviceToHost, st));
         PB_CUDA(cudaStreamSynchronize(st));
+        PB_REQUIRE(hovf == 0, PB_EINVAL, "octree too deep for the list search stack");
+        T->n_v = htot[0];
+        T->n_x = htot[1];
+        for (int i = 0; i < 6; ++i) T->work[i] = (long long)hw[i];
+        T->n_tleaf = cnt[0];
+        T->n_xbox = cnt[2];
         T->nleaf = (int)std::count(nch.begin(), nch.end(), 0);
+        // both sets are in box order = level order: level boundaries
+        auto bounds = [&](const std::vector<int>& ids, int n, std::vector<int>& off) {
+            off.assign(T->nlev + 1, 0);
+            for (int l = 0; l <= T->nlev; ++l)
+                off[l] = (int)(std::lower_bound(ids.begin(), ids.begin() + n, T->lvl_off[l]) - ids.begin());
+        };
+        bounds(sid, cnt[1], T->sleaf_lvl_off);
+        bounds(xid, cnt[2], T->xbox_lvl_off);
     }
 
-    // 8. M2L tile schedule: boxes with a non-empty V list, per level, tiles of kM2LTile
-    {
-        std::vector<int> vn(nb);
-        PB_CUDA(cudaMemcpyAsync(vn.data(), T->V_n.p, nb * sizeof(int), cudaMemcpyDeviceToHost, st));
-        PB_CUDA(cudaStreamSynchronize(st));
-        std::vector<int> tiles, tlev;
-        for (int l = 0; l < T->nlev; ++l) {
-            std::vector<int> cur;
-            for (int b = T->lvl_off[l]; b < T->lvl_off[l + 1]; ++b)
-                if (vn[b] > 0) cur.push_back(b);
-            for (size_t i = 0; i < cur.size(); i += kM2LTile) {
-                for (int c = 0; c < kM2LTile; ++c)
-                    tiles.push_back(i + c < cur.size() ? cur[i + c] : -1);
-                tlev.push_back(l);
-            }
-        }
-        M2LSchedule& S = T->m2l;
-        S.ntile = (int)tlev.size();
-        S.tile_level_h = tlev;
-        S.npairs = T->n_v;
-        if (S.ntile > 0) {
-            S.tile_box.alloc(tiles.size(), st);
-            S.tile_level.alloc(S.ntile, st);
-            PB_CUDA(cudaMemcpyAsync(S.tile_box.p, tiles.data(), tiles.size() * sizeof(int), cudaMemcpyHostToDevice, st));
-            PB_CUDA(cudaMemcpyAsync(S.tile_level.p, tlev.data(), tlev.size() * sizeof(int), cudaMemcpyHostToDevice, st));
-            DBuf<int> cnt;
-            cnt.alloc(S.ntile + 1, st);
-            cnt.zero(st);
-            S.entry_off.alloc(S.ntile + 1, st);
-            k_m2l_schedule<<<S.ntile, 128, 0, st>>>(S.ntile, S.tile_box.p, T->anchor.p, T->V.p, T->V_n.p, nullptr,
-                                                    cnt.p, nullptr, nullptr, 0);
-            PB_CHECK_LAUNCH();
-            exclusive_scan(cnt.p, S.entry_off.p, S.ntile + 1, st);
-            S.nentry = read1(S.entry_off.p + S.ntile, st);
-            S.entry_offset_idx.alloc(std::max<long long>(S.nentry, 1), st);
-            S.entry_src.alloc(std::max<long long>(S.nentry, 1) * kM2LTile, st);
-            k_m2l_schedule<<<S.ntile, 128, 0, st>>>(S.ntile, S.tile_box.p, T->anchor.p, T->V.p, T->V_n.p,
-                                                    S.entry_off.p, nullptr, S.entry_offset_idx.p, S.entry_src.p, 1);
-            PB_CHECK_LAUNCH();
-        }
-    }
-    // 9. V-list pairs grouped by (level, offset) for the tensor-core M2L
+    // 8. V-list pairs grouped by (level, offset) for the tensor-core M2L
     build_m2l_pairs(T);
     build_pc_pairs(T);
     build_c2e_items(T);

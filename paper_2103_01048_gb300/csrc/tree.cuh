@@ -105,7 +105,8 @@ struct fmm_tree {
     int n_xbox = 0;
     std::vector<int> xbox_lvl_off;           // [nlev + 1]
     // non-leaf boxes per level (M2M parents) and all boxes per level for L2L
-    pbfmm::M2LSchedule m2l;
+    pbfmm::M2LSchedule m2l;                  // (built on first use: build_m2l_schedule)
+    bool m2l_built = false;
     pbfmm::M2LPairs m2l_pairs;
     pbfmm::PCPairs pc_pairs;
     // tensor-core items of the check -> equivalent solves: (first, count,
