@@ -40,21 +40,29 @@ constexpr int kHRowsPerThr = kHRows / (kHProdWarps * 4);  // rows a producer thr
 constexpr int kHThreads = 32 * (kHProdWarps + kHEpiWarps + 1);
 constexpr uint32_t kHStageBytes = kHRows * 128; // one K block of a row tile, hi and lo
 
-// Per padded size: NS row parts of the operator (the part a CTA holds is
-// N = npad / NS rows, all columns), A stages.  Sizes: operator part npad * N * 4 B <= 128 KB, the rest of
-// the 227 KB for the stages.
+// Per padded size: the operator is cut into NS row parts times KS column
+// parts, each N = npad / NS rows by npad / KS columns (<= 128 KB as hi + lo
+// halves), one of them held by a CTA at a time; STAGES A stages in the rest of
+// the 227 KB.  Row parts gather every source row again, column parts add
+// every target row again, and a narrow tile leaves the tensor core idle: six
+// MMAs take 72 cycles each at N = 64 or 80 (32 and 40 of work), 84 at N = 160.
+// Measured, NS x KS: p = 8 with 500,000 points 4 x 1 1.066 ms, 2 x 2 0.847;
+// p = 10 with 197,000 points 8 x 1 1.52 ms, 4 x 2 1.051, 2 x 4 1.008.
 template <int NPAD> struct HCfg;
-template <> struct HCfg<32> { static constexpr int NS = 1, STAGES = 4; };
-template <> struct HCfg<64> { static constexpr int NS = 1, STAGES = 8; };
-template <> struct HCfg<128> { static constexpr int NS = 1, STAGES = 8; };
-template <> struct HCfg<160> { static constexpr int NS = 1, STAGES = 6; };
-template <> struct HCfg<320> { static constexpr int NS = 4, STAGES = 6; };
-template <> struct HCfg<512> { static constexpr int NS = 8, STAGES = 5; };
+template <> struct HCfg<32> { static constexpr int NS = 1, KS = 1, STAGES = 4; };
+template <> struct HCfg<64> { static constexpr int NS = 1, KS = 1, STAGES = 8; };
+template <> struct HCfg<128> { static constexpr int NS = 1, KS = 1, STAGES = 8; };
+template <> struct HCfg<160> { static constexpr int NS = 1, KS = 1, STAGES = 6; };
+template <> struct HCfg<320> { static constexpr int NS = 2, KS = 2, STAGES = 6; };
+template <> struct HCfg<512> { static constexpr int NS = 2, KS = 4, STAGES = 5; };
 
 bool m2l_h_supported(int npad) {
     return npad == 32 || npad == 64 || npad == 128 || npad == 160 || npad == 320 || npad == 512;
 }
-static int h_parts(int npad) { return npad == 320 ? HCfg<320>::NS : (npad == 512 ? HCfg<512>::NS : 1); }
+static void h_split(int npad, int& ns, int& ks) {
+    ns = npad == 320 ? HCfg<320>::NS : (npad == 512 ? HCfg<512>::NS : 1);
+    ks = npad == 320 ? HCfg<320>::KS : (npad == 512 ? HCfg<512>::KS : 1);
+}
 
 // 2^s with the largest scaled entry in [2^14, 2^15); 0 for zero, infinite or NaN rows
 __device__ __forceinline__ int h_scale_exp(float m) {
@@ -140,7 +148,7 @@ __global__ void __launch_bounds__(256) k_h_pack_rows(int nbox, int npad, HPack P
 // Operators: [operator][part][K block][N rows][32 hi | 32 lo] halves,
 // swizzled, and the inverse scales.  One CTA per operator; slot -> offset by
 // the rule of the file's head.
-__global__ void __launch_bounds__(256) k_h_pack_ops(int npad, int NS, int nslot, int level0, const float* __restrict__ m2l,
+__global__ void __launch_bounds__(256) k_h_pack_ops(int npad, int NS, int KS, int nslot, int level0, const float* __restrict__ m2l,
                                                     uint8_t* __restrict__ out, float* __restrict__ inv) {
     __shared__ float red[256];
     const int slot = blockIdx.x, lev = blockIdx.y;
@@ -161,15 +169,15 @@ __global__ void __launch_bounds__(256) k_h_pack_ops(int npad, int NS, int nslot,
     const size_t op = (size_t)lev * nslot + slot;
     if (threadIdx.x == 0) inv[op] = h_pow2(-s);
     uint8_t* base = out + op * m2 * 4;
-    const int N = npad / NS, ng = npad / 8;
+    const int N = npad / NS, KB = npad / KS / 32, ng = npad / 8;
     for (int e = threadIdx.x; e < npad * ng; e += 256) {
         const int n = e / ng, g = e % ng;
         float v[8];
         for (int i = 0; i < 8; ++i) v[i] = M[(size_t)n * npad + 32 * (g >> 2) + h_col(g & 3, i)];
         uint4 hi, lo;
         h_split8(v, sc, hi, lo);
-        const int part = n / N, r = n % N, kb = g >> 2, c = g & 3;
-        uint8_t* blk = base + (size_t)part * N * npad * 4 + (size_t)kb * N * 128 + (r >> 3) * 1024 + (r & 7) * 128;
+        const int r = n % N, kb = g >> 2, c = g & 3, part = (n / N) * KS + kb / KB;
+        uint8_t* blk = base + ((size_t)part * KB + kb % KB) * N * 128 + (r >> 3) * 1024 + (r & 7) * 128;
         *reinterpret_cast<uint4*>(blk + ((c ^ (r & 7)) << 4)) = hi;
         *reinterpret_cast<uint4*>(blk + (((4 + c) ^ (r & 7)) << 4)) = lo;
     }
@@ -183,7 +191,9 @@ void pack_m2l_h(Operators& O, cudaStream_t st) {
     const size_t nop = (size_t)lev * O.h_nslot;
     O.m2l_h.alloc(nop * O.npad * O.npad * 4, st);
     O.m2l_h_inv.alloc(nop, st);
-    k_h_pack_ops<<<dim3(O.h_nslot, lev), 256, 0, st>>>(O.npad, h_parts(O.npad), O.h_nslot, l0, O.m2l.p, O.m2l_h.p,
+    int ns, ks;
+    h_split(O.npad, ns, ks);
+    k_h_pack_ops<<<dim3(O.h_nslot, lev), 256, 0, st>>>(O.npad, ns, ks, O.h_nslot, l0, O.m2l.p, O.m2l_h.p,
                                                        O.m2l_h_inv.p);
     PB_CHECK_LAUNCH();
 }
@@ -288,7 +298,8 @@ struct HCursor {
 template <int NPAD>
 __global__ void __launch_bounds__(kHThreads, 1) k_m2l_f16(const HArgs A) {
     using C = HCfg<NPAD>;
-    constexpr int N = NPAD / C::NS, KB = NPAD / 32, STAGES = C::STAGES;
+    constexpr int NP = C::NS * C::KS;            // operator parts
+    constexpr int N = NPAD / C::NS, KB = NPAD / C::KS / 32, STAGES = C::STAGES;
     static_assert(N % 16 == 0 && N <= 256, "split");
     constexpr uint32_t BBYTES = KB * N * 128;
     constexpr uint32_t ACOLS = N <= 32 ? 32 : (N <= 64 ? 64 : (N <= 128 ? 128 : 256));
@@ -304,7 +315,7 @@ __global__ void __launch_bounds__(kHThreads, 1) k_m2l_f16(const HArgs A) {
     const long long wl = A.wait_limit;
     int nu = 0;                                  // this CTA's units
     for (int k = 0; k < A.nseg; ++k) {
-        const long long n = (long long)(A.seg[k + 1] - A.seg[k]) * C::NS;
+        const long long n = (long long)(A.seg[k + 1] - A.seg[k]) * NP;
         nu += (int)(n * (blockIdx.x + 1) / gridDim.x) - (int)(n * blockIdx.x / gridDim.x);
     }
     nu *= A.nset;
@@ -333,7 +344,7 @@ __global__ void __launch_bounds__(kHThreads, 1) k_m2l_f16(const HArgs A) {
     const uint32_t taddr = S->tmem_slot;
 
     HCursor cur;
-    cur.start(A, C::NS);
+    cur.start(A, NP);
     if (warp < kHProdWarps) {
         // PF K blocks of loads in flight in registers (more spill: 2.09
         // against 1.61 ms at 4M points, p = 6, with PF = 4)
@@ -357,27 +368,32 @@ __global__ void __launch_bounds__(kHThreads, 1) k_m2l_f16(const HArgs A) {
         uint32_t xm[PF];
         int sc[kHRowsPerThr], sn[kHRowsPerThr];
         int fu = 0, fkb = 0;                     // the next block to fetch
-        int set1 = cur.set, set2;                // sets of the units fu + 1 and fu + 2
-        const uint4* X = A.X[set1 < A.nset ? set1 : 0] + l8;
+        // a unit's set and column part of the source rows, and where these begin
+        auto sp_of = [&]() { return cur.set * C::KS + cur.part % C::KS; };
+        auto x_of = [&](int sp) {
+            return sp < A.nset * C::KS ? A.X[sp / C::KS] + (sp % C::KS) * KB * 8 + l8 : nullptr;
+        };
+        int sp1 = sp_of(), sp2;                  // of the units fu + 1 and fu + 2
+        const uint4* X = x_of(sp1);
         load_src(tile_of(), sc);
-        cur.next(A, C::NS);
-        set1 = cur.set;
+        cur.next(A, NP);
+        sp1 = sp_of();
         load_src(tile_of(), sn);
-        cur.next(A, C::NS);
-        set2 = cur.set;
+        cur.next(A, NP);
+        sp2 = sp_of();
         int2 td = tile_of();
         auto fetch = [&](uint4* d, uint32_t& x) {
             if (fkb == KB) {
                 fkb = 0;
                 ++fu;
-                if (set1 < A.nset) X = A.X[set1] + l8;
+                X = x_of(sp1);
 #pragma unroll
                 for (int i = 0; i < kHRowsPerThr; ++i) sc[i] = sn[i];
                 load_src(td, sn);
-                cur.next(A, C::NS);
+                cur.next(A, NP);
                 td = tile_of();
-                set1 = set2;
-                set2 = cur.set;
+                sp1 = sp2;
+                sp2 = sp_of();
             }
             x = 0;
             if (fu < nu) {
@@ -435,12 +451,12 @@ __global__ void __launch_bounds__(kHThreads, 1) k_m2l_f16(const HArgs A) {
             if (sx < 0) return 0.f;
             return A.ix[set][sx & 0x0fffffff] * A.iop[set][(A.single[set] ? 0 : (z & 31) * A.nslot) + (z >> 5)];
         };
-        for (int i = 0; i < eg; ++i) cur.next(A, C::NS);
+        for (int i = 0; i < eg; ++i) cur.next(A, NP);
         int set = cur.set, part = cur.part;
         int4 t = tile_of();
         Row row = load_row(t);
         float f = load_scale(set, t.z, row.sx);
-        for (int i = 0; i < EG; ++i) cur.next(A, C::NS);
+        for (int i = 0; i < EG; ++i) cur.next(A, NP);
         int set1 = cur.set, part1 = cur.part;
         t = tile_of();
         for (int k = eg; k < nu; k += EG) {
@@ -448,7 +464,7 @@ __global__ void __launch_bounds__(kHThreads, 1) k_m2l_f16(const HArgs A) {
             const int x = (row.sx >> 28) & 7;
             const Row row1 = load_row(t);
             const int z1 = t.z;
-            for (int i = 0; i < EG; ++i) cur.next(A, C::NS);
+            for (int i = 0; i < EG; ++i) cur.next(A, NP);
             const int set2 = cur.set, part2 = cur.part;
             t = tile_of();
             // after the transpose a lane adds 16 B of the rows j * 8 + lane / 4
@@ -456,9 +472,9 @@ __global__ void __launch_bounds__(kHThreads, 1) k_m2l_f16(const HArgs A) {
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int tr = __shfl_sync(0xffffffffu, row.tgt, j * 8 + (lane >> 2));
-                y[j] = tr >= 0 ? A.Y[set] + (size_t)tr * NPAD + part * N + (lane & 3) * 4 : nullptr;
+                y[j] = tr >= 0 ? A.Y[set] + (size_t)tr * NPAD + (part / C::KS) * N + (lane & 3) * 4 : nullptr;
             }
-            const int cmax = A.ncols - part * N - (lane & 3) * 4;      // this lane's columns end
+            const int cmax = A.ncols - (part / C::KS) * N - (lane & 3) * 4;      // this lane's columns end
             const bool ok = h_wait(&S->accf[a], (k >> 1) & 1, failed, wl);
             if (!__all_sync(0xffffffffu, ok)) break;
             tc_fence_after();
@@ -522,8 +538,8 @@ __global__ void __launch_bounds__(kHThreads, 1) k_m2l_f16(const HArgs A) {
         for (int k = 0; ok && k < nu; ++k) {
             const int a = k & 1;
             const int op = (A.single[cur.set] ? 0 : (t.z & 31) * A.nslot) + (t.z >> 5);
-            const uint8_t* want = A.ops[cur.set] + ((size_t)op * C::NS + cur.part) * BBYTES;
-            cur.next(A, C::NS);
+            const uint8_t* want = A.ops[cur.set] + ((size_t)op * NP + cur.part) * BBYTES;
+            cur.next(A, NP);
             if (k + 1 < nu) t = A.tiles[cur.tile];
             if (want != held) {
                 // every MMA that reads the held part is done before it is overwritten
@@ -579,7 +595,7 @@ __global__ void __launch_bounds__(kHThreads, 1) k_m2l_f16(const HArgs A) {
 template <int NPAD>
 static constexpr size_t h_smem_bytes() {
     using C = HCfg<NPAD>;
-    return 1024 + (size_t)NPAD * (NPAD / C::NS) * 4 + C::STAGES * (size_t)kHStageBytes +
+    return 1024 + (size_t)(NPAD / C::KS) * (NPAD / C::NS) * 4 + C::STAGES * (size_t)kHStageBytes +
            kHEpiWarps * 32 * 16 * sizeof(float) + sizeof(HSmem<C::STAGES>);
 }
 static_assert(h_smem_bytes<128>() <= 232448 && h_smem_bytes<160>() <= 232448 && h_smem_bytes<320>() <= 232448 &&
@@ -596,7 +612,7 @@ static void h_launch(const HArgs& a, int ntile, int sm_count, cudaStream_t st) {
                                      (int)h_smem_bytes<NPAD>()));
         done[dev] = true;
     }
-    const int grid = (int)std::min<long long>(sm_count, (long long)ntile * HCfg<NPAD>::NS * a.nset);
+    const int grid = (int)std::min<long long>(sm_count, (long long)ntile * HCfg<NPAD>::NS * HCfg<NPAD>::KS * a.nset);
     k_m2l_f16<NPAD><<<grid, kHThreads, h_smem_bytes<NPAD>(), st>>>(a);
     PB_CHECK_LAUNCH();
 }
@@ -671,7 +687,9 @@ void m2l_h_selftest(int nrows, int npad, const float* Q, const float* Op, const 
     PB_CUDA(cudaMemcpyAsync(m2l.p + kOffset * m2, Op, m2 * sizeof(float), cudaMemcpyDeviceToDevice, st));
     ops.alloc(64 * m2 * 4, st);
     inv.alloc(64, st);
-    k_h_pack_ops<<<dim3(64, 1), 256, 0, st>>>(npad, h_parts(npad), 64, 0, m2l.p, ops.p, inv.p);
+    int ns, ks;
+    h_split(npad, ns, ks);
+    k_h_pack_ops<<<dim3(64, 1), 256, 0, st>>>(npad, ns, ks, 64, 0, m2l.p, ops.p, inv.p);
     PB_CHECK_LAUNCH();
     std::vector<int> ht(nrows), hs(nrows);
     for (int i = 0; i < nrows; ++i) { ht[i] = i; hs[i] = i | (xs ? xs[i] & 7 : 0) << 28; }
