@@ -714,23 +714,25 @@ def main():
             "dominant_phase": dom}
     launches = prof["launches"]
     # M2L on the tensor cores: algorithmic FLOPs 2 n_e^2 per V-list pair and
-    # kernel (the un-split product) against the measured TF32 rate
+    # kernel (the un-split product) against the measured half-precision rate
+    # (BF16 and half have the same)
     m2l_ms = phases["m2l"][0] / args.steps if "m2l" in phases else None
     roof_m2l = None
     if m2l_ms:
         npad = (ne + 31) // 32 * 32
         m2l_flops = 2 * 2.0 * ne * ne * info.n_v
-        roof_m2l = {"kernel": "k_m2l_tc (tcgen05 kind::tf32, Laplace+Yukawa in one launch)", "bound": "tensor",
-                    "achieved": m2l_flops / (m2l_ms * 1e-3) / 1e12, "peak": peaks["tf32_tc_tflops"],
-                    "unit": "TFLOP/s", "frac": m2l_flops / (m2l_ms * 1e-3) / 1e12 / peaks["tf32_tc_tflops"],
+        roof_m2l = {"kernel": "k_m2l_f16 (tcgen05 kind::f16 on split halves, Laplace+Yukawa in one launch)", "bound": "tensor",
+                    "achieved": m2l_flops / (m2l_ms * 1e-3) / 1e12, "peak": peaks["bf16_tc_tflops"],
+                    "unit": "TFLOP/s", "frac": m2l_flops / (m2l_ms * 1e-3) / 1e12 / peaks["bf16_tc_tflops"],
                     "issued_frac": 3 * 2 * 2.0 * npad * npad * info.n_v / (m2l_ms * 1e-3) / 1e12
-                    / peaks["tf32_tc_tflops"],
+                    / peaks["bf16_tc_tflops"],
                     "frac_of_fp32_accurate_roof": m2l_flops / (m2l_ms * 1e-3) / 1e12
-                    / (peaks["tf32_tc_tflops"] / 3.0),
+                    / (peaks["bf16_tc_tflops"] / 3.0),
                     "note": "achieved = 2 n_e^2 x V-list pairs x 2 kernels / M2L phase time; issued_frac counts "
-                            "the 3 TF32 products (hi*hi, hi*lo, lo*hi) at the padded size n_pad actually issued; "
-                            "frac_of_fp32_accurate_roof divides by TF32 / 3, the rate of a contraction that keeps "
-                            "FP32 accuracy with three TF32 products"}
+                            "the 3 half-precision products (hi*hi, hi*lo, lo*hi) at the padded size n_pad actually issued; "
+                            "frac_of_fp32_accurate_roof divides by that rate / 3, the rate of a contraction that "
+                            "keeps FP32 accuracy with three products of 11-bit halves; the kernel is bound by "
+                            "the L2's reductions into the target rows"}
 
     clocks = clk.summary()
 

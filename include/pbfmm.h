@@ -149,18 +149,17 @@ int pb_profile(pb_ctx* ctx, int enable);
  *                         residual with one mat-vec and starts a new cycle.
  *   PB_OPT_LEAF_NT        targets per thread of the leaf (P2P + M2P + L2P)
  *                         kernel of fmm_apply_pair: 0 (default): 4 in FP32,
- *                         2 in FP64; 2 or 4.  A tile-shape knob of the
+ *                         2 in FP64 and with target-normal derivatives; 2 or
+ *                         4.  A tile-shape knob of the
  *                         autotuner (pb_tune); results differ only by
  *                         the summation order of each target's partial sums.
- *   PB_OPT_LEAF_PACKED    1 (default): the FP32 leaf kernel of fmm_apply_pair
- *                         without target-normal derivatives takes two sources
- *                         per packed instruction (add/mul/fma .f32x2); 0: one
+ *   PB_OPT_LEAF_PACKED    1 (default): the FP32 leaf kernel takes two sources per
+ *                         packed instruction (add/mul/fma .f32x2); 0: one
  *                         source per scalar instruction.  Same arithmetic per
  *                         pair, summation order of the partial sums differs.
  *   PB_OPT_M2L_TILE       0 or 1: accepted for compatibility, without effect
  *                         (the tensor-core M2L has one row tile, 128 pairs).
- *   PB_OPT_LIST_DIRECT    1 (default): in the FP32 applies without
- *                         target-normal derivatives (fmm_apply_pair and
+ *   PB_OPT_LIST_DIRECT    1 (default): in the FP32 applies (fmm_apply_pair and
  *                         fmm_apply on the packed kernels, PB_OPT_LEAF_PACKED
  *                         1), the pairs of the adaptive lists are summed directly
  *                         where that is less work than the equivalent

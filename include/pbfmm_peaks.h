@@ -2,8 +2,8 @@
  * Measured arithmetic peaks of a GPU: the denominators of the pbfmm
  * kernels' rooflines (the near field and check potentials are bound by the
  * FP32 fused multiply-add pipe and the MUFU reciprocal-square-root and
- * exponential units; the box operators by the tensor cores' TF32 rate; the
- * all-FP64 path by FP64 arithmetic).  Not part of the solver's interface.
+ * exponential units; the box operators by the tensor cores' TF32 rate, the
+ * M2L by their half-precision rate, which is BF16's; the all-FP64 path by FP64 arithmetic).  Not part of the solver's interface.
  */
 #ifndef PBFMM_PEAKS_H
 #define PBFMM_PEAKS_H

@@ -1258,16 +1258,23 @@ static const LeafStream& leaf_stream(fmm_tree* T, int thrW, int thrX) {
     return *p;
 }
 
-// The paired leaf kernel in packed FP32: the work split of k_leaf_pair (NT targets per thread, G groups, the near field
-// in windows of the concatenated U-list sources, the leaf itself first, then
-// the far field in windows of generated equivalent points), with each window
+// The paired leaf kernel in packed FP32: the work split of k_leaf_pair (NT
+// targets per thread, G groups, the near field in windows of the concatenated
+// U-list sources, the leaf itself first, then the far field in windows of
+// generated equivalent points), with each window
 // stored as pairs of points, every value pair one 64-bit half of a 16-byte
 // vector, so that group g takes the pairs g, g + G, ... and one packed
 // instruction serves two sources.  An odd window is padded with a point of
 // zero weight 1e10 away (its terms are exactly 0).
 // Grid y: the windows are dealt out to S = gridDim.y CTAs (windows of 1,024 / S
 // points), each with its own partial outputs, added in order by the scatter:
-// trees of a few hundred leaves fill the GPU (see leaf_split).
+// trees of a few hundred leaves fill the GPU (see leaf_split); SPLIT is a
+// template parameter because a run-time S cost the large trees 7% (4M points:
+// 4.29 against 4.00 ms).
+// Bound: the FP32 FMA pipe.  At 4M points, p = 6, 3.76 ms: near sums 2.3 (4.8e9
+// pairs at the pipe's rate), far sums 0.5, filling windows and waiting for
+// them the rest.  15,000 points 0.127 -> 0.057 ms; adjoint (DN), 240,000
+// points 0.78 -> 0.44 against the scalar kernel.
 template <bool DL, bool DN, int NT, int PART, int KM, bool SPLIT>
 __global__ void __launch_bounds__(128, 5) k_leaf_pair_x2(const LeafStream::Rec* __restrict__ recs,
                                                       const int2* __restrict__ near_l,

@@ -26,7 +26,11 @@
 //
 // Bound: the reductions into Qd.  They cost n_e * 4 B per pair at the L2's
 // rate for them (measured on random rows: 5.9 TB/s for 64-byte pieces of
-// red.v4; 16-byte pieces 3.3, 32-byte 4.2).
+// red.v4; 16-byte pieces 3.3, 32-byte 4.2).  At p = 8 and 10 the MMAs (three
+// products) take as long.  Before (TF32, one operator per offset, CTA pairs)
+// -> now, both kernels: p = 4, 3M points 1.35 -> 0.62 ms; p = 6, 15,000 0.18
+// -> 0.03, 240,000 0.40 -> 0.14, 4M 2.74 -> 1.62; p = 8, 500,000 1.98 -> 0.85;
+// p = 10, 197,000 3.19 -> 1.01.
 #include "fmm.cuh"
 #include "tc_ptx.cuh"
 #include <cuda_fp16.h>
@@ -287,7 +291,9 @@ struct HCursor {
 // boxes (consecutive boxes of a level, hence neighbours), slot-major inside
 // a segment: all CTAs work on one segment at a time, so its rows of Qu and
 // Qd stay in L2 while its ~300 offsets pass over them, and a CTA reloads its
-// operator part only where its contiguous range crosses a slot.
+// operator part only where its contiguous range crosses a slot.  (Reductions
+// by bulk copies from a staging buffer, which takes the place of A stages:
+// 1.84 ms at 4M points, p = 6.)
 //   warps 0-7   producers: gather source rows (16 B per lane, eight lanes per
 //               128-byte K-block row), reflect them, write them swizzled
 //               into a ring of A stages;

@@ -2,10 +2,10 @@
 // of the kernels that are bound by plain ALU work (the near field and the
 // check potentials: FP32 fused multiply-add and the MUFU reciprocal square
 // root and base-2 exponential), by FP64 arithmetic (the all-FP64 path), or
-// by the tensor cores (box operators: tcgen05 kind::tf32).  The BF16
-// tensor-core rate is measured with the same loop to compare this method
-// with a library GEMM's measured rate, and the packed FP32 FMA
-// (fma.rn.f32x2, two FMAs per instruction) to see whether packing raises
+// by the tensor cores (box operators: tcgen05 kind::tf32; M2L: kind::f16,
+// whose half and BF16 rates are equal).  The BF16 rate also compares this
+// method with a library GEMM's measured rate.  The packed FP32 FMA
+// (fma.rn.f32x2, two FMAs per instruction) shows whether packing raises
 // the FP32 rate or only halves the instructions.
 //
 // Each ALU kernel runs independent dependency chains in every thread (enough
