@@ -1258,6 +1258,15 @@ static const LeafStream& leaf_stream(fmm_tree* T, int thrW, int thrX) {
     return *p;
 }
 
+// The streams of an apply, built here if they are not (on the context stream:
+// before any fork to the second one, whose kernels wait for the fork only);
+// null where the scalar leaf kernels run.
+template <typename T>
+static const LeafStream* leaf_streams_for(fmm_tree* Tr, const Operators& O, int thrW, int thrX) {
+    if (!std::is_same<T, float>::value || !Tr->ctx->leaf_packed || O.ne > 1024 || Tr->n_tleaf <= 0) return nullptr;
+    return &leaf_stream(Tr, thrW, thrX);
+}
+
 // The paired leaf kernel in packed FP32: the work split of k_leaf_pair (NT
 // targets per thread, G groups, the near field in windows of the concatenated
 // U-list sources, the leaf itself first, then the far field in windows of
@@ -1687,21 +1696,20 @@ static int leaf_split(const fmm_tree* Tr, bool fp64) {
 }
 
 template <typename T, bool YUK, bool DL, bool DN>
-static void launch_leaf(cudaStream_t st, fmm_tree* Tr, Work<T>& W, const Operators& O, T kappa, int thrW = -1,
-                        int thrX = -1, int split = 1) {
+static void launch_leaf(cudaStream_t st, fmm_tree* Tr, Work<T>& W, const Operators& O, T kappa, const LeafStream* L,
+                        int split) {
     if (Tr->n_tleaf <= 0) return;
     const float4* tpos = Tr->same ? Tr->pos_s.p : Tr->pos_t.p;
     const int* tb = Tr->same ? Tr->sb.p : Tr->tb.p;
     const int* te = Tr->same ? Tr->se.p : Tr->te.p;
     if constexpr (std::is_same<T, float>::value) {
-        if (Tr->ctx->leaf_packed && O.ne <= 1024) {
+        if (L) {
             // the packed leaf kernel for one kernel (KM 1: Laplace, 2: Yukawa)
             constexpr int KM = YUK ? 2 : 1;
             const int NT = Tr->ctx->leaf_nt ? Tr->ctx->leaf_nt : (DN ? 2 : 4);
             auto k = split > 1 ? (NT == 4 ? k_leaf_pair_x2<DL, DN, 4, 0, KM, true> : k_leaf_pair_x2<DL, DN, 2, 0, KM, true>)
                                : (NT == 4 ? k_leaf_pair_x2<DL, DN, 4, 0, KM, false> : k_leaf_pair_x2<DL, DN, 2, 0, KM, false>);
-            const LeafStream& L = leaf_stream(Tr, thrW, thrX);
-            k<<<dim3(Tr->n_tleaf, split), 128, 0, st>>>(L.rec.p, L.near.p, L.far_geo.p, L.far_box.p, tpos, W.sq.p,
+            k<<<dim3(Tr->n_tleaf, split), 128, 0, st>>>(L->rec.p, L->near.p, L->far_geo.p, L->far_box.p, tpos, W.sq.p,
                                                         W.sm.p, W.Qu.p, W.Qd.p, nullptr, nullptr,
                                                         (const float4*)O.surf_f.p, O.ne, O.npad, kappa,
                                                         YUK ? nullptr : W.pot.p, YUK ? W.pot.p : nullptr, W.tn.p,
@@ -1711,8 +1719,7 @@ static void launch_leaf(cudaStream_t st, fmm_tree* Tr, Work<T>& W, const Operato
             return;
         }
     }
-    PB_REQUIRE(thrW < 0 && thrX < 0 && split == 1, PB_EINVAL,
-               "direct W/X-list evaluation and split leaves need the packed leaf kernel");
+    PB_REQUIRE(split == 1, PB_EINVAL, "split leaves need the packed leaf kernel");
     constexpr int NT = 2;     // 4 measured slower (register pressure)
     k_leaf_eval<T, YUK, DL, DN, NT><<<Tr->n_tleaf, 128, 0, st>>>(
         Tr->leaf_ids.p, Tr->n_tleaf, tb, te, Tr->sb.p, Tr->se.p, Tr->U_off.p, Tr->U_ids.p, Tr->W_off.p, Tr->W_ids.p,
@@ -1955,6 +1962,7 @@ static void apply_t(fmm_tree* Tr, const Operators& O, double kappa_d, const In* 
     const bool ld = packed && ldm != 0;
     const int split = packed ? leaf_split(Tr, false) : 1;
     const int thrW = ld && ldm != 2 ? O.ne / 2 : -1, thrX = ld && ldm != 3 ? O.ne : -1;
+    const LeafStream* L = leaf_streams_for<T>(Tr, O, thrW, thrX);
     Work<T> W;
     W.sq.alloc(ns, st);
     if (DL) W.sm.alloc(ns, st);
@@ -1999,9 +2007,9 @@ static void apply_t(fmm_tree* Tr, const Operators& O, double kappa_d, const In* 
     far_l2l(Tr, O, W);
     ph.reset(); ph = std::make_unique<PhaseTimer>(ctx, PB_PH_LEAF);
     // ---- leaves: P2P + M2P + L2P
-    if (DL) launch_leaf<T, YUK, true, false>(st, Tr, W, O, kappa, thrW, thrX, split);
-    else if (DN) launch_leaf<T, YUK, false, true>(st, Tr, W, O, kappa, thrW, thrX, split);
-    else launch_leaf<T, YUK, false, false>(st, Tr, W, O, kappa, thrW, thrX, split);
+    if (DL) launch_leaf<T, YUK, true, false>(st, Tr, W, O, kappa, L, split);
+    else if (DN) launch_leaf<T, YUK, false, true>(st, Tr, W, O, kappa, L, split);
+    else launch_leaf<T, YUK, false, false>(st, Tr, W, O, kappa, L, split);
     ph.reset(); ph = std::make_unique<PhaseTimer>(ctx, PB_PH_SCATTER);
     const int* pt = Tr->same ? Tr->perm_s.p : Tr->perm_t.p;
     const Scatter<T, In> sc{{W.pot.p, W.dn.p}, {out, out_dn}};
@@ -2070,19 +2078,18 @@ static void launch_p2check_pair(cudaStream_t st, int nbox, const int* boxes, int
 
 template <typename T, bool DL, bool DN, int PART>
 static void launch_leaf_pair(cudaStream_t st, fmm_tree* Tr, Work<T>& WL, Work<T>& WY, const Operators& O, T kappa,
-                             int thrW = -1, int thrX = -1, int split = 1) {
+                             const LeafStream* L, int split) {
     if (Tr->n_tleaf <= 0) return;
     const float4* tpos = Tr->same ? Tr->pos_s.p : Tr->pos_t.p;
     const int* tb = Tr->same ? Tr->sb.p : Tr->tb.p;
     const int* te = Tr->same ? Tr->se.p : Tr->te.p;
     const int nt_opt = Tr->ctx->leaf_nt;
     if constexpr (std::is_same<T, float>::value) {
-        if (Tr->ctx->leaf_packed && O.ne <= 1024) {
+        if (L) {
             const int NT = nt_opt ? nt_opt : (DN ? 2 : 4);
             auto k = split > 1 ? (NT == 4 ? k_leaf_pair_x2<DL, DN, 4, PART, 3, true> : k_leaf_pair_x2<DL, DN, 2, PART, 3, true>)
                                : (NT == 4 ? k_leaf_pair_x2<DL, DN, 4, PART, 3, false> : k_leaf_pair_x2<DL, DN, 2, PART, 3, false>);
-            const LeafStream& L = leaf_stream(Tr, thrW, thrX);
-            k<<<dim3(Tr->n_tleaf, split), 128, 0, st>>>(L.rec.p, L.near.p, L.far_geo.p, L.far_box.p, tpos, WL.sq.p,
+            k<<<dim3(Tr->n_tleaf, split), 128, 0, st>>>(L->rec.p, L->near.p, L->far_geo.p, L->far_box.p, tpos, WL.sq.p,
                                                         WL.sm.p, WL.Qu.p, WL.Qd.p, WY.Qu.p, WY.Qd.p,
                                                         (const float4*)O.surf_f.p, O.ne, O.npad, kappa, WL.pot.p,
                                                         WY.pot.p, WL.tn.p, WL.dn.p, WY.dn.p,
@@ -2091,7 +2098,6 @@ static void launch_leaf_pair(cudaStream_t st, fmm_tree* Tr, Work<T>& WL, Work<T>
             return;
         }
     }
-    PB_REQUIRE(thrW < 0 && thrX < 0, PB_EINVAL, "direct W/X-list evaluation needs the packed leaf kernel");
     const int NT = nt_opt ? nt_opt : (sizeof(T) == 4 ? 4 : 2);
     auto k = NT == 4 ? k_leaf_pair<T, DL, DN, 4, PART> : k_leaf_pair<T, DL, DN, 2, PART>;
     k<<<dim3(Tr->n_tleaf, split), 128, 0, st>>>(
@@ -2126,6 +2132,7 @@ static void apply_pair_t(fmm_tree* Tr, const Operators& OL, const Operators& OY,
     if (DL && DN) throw Error(PB_EINVAL, "double layer with target-normal derivative is not provided");
     int thrW, thrX;
     list_direct(Tr, OL, std::is_same<T, float>::value, thrW, thrX);
+    const LeafStream* L = leaf_streams_for<T>(Tr, OL, thrW, thrX);
     Work<T> WL, WY;
     WL.sq.alloc(ns, st);
     WL.sm.alloc(ns, st);
@@ -2152,9 +2159,9 @@ static void apply_pair_t(fmm_tree* Tr, const Operators& OL, const Operators& OY,
         PB_CUDA(cudaStreamWaitEvent(ctx->aux, ctx->ev_fork, 0));
         {
             PhaseTimer phn(ctx, PB_PH_LEAF, ctx->aux);
-            if (DL) launch_leaf_pair<T, true, false, 1>(ctx->aux, Tr, WL, WY, OL, kappa, thrW, thrX, split);
-            else if (DN) launch_leaf_pair<T, false, true, 1>(ctx->aux, Tr, WL, WY, OL, kappa, thrW, thrX, split);
-            else launch_leaf_pair<T, false, false, 1>(ctx->aux, Tr, WL, WY, OL, kappa, thrW, thrX, split);
+            if (DL) launch_leaf_pair<T, true, false, 1>(ctx->aux, Tr, WL, WY, OL, kappa, L, split);
+            else if (DN) launch_leaf_pair<T, false, true, 1>(ctx->aux, Tr, WL, WY, OL, kappa, L, split);
+            else launch_leaf_pair<T, false, false, 1>(ctx->aux, Tr, WL, WY, OL, kappa, L, split);
         }
         PB_CUDA(cudaEventRecord(ctx->ev_join, ctx->aux));
     }
@@ -2185,13 +2192,13 @@ static void apply_pair_t(fmm_tree* Tr, const Operators& OL, const Operators& OY,
     if (fork) PB_CUDA(cudaStreamWaitEvent(st, ctx->ev_join, 0));
     ph.reset(); ph = std::make_unique<PhaseTimer>(ctx, PB_PH_LEAF);
     if (fork) {
-        if (DL) launch_leaf_pair<T, true, false, 2>(st, Tr, WL, WY, OL, kappa, thrW, thrX, split);
-        else if (DN) launch_leaf_pair<T, false, true, 2>(st, Tr, WL, WY, OL, kappa, thrW, thrX, split);
-        else launch_leaf_pair<T, false, false, 2>(st, Tr, WL, WY, OL, kappa, thrW, thrX, split);
+        if (DL) launch_leaf_pair<T, true, false, 2>(st, Tr, WL, WY, OL, kappa, L, split);
+        else if (DN) launch_leaf_pair<T, false, true, 2>(st, Tr, WL, WY, OL, kappa, L, split);
+        else launch_leaf_pair<T, false, false, 2>(st, Tr, WL, WY, OL, kappa, L, split);
     } else {
-        if (DL) launch_leaf_pair<T, true, false, 0>(st, Tr, WL, WY, OL, kappa, thrW, thrX, split);
-        else if (DN) launch_leaf_pair<T, false, true, 0>(st, Tr, WL, WY, OL, kappa, thrW, thrX, split);
-        else launch_leaf_pair<T, false, false, 0>(st, Tr, WL, WY, OL, kappa, thrW, thrX, split);
+        if (DL) launch_leaf_pair<T, true, false, 0>(st, Tr, WL, WY, OL, kappa, L, split);
+        else if (DN) launch_leaf_pair<T, false, true, 0>(st, Tr, WL, WY, OL, kappa, L, split);
+        else launch_leaf_pair<T, false, false, 0>(st, Tr, WL, WY, OL, kappa, L, split);
     }
     ph.reset(); ph = std::make_unique<PhaseTimer>(ctx, PB_PH_SCATTER);
     const int* pt = Tr->same ? Tr->perm_s.p : Tr->perm_t.p;
