@@ -2121,6 +2121,29 @@ static void list_direct(const fmm_tree* Tr, const Operators& O, bool fp32, int& 
     thrX = on && mode != 3 ? O.ne : -1;
 }
 
+// Fork of the context's second stream.  The main stream waits for the second
+// one in join(), or on the way out of a failed call: the call's buffers are
+// given back on the main stream, and the second one's kernels still use them.
+struct AuxFork {
+    pb_ctx* ctx;
+    bool open = false;
+    explicit AuxFork(pb_ctx* c) : ctx(c) {}
+    void fork() {
+        PB_CUDA(cudaEventRecord(ctx->ev_fork, ctx->stream));
+        PB_CUDA(cudaStreamWaitEvent(ctx->aux, ctx->ev_fork, 0));
+        open = true;
+    }
+    void done() { PB_CUDA(cudaEventRecord(ctx->ev_join, ctx->aux)); }
+    void join() {
+        PB_CUDA(cudaStreamWaitEvent(ctx->stream, ctx->ev_join, 0));
+        open = false;
+    }
+    ~AuxFork() {
+        if (open && cudaEventRecord(ctx->ev_join, ctx->aux) == cudaSuccess)
+            cudaStreamWaitEvent(ctx->stream, ctx->ev_join, 0);
+    }
+};
+
 template <typename T, typename In>
 static void apply_pair_t(fmm_tree* Tr, const Operators& OL, const Operators& OY, double kappa_d, const In* qL,
                          const In* qY, const In* dip, const In* src_n, const In* tgt_n, In* outL, In* outY,
@@ -2154,16 +2177,16 @@ static void apply_pair_t(fmm_tree* Tr, const Operators& OL, const Operators& OY,
     // the near field needs only the gathered sources: on the second stream,
     // beside the far-field passes below (joined before the far leaf part)
     const bool fork = ctx->aux && ctx->overlap && Tr->n_tleaf > 0;
+    AuxFork near(ctx);                   // (after the buffers: their release follows the join)
     if (fork) {
-        PB_CUDA(cudaEventRecord(ctx->ev_fork, st));
-        PB_CUDA(cudaStreamWaitEvent(ctx->aux, ctx->ev_fork, 0));
+        near.fork();
         {
             PhaseTimer phn(ctx, PB_PH_LEAF, ctx->aux);
             if (DL) launch_leaf_pair<T, true, false, 1>(ctx->aux, Tr, WL, WY, OL, kappa, L, split);
             else if (DN) launch_leaf_pair<T, false, true, 1>(ctx->aux, Tr, WL, WY, OL, kappa, L, split);
             else launch_leaf_pair<T, false, false, 1>(ctx->aux, Tr, WL, WY, OL, kappa, L, split);
         }
-        PB_CUDA(cudaEventRecord(ctx->ev_join, ctx->aux));
+        near.done();
     }
     const int nsl = Tr->sleaf_lvl_off[Tr->nlev];
     ph.reset(); ph = std::make_unique<PhaseTimer>(ctx, PB_PH_P2M);
@@ -2189,7 +2212,7 @@ static void apply_pair_t(fmm_tree* Tr, const Operators& OL, const Operators& OY,
     far_pair_m2l(Tr, OL, OY, WL, WY);
     ph.reset(); ph = std::make_unique<PhaseTimer>(ctx, PB_PH_DOWN);
     far_pair_l2l(Tr, OL, OY, WL, WY);
-    if (fork) PB_CUDA(cudaStreamWaitEvent(st, ctx->ev_join, 0));
+    if (fork) near.join();
     ph.reset(); ph = std::make_unique<PhaseTimer>(ctx, PB_PH_LEAF);
     if (fork) {
         if (DL) launch_leaf_pair<T, true, false, 2>(st, Tr, WL, WY, OL, kappa, L, split);

@@ -64,3 +64,54 @@ def test_first_apply_on_two_streams(n, ncrit, options, layer):
         for k, (o, s, r) in enumerate(zip(out, one[0], want)):
             assert rel_l2(o[idx], r) < (1e-5 if k < 2 else 1e-4), k
             assert rel_l2(o, s) < 1e-6, k
+
+
+def test_failed_apply_on_two_streams():
+    """An allocation that fails while the second stream runs: PB_ENOMEM,
+    and the next apply (which takes the returned memory) is right."""
+    import paper_2103_01048_gb300 as pb
+    rng = np.random.default_rng(41)         # a cluster in a cloud: X lists, hence allocations after the fork
+    x = np.concatenate([rng.normal(0.2, 0.02, (6000, 3)), rng.uniform(-1, 1, (6000, 3))]).astype(np.float32)
+    n = len(x)
+    q = synthetic.uniform_densities(n, seed=13)
+    X, Q = dev(x), dev(q)
+    idx = synthetic.random_subsample(n, 300, seed=15)
+    want = [direct_sum(kern, kap, x, q=q, tgt=x[idx]) for kern, kap in ((LAPLACE, 0.0), (YUKAWA, KAPPA))]
+    ctx = pb.pb_create(0, torch.cuda.Stream())
+    try:
+        pb.pb_set_option(ctx, pb.PB_OPT_OVERLAP, 1)
+
+        def run(tree):
+            o = [torch.zeros(n, device="cuda") for _ in range(2)]
+            torch.cuda.synchronize()
+            pb.fmm_apply_pair(ctx, tree, KAPPA, 6, o[0], o[1], q_lap=Q, q_yuk=Q)
+            pb.pb_sync(ctx)
+            return [a.cpu().numpy() for a in o]
+
+        keep = pb.fmm_tree_build(ctx, X, 24)     # holds the operators: the fresh trees allocate lists and workspace only
+        run(keep)
+        failed = 0
+        for nth in range(1, 60):
+            tree = pb.fmm_tree_build(ctx, X, 24)
+            try:
+                pb._test_fail_alloc(nth)
+                try:
+                    out = run(tree)
+                except pb.PBError as e:
+                    assert e.code == pb.PB_ENOMEM
+                    failed += 1
+                    out = None
+                finally:
+                    pb._test_fail_alloc(0)
+                done = out is not None
+                out = out or run(tree)
+                for o, r in zip(out, want):
+                    assert rel_l2(o[idx], r) < 1e-5
+            finally:
+                pb.fmm_tree_destroy(tree)
+            if done:
+                break
+        assert done and failed >= 10
+        pb.fmm_tree_destroy(keep)
+    finally:
+        pb.pb_destroy(ctx)
