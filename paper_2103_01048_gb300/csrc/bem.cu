@@ -899,14 +899,16 @@ static void reaction_potential(pb_mesh* M, pb_result* R, double* phir) {
 // caller launches the kernels itself.
 static bool matvec_graph(pb_mesh* M, pb_result* R) {
     pb_ctx* ctx = M->ctx;
-    const double key[9] = {R->eps_in, R->eps_out, R->kappa, (double)R->precision,
-                           (double)(ctx->deterministic + 2 * ctx->overlap), (double)ctx->singular,
-                           (double)(uintptr_t)M->S_d.p, (double)(uintptr_t)M->D1.p, (double)R->formulation};
-    const bool same = std::equal(key, key + 9, M->mv_key);
+    // every option that selects a kernel or a list of the mat-vec is in the key
+    const double key[pb_mesh::kMvKey] = {
+        R->eps_in, R->eps_out, R->kappa, (double)R->precision, (double)(ctx->deterministic + 2 * ctx->overlap),
+        (double)ctx->singular, (double)(uintptr_t)M->S_d.p, (double)(uintptr_t)M->D1.p, (double)R->formulation,
+        (double)ctx->leaf_nt, (double)ctx->leaf_packed, (double)ctx->list_direct};
+    const bool same = std::equal(key, key + pb_mesh::kMvKey, M->mv_key);
     if (same && M->mv_exec) return true;
     if (!same || !M->mv_warm) {
         // first solve with these parameters: run uncaptured, capture next time
-        std::copy(key, key + 9, M->mv_key);
+        std::copy(key, key + pb_mesh::kMvKey, M->mv_key);
         M->mv_warm = false;
         if (M->mv_exec) { cudaGraphExecDestroy(M->mv_exec); M->mv_exec = nullptr; }
         if (M->mv_graph) { cudaGraphDestroy(M->mv_graph); M->mv_graph = nullptr; }

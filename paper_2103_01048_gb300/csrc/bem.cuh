@@ -41,7 +41,8 @@ struct pb_mesh {
     cudaGraph_t mv_graph = nullptr;
     cudaGraphExec_t mv_exec = nullptr;
     pbfmm::DBuf<double> mv_in, mv_out;
-    double mv_key[9] = {};
+    static constexpr int kMvKey = 12;
+    double mv_key[kMvKey] = {};
     bool mv_warm = false;             // one uncaptured mat-vec ran with mv_key (caches filled)
     ~pb_mesh() {
         if (mv_exec) cudaGraphExecDestroy(mv_exec);
