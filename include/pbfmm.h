@@ -271,9 +271,14 @@ int fmm_tree_export_list(const fmm_tree* tree, int which, int64_t* off, int32_t*
  * Buffers may be host or device memory (see conventions).  With device
  * buffers the call is asynchronous; with any host buffer it synchronises.
  * Operators for (kernel, kappa, p, tree size) are precomputed on first use
- * and cached in the tree.  With PB_MIXED and p in 2..6, 8 or 10 the M2L,
- * M2M, L2L and the check -> equivalent solves run on the tensor cores (FP32
- * operands split into hi + lo parts, scaled halves for the M2L and TF32 for
+ * and cached in the tree, as are the lists that an order and the options
+ * PB_OPT_LIST_DIRECT and PB_OPT_DETERMINISTIC need.  A first apply may be
+ * captured into a CUDA graph where the context already holds the operators
+ * (another tree with the same box sizes used them) and the tree has no X
+ * lists or takes none directly (PB_OPT_LIST_DIRECT 0 or 3); any other first
+ * apply waits for the stream and cannot be captured.  With PB_MIXED and p
+ * in 2..6, 8 or 10 the M2L, M2M, L2L and the check -> equivalent solves run
+ * on the tensor cores (FP32 operands split into hi + lo parts, scaled halves for the M2L and TF32 for
  * the others, three products per step; at p = 8 and 10 each operator is
  * split into parts that fit in shared memory); with p = 7 or 9
  * or PB_FP64 on the CUDA cores, the

@@ -113,6 +113,30 @@ struct DBuf {
     }
 };
 
+// A stream of its own for work that a captured call needs done before the
+// graph runs (lists that a tree keeps): not part of the caller's capture, and
+// waited for by the host alone.  The capture mode is relaxed meanwhile, as a
+// capturing thread may not wait for any stream otherwise.
+struct SideStream {
+    cudaStream_t s = nullptr;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    SideStream() {
+        PB_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+        const cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+        if (e != cudaSuccess) {
+            cudaThreadExchangeStreamCaptureMode(&mode);
+            PB_CUDA(e);
+        }
+    }
+    SideStream(const SideStream&) = delete;
+    SideStream& operator=(const SideStream&) = delete;
+    ~SideStream() {
+        cudaStreamSynchronize(s);
+        cudaStreamDestroy(s);
+        cudaThreadExchangeStreamCaptureMode(&mode);
+    }
+};
+
 inline int div_up(long long a, long long b) { return (int)((a + b - 1) / b); }
 
 }  // namespace pbfmm

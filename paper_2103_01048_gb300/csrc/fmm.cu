@@ -1242,18 +1242,26 @@ static const LeafStream& leaf_stream(fmm_tree* T, int thrW, int thrX) {
     cudaStream_t st = T->ctx->stream;
     cudaStreamCaptureStatus cap;
     PB_CUDA(cudaStreamIsCapturing(st, &cap));
-    PB_REQUIRE(cap == cudaStreamCaptureStatusNone, PB_EINVAL, "leaf lists are not built yet (first apply is captured)");
+    // inside a capture on a stream of its own: the tree keeps the lists, a
+    // graph would only build them when it runs
+    std::unique_ptr<SideStream> side;
+    if (cap != cudaStreamCaptureStatusNone) side = std::make_unique<SideStream>();
+    cudaStream_t bs = side ? side->s : st;
     auto L = std::make_unique<LeafStream>();
     const int n = T->n_tleaf;
-    L->rec.alloc(n, st);
-    L->near.alloc(T->n_u + T->n_w + (long long)kXCap * n, st);
-    L->far_geo.alloc(T->n_w + n, st);
-    L->far_box.alloc(T->n_w + n, st);
-    k_leaf_stream<<<div_up(n, 4), 128, 0, st>>>(n, T->leaf_ids.p, T->same ? T->sb.p : T->tb.p,
+    L->rec.alloc(n, bs);
+    L->near.alloc(T->n_u + T->n_w + (long long)kXCap * n, bs);
+    L->far_geo.alloc(T->n_w + n, bs);
+    L->far_box.alloc(T->n_w + n, bs);
+    k_leaf_stream<<<div_up(n, 4), 128, 0, bs>>>(n, T->leaf_ids.p, T->same ? T->sb.p : T->tb.p,
                                                 T->same ? T->se.p : T->te.p, T->sb.p, T->se.p, T->U_off.p, T->U_ids.p,
                                                 T->W_off.p, T->W_ids.p, T->X.p, T->X_n.p, T->level.p, T->center.p, thrW,
                                                 thrX, L->rec.p, L->near.p, L->far_geo.p, L->far_box.p);
     PB_CHECK_LAUNCH();
+    if (side) {
+        PB_CUDA(cudaStreamSynchronize(bs));
+        L->rec.s = L->near.s = L->far_geo.s = L->far_box.s = st;      // given back on the context stream
+    }
     p = std::move(L);
     return *p;
 }

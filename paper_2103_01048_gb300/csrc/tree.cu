@@ -407,10 +407,19 @@ static T read1(const T* d, cudaStream_t st) {
 
 // M2L tile schedule: boxes with a non-empty V list, per level, tiles of
 // kM2LTile.  Only the fixed-order M2L of PB_OPT_DETERMINISTIC uses it: built
-// at its first apply on the tree (0.4 of the 2.3 ms of a 120,000-point build).
+// at its first apply on the tree (0.4 of the 2.3 ms of a 120,000-point build),
+// on a stream of its own, so that the apply waits for nothing the caller has
+// enqueued and may be captured.
 void build_m2l_schedule(fmm_tree* T) {
     if (T->m2l_built) return;
-    cudaStream_t st = T->ctx->stream;
+    SideStream side;
+    M2LSchedule& S = T->m2l;
+    struct Rehome {                      // the buffers are given back on the context stream
+        M2LSchedule& S;
+        cudaStream_t st;
+        ~Rehome() { S.tile_box.s = S.tile_level.s = S.entry_off.s = S.entry_offset_idx.s = S.entry_src.s = st; }
+    } rehome{S, T->ctx->stream};
+    cudaStream_t st = side.s;
     const int nb = T->nbox;
     std::vector<int> vn(nb);
     PB_CUDA(cudaMemcpyAsync(vn.data(), T->V_n.p, nb * sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -426,7 +435,6 @@ void build_m2l_schedule(fmm_tree* T) {
             tlev.push_back(l);
         }
     }
-    M2LSchedule& S = T->m2l;
     S.ntile = (int)tlev.size();
     S.tile_level_h = tlev;
     S.npairs = T->n_v;
