@@ -533,7 +533,7 @@ __global__ void __launch_bounds__(kHThreads, 1) k_m2l_f16(const HArgs A) {
         // the whole warp runs the loop, one elected lane issues: the operands
         // of tcgen05.mma stay in uniform registers (84 against 91 cycles per
         // MMA at N = 160, 72 against 91 at N = 64, measured alone)
-        uint64_t* last = nullptr;
+        uint64_t* last = nullptr;      // barrier of the last commit, and its phase parity
         uint32_t last_par = 0;
         int s = 0, nload = 0;
         uint32_t par = 0;
@@ -583,12 +583,16 @@ __global__ void __launch_bounds__(kHThreads, 1) k_m2l_f16(const HArgs A) {
                 last_par = par;
                 if (++s == STAGES) { s = 0; par ^= 1; }
             }
+            if (ok) {
+                last = &S->accf[a];
+                last_par = (k >> 1) & 1;
+            }
         }
-        // on a failure every MMA and operator copy issued here ends before the CTA's memory is given up
-        if (!ok) {
-            if (last) mbar_wait(last, last_par);
-            if (nload) mbar_wait(&S->barB, (nload - 1) & 1);
-        }
+        // every MMA and operator copy issued here ends before TMEM is freed
+        // and the CTA's shared memory given up, whichever role gave up
+        // waiting: an epilogue that timed out leaves the last ones in flight
+        if (last) mbar_wait(last, last_par);
+        if (nload) mbar_wait(&S->barB, (nload - 1) & 1);
     }
     __syncwarp();
     tc_fence_before();

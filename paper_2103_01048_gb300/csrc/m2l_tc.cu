@@ -556,8 +556,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_m2l_tc(const int4* __restrict
                 last = &S->accf[a];
                 last_par = u & 1;
             }
-            // after a failure: every MMA issued here has completed before TMEM is freed
-            if (!ok && last) mbar_wait(last, last_par);
+            // every MMA issued here has completed before TMEM is freed and the
+            // CTA's shared memory given up, whichever role gave up waiting: an
+            // epilogue that timed out leaves the last ones in flight
+            if (last) mbar_wait(last, last_par);
         }
         __syncwarp();
     }
