@@ -1147,6 +1147,7 @@ __device__ __forceinline__ void put_src_x2(ulonglong2* sA, ulonglong2* sB, ulong
 // were seven dependent loads and a scan over every entry, 0.76 of 4.0 ms at
 // 4M points, p = 6.  Kept until the tree goes: captured graphs point to them.
 // ---------------------------------------------------------------------------
+static_assert(sizeof(LeafStream::Rec::near_off) == 8, "kXCap entries a leaf pass 2^31 at 74 million leaves on a curve");
 __global__ void __launch_bounds__(128) k_leaf_stream(
     int nleaf, const int* __restrict__ leaves, const int* __restrict__ tb, const int* __restrict__ te,
     const int* __restrict__ sb, const int* __restrict__ se, const int* __restrict__ U_off, const int* __restrict__ U_ids,
@@ -1161,7 +1162,8 @@ __global__ void __launch_bounds__(128) k_leaf_stream(
     const int u0 = U_off[b], w0 = W_off[b], nu = U_off[b + 1] - u0, nw = W_off[b + 1] - w0;
     const int s_own = sb[b], nself = se[b] - s_own, t0 = tb[b], t1 = te[b];
     const int nx = thrX >= 0 && t1 - t0 <= thrX ? Xn[b] : 0;
-    const int near_off = u0 + w0 + kXCap * li, far_off = w0 + li;       // room for every list entry
+    const long long near_off = (long long)u0 + w0 + (long long)kXCap * li;       // room for every list entry
+    const int far_off = w0 + li;
     int2* nl = near_l + near_off;
     int n = 0, nf = 0;                                   // ranges and far boxes written
     if (nself > 0) {
@@ -1230,7 +1232,6 @@ __global__ void __launch_bounds__(128) k_leaf_stream(
         r.t0 = t0; r.t1 = t1; r.nself = nself;
         r.near_off = near_off; r.near_n = n;
         r.far_off = far_off; r.far_n = nf;
-        r.pad = 0;
         r.cx = cb.x; r.cy = cb.y; r.cz = cb.z;
         recs[li] = r;
     }

@@ -58,9 +58,9 @@ struct LeafStream {
     struct Rec {
         int t0, t1;                // targets
         int nself;                 // the leaf's own sources (its first near range; 0: no such range)
-        int near_off, near_n;      // near: (first source, count)
+        int near_n;                // near: (first source, count)
+        long long near_off;        // (room for kXCap X entries a leaf: past 2^31 before the box count is)
         int far_off, far_n;
-        int pad;
         double cx, cy, cz;         // centre of the leaf
     };
     DBuf<Rec> rec;
