@@ -175,7 +175,7 @@ struct BatchSystem {
 
 static void batch_dots(BatchSystem& S, const double* Vb, int nk, const double* vec, double* out, int acc) {
     cudaStream_t st = S.sub.stream;
-    k_dots<<<S.nb, 256, 0, st>>>(S.n, Vb, S.n, nk, vec, S.partial.p, S.kmax + 1);
+    k_dots<<<S.nb, kDotThreads, 0, st>>>(S.n, Vb, S.n, nk, vec, S.partial.p, S.kmax + 1);
     PB_CHECK_LAUNCH();
     k_dots_reduce<<<div_up(nk, 4), 128, 0, st>>>(S.nb, nk, S.partial.p, S.kmax + 1, out, acc, nullptr);
     PB_CHECK_LAUNCH();
@@ -331,14 +331,14 @@ void solve_batch(pb_ctx* ctx, pb_mesh* const* meshes, int nsys, pb_result** resu
                             R->formulation);
                 for (int pass = 0; pass < 2; ++pass) {       // CGS2
                     double* hp = pass == 0 ? S.h.p : S.h2.p;
-                    k_b_dots<<<S.nb, 256, 0, st>>>(S.n, S.V.p, S.n, S.xout.p, S.partial.p, S.kmax + 1, S.dev.p, 1);
+                    k_b_dots<<<S.nb, kDotThreads, 0, st>>>(S.n, S.V.p, S.n, S.xout.p, S.partial.p, S.kmax + 1, S.dev.p, 1);
                     k_b_dots_reduce<<<div_up(S.kmax + 1, 4), 128, 0, st>>>(S.nb, S.partial.p, S.kmax + 1, hp, S.dev.p, 1);
                     k_b_update<<<S.ub, 256, (S.kmax + 1) * sizeof(double), st>>>(S.n, S.V.p, S.n, hp, S.xout.p,
                                                                                 S.dev.p);
                     PB_CHECK_LAUNCH();
                 }
                 k_b_vadd<<<1, 256, 0, st>>>(S.h2.p, S.h.p, S.dev.p);
-                k_b_dots<<<S.nb, 256, 0, st>>>(S.n, S.xout.p, S.n, S.xout.p, S.partial.p, S.kmax + 1, S.dev.p, 0);
+                k_b_dots<<<S.nb, kDotThreads, 0, st>>>(S.n, S.xout.p, S.n, S.xout.p, S.partial.p, S.kmax + 1, S.dev.p, 0);
                 k_b_dots_reduce<<<1, 128, 0, st>>>(S.nb, S.partial.p, S.kmax + 1, S.nrm2.p, S.dev.p, 0);
                 k_b_givens<<<1, 1, 0, st>>>(S.kmax, S.h.p, S.nrm2.p, S.H.p, S.cs.p, S.sn.p, S.g.p, S.beta, tol,
                                             S.dev.p);

@@ -413,7 +413,7 @@ __global__ void k_energy(int na, const double4* __restrict__ atoms, const double
 constexpr int kDotBlocks = 304;
 
 // partial[blk][k] = sum over the block's rows of V[k][i] w[i], k < nk
-__global__ void __launch_bounds__(256) k_dots(long long n, const double* __restrict__ V, long long ld, int nk,
+__global__ void __launch_bounds__(kDotThreads) k_dots(long long n, const double* __restrict__ V, long long ld, int nk,
                                               const double* __restrict__ w, double* __restrict__ partial, int kmax) {
     long long i0, i1;
     block_rows(n, i0, i1);
@@ -435,7 +435,7 @@ __global__ void k_dots_reduce(int nblk, int nk, const double* __restrict__ parti
 
 // w -= sum_k h[k] V[k] on the block's rows, then the partial dots of the new
 // w with the basis (self = 0: second Gram-Schmidt pass) or with itself (1)
-__global__ void __launch_bounds__(256) k_update_dots(long long n, const double* __restrict__ V, long long ld, int nk,
+__global__ void __launch_bounds__(kDotThreads) k_update_dots(long long n, const double* __restrict__ V, long long ld, int nk,
                                                      const double* __restrict__ h, double* w,
                                                      double* __restrict__ partial, int kmax, int self) {
     extern __shared__ double sh[];
@@ -729,7 +729,7 @@ int gmres(pb_mesh* M, const std::function<void(const double*, double*)>& matvec,
     };
     const int ub = std::min<long long>(4 * M->ctx->sm_count, (n + 255) / 256);
     // r0 = P^{-1} b (b is already preconditioned), beta = ||r0||
-    k_dots<<<nb, 256, 0, st>>>(n, b, n, 1, b, partial.p, kmax + 1);
+    k_dots<<<nb, kDotThreads, 0, st>>>(n, b, n, 1, b, partial.p, kmax + 1);
     PB_CHECK_LAUNCH();
     reduce(1, nrm2.p, nullptr);
     double beta = std::sqrt(read_scalar(nrm2.p, st));
@@ -746,13 +746,13 @@ int gmres(pb_mesh* M, const std::function<void(const double*, double*)>& matvec,
         // CGS2: two passes of classical Gram-Schmidt, each update fused with
         // the products that follow it
         const size_t sm = (j + 1) * sizeof(double);
-        k_dots<<<nb, 256, 0, st>>>(n, V.p, n, j + 1, w.p, partial.p, kmax + 1);
+        k_dots<<<nb, kDotThreads, 0, st>>>(n, V.p, n, j + 1, w.p, partial.p, kmax + 1);
         PB_CHECK_LAUNCH();
         reduce(j + 1, h.p, nullptr);
-        k_update_dots<<<nb, 256, sm, st>>>(n, V.p, n, j + 1, h.p, w.p, partial.p, kmax + 1, 0);
+        k_update_dots<<<nb, kDotThreads, sm, st>>>(n, V.p, n, j + 1, h.p, w.p, partial.p, kmax + 1, 0);
         PB_CHECK_LAUNCH();
         reduce(j + 1, h2.p, h.p);
-        k_update_dots<<<nb, 256, sm, st>>>(n, V.p, n, j + 1, h2.p, w.p, partial.p, kmax + 1, 1);
+        k_update_dots<<<nb, kDotThreads, sm, st>>>(n, V.p, n, j + 1, h2.p, w.p, partial.p, kmax + 1, 1);
         PB_CHECK_LAUNCH();
         k_norm_givens<<<1, 128, 3 * (j + 2) * sizeof(double), st>>>(nb, partial.p, j, kmax, h.p, nrm2.p, H.p, cs.p, sn.p,
                                                                      g.p, resid.p);

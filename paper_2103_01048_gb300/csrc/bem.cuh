@@ -52,34 +52,74 @@ struct pb_mesh {
 
 namespace pbfmm {
 // ---- Gram-Schmidt products of the GMRES kernels (bem.cu, batch.cu)
-// partial[k] = sum over the rows [i0, i1) of V[k][i] w[i], k < nk: one warp per
-// four vectors (one read of w for four products), no block barrier.  The
-// basis is read once per pass; at the sizes of a solve it stays in L2 and the
-// pass is bound by its latency (a barrier tree per vector took 1.5 us each).
+constexpr int kDotThreads = 256;
+
+// s[u] += sum over i = i0, i0 + step, ... < i1 of V[u][i] w[i], M vectors
+template <int M>
+__device__ __forceinline__ void dot_rows(long long i0, long long i1, int step, const double* v, long long ld,
+                                         const double* w, double* s) {
+#pragma unroll 4
+    for (long long i = i0; i < i1; i += step) {
+        const double x = w[i];
+#pragma unroll
+        for (int u = 0; u < M; ++u) s[u] += v[u * ld + i] * x;
+    }
+}
+
+// the products of group g (vectors 4 g ...) with w by a warp, in every lane
+__device__ __forceinline__ void dot_group(long long a, long long i1, int step, const double* V, long long ld, int nk,
+                                          int g, const double* w, double* s) {
+    const double* v = V + (long long)(4 * g) * ld;
+    switch (min(4, nk - 4 * g)) {
+        case 4: dot_rows<4>(a, i1, step, v, ld, w, s); break;
+        case 3: dot_rows<3>(a, i1, step, v, ld, w, s); break;
+        case 2: dot_rows<2>(a, i1, step, v, ld, w, s); break;
+        default: dot_rows<1>(a, i1, step, v, ld, w, s); break;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+        for (int o = 16; o > 0; o >>= 1) s[u] += __shfl_xor_sync(0xffffffffu, s[u], o);
+}
+
+// partial[k] = sum over the rows [i0, i1) of V[k][i] w[i], k < nk: a warp
+// takes four vectors (one read of w for four products).  With fewer groups of
+// four than warps the rows are dealt out to the idle ones and their sums
+// added in order (one barrier; every thread of a block of kDotThreads calls).
+// A pass is bound by its latency at some 1,000 triangles (a barrier tree per
+// vector took 1.5 us each) and by the loads in flight at a million: with one
+// warp for up to four vectors, the GMRES part of 1 / 4 / 12 / 40 iterations on
+// 1,310,720 triangles took 0.30 / 1.91 / 7.8 / 37.0 ms, so 0.11 / 0.63 / 3.4 /
+// 25.8 (81,920 triangles, 12 iterations: 1.09 and 0.92; 5,120: 0.68 both).
 __device__ __forceinline__ void block_dots(long long i0, long long i1, const double* V, long long ld,
                                            int nk, const double* w, double* __restrict__ partial) {
-    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int k0 = (threadIdx.x >> 5) * 4; k0 < nk; k0 += nw * 4) {
+    constexpr int NW = kDotThreads / 32;
+    __shared__ double red[NW][4];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int ng = (nk + 3) >> 2;
+    if (2 * ng > NW) {
+        for (int g = warp; g < ng; g += NW) {
+            double s[4] = {0.0, 0.0, 0.0, 0.0};
+            dot_group(i0 + lane, i1, 32, V, ld, nk, g, w, s);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (lane == 0 && 4 * g + u < nk) partial[4 * g + u] = s[u];
+        }
+        return;
+    }
+    const int ns = NW / ng, r = warp / ng, g = warp - r * ng;      // shares of the rows, this warp's share and group
+    if (r < ns) {
         double s[4] = {0.0, 0.0, 0.0, 0.0};
-        const int m = min(4, nk - k0);
-        const double* v = V + (long long)k0 * ld;
-        if (m == 4) {
-            for (long long i = i0 + lane; i < i1; i += 32) {
-                const double x = w[i];
+        dot_group(i0 + 32 * r + lane, i1, 32 * ns, V, ld, nk, g, w, s);
+        if (lane == 0) {
 #pragma unroll
-                for (int u = 0; u < 4; ++u) s[u] += v[u * ld + i] * x;
-            }
-        } else {
-            for (long long i = i0 + lane; i < i1; i += 32) {
-                const double x = w[i];
-                for (int u = 0; u < m; ++u) s[u] += v[u * ld + i] * x;
-            }
+            for (int u = 0; u < 4; ++u) red[warp][u] = s[u];
         }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            for (int o = 16; o > 0; o >>= 1) s[u] += __shfl_xor_sync(0xffffffffu, s[u], o);
-            if (lane == 0 && u < m) partial[k0 + u] = s[u];
-        }
+    }
+    __syncthreads();
+    if (threadIdx.x < nk) {
+        double s = 0.0;
+        for (int k = 0; k < ns; ++k) s += red[k * ng + (threadIdx.x >> 2)][threadIdx.x & 3];
+        partial[threadIdx.x] = s;
     }
 }
 __device__ __forceinline__ void block_rows(long long n, long long& i0, long long& i1) {
