@@ -53,6 +53,15 @@ struct PCPairs {
     int nitems = 0;
 };
 
+// X-list boxes that keep P2L at a direct-list threshold, with the items of
+// their check -> equivalent solve (built in m2l_tc.cu)
+struct XFar {
+    DBuf<int> ids;
+    int n = 0;
+    DBuf<int4> items;
+    int nitems = 0;
+};
+
 // Source streams of the packed leaf kernel (built in fmm.cu)
 struct LeafStream {
     struct Rec {
@@ -114,13 +123,10 @@ struct fmm_tree {
     pbfmm::DBuf<int4> c2e_items_up, c2e_items_dn;
     int n_c2e_up = 0, n_c2e_dn = 0;
     // X-list boxes whose X lists the leaf kernel does not sum directly (it
-    // does for leaves of at most xfar_thr targets): P2L and its solve run on
-    // these only.  Built on first use for a threshold (-1: not built).
-    int xfar_thr = -1;
-    pbfmm::DBuf<int> xfar_ids;
-    int n_xfar = 0;
-    pbfmm::DBuf<int4> c2e_items_xfar;
-    int n_c2e_xfar = 0;
+    // does for leaves of at most so many targets, the key): P2L and its solve
+    // run on these only.  Built on first use of a threshold (one an expansion
+    // order) and kept until the tree goes: captured graphs point to them.
+    std::map<int, std::unique_ptr<pbfmm::XFar>> xfar;
 
     // by (W threshold, X threshold): at most four combinations of options per expansion order
     std::map<std::pair<int, int>, std::unique_ptr<pbfmm::LeafStream>> leaf_streams;

@@ -76,3 +76,51 @@ def test_first_apply_captured(options, dn):
         pb.fmm_tree_destroy(first)
     finally:
         pb.pb_destroy(ctx)
+
+
+def test_replay_after_other_orders():
+    """A captured apply at p = 6 on a tree with X lists, replayed after the tree
+    has been used at other orders (which take other lists) and memory has
+    changed hands."""
+    import paper_2103_01048_gb300 as pb
+    rng = np.random.default_rng(8)
+    x = np.concatenate([rng.normal(0.2, 0.02, (4000, 3)), rng.uniform(-1, 1, (4000, 3))]).astype(np.float32)
+    n = len(x)
+    q = synthetic.uniform_densities(n, seed=9)
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    X, Q = dev(x), dev(q)
+    want = [direct_sum(kern, kap, x, q=q) for kern, kap in ((LAPLACE, 0.0), (YUKAWA, KAPPA))]
+    stream = torch.cuda.Stream()
+    ctx = pb.pb_create(0, stream)
+    try:
+        o = [torch.zeros(n, device="cuda") for _ in range(2)]
+        torch.cuda.synchronize()
+        tree = pb.fmm_tree_build(ctx, X, 200)        # leaves above and below the thresholds of all three orders
+        assert pb.fmm_tree_info(tree).n_x > 0
+
+        def apply(t, p):
+            pb.fmm_apply_pair(ctx, t, KAPPA, p, o[0], o[1], q_lap=Q, q_yuk=Q)
+
+        apply(tree, 6)
+        pb.pb_sync(ctx)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            apply(tree, 6)
+        for p in (8, 4):
+            apply(tree, p)
+            other = pb.fmm_tree_build(ctx, X, 30)
+            apply(other, p)
+            pb.pb_sync(ctx)
+            pb.fmm_tree_destroy(other)
+            for a in o:
+                a.fill_(float("nan"))
+            torch.cuda.synchronize()
+            graph.replay()
+            torch.cuda.synchronize()
+            pb.pb_sync(ctx)
+            for a, r in zip(o, want):
+                assert rel_l2(a.cpu().numpy(), r) < 1e-5
+        del graph
+        pb.fmm_tree_destroy(tree)
+    finally:
+        pb.pb_destroy(ctx)
