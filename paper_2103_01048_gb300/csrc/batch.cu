@@ -539,10 +539,9 @@ void tune_fmm(pb_ctx* ctx, const float* xyz_dev, long long n, int p, const int* 
     cudaEventDestroy(a);
     cudaEventDestroy(b);
     ctx->leaf_nt = bnt;
-    ctx->m2l_tile = 0;               // one M2L row tile is left (128 pairs)
     *best = bc;
     if (best_nt) *best_nt = bnt;
-    if (best_tile) *best_tile = 0;
+    if (best_tile) *best_tile = 0;   // (one M2L row tile is left)
     if (best_ms) *best_ms = bestv;
 }
 

@@ -163,7 +163,6 @@ struct pb_ctx {
     int overlap = 0;           // 1: near field of the paired apply on `aux`, beside the far field
     int leaf_nt = 0;           // targets per thread of the paired leaf kernel (0: by precision)
     int leaf_packed = 1;       // FP32 paired leaf kernel with packed (f32x2) arithmetic
-    int m2l_tile = 0;          // PB_OPT_M2L_TILE: accepted, without effect
     int list_direct = 1;       // small W boxes and small leaves' X lists evaluated directly (packed path)
     int restart = 0;           // GMRES restart length of the batched solves (0: none)
     // second stream (and fork / join events) for the near field of the paired

@@ -1644,7 +1644,10 @@ static void gemm_launch(cudaStream_t st, int nblocks, const GemmArgs& a, const T
         case G_PAIRS: k_m2l_simt<T, TO, NPAD><<<nblocks, 256, 0, st>>>(a, ops, X, Y); break;
         case G_M2M: k_m2m<T, TO, NPAD><<<nblocks, 256, 0, st>>>(a, ops, X, Y); break;
         case G_L2L: k_l2l<T, TO, NPAD><<<nblocks, 256, 0, st>>>(a, ops, X, Y); break;
-        default: k_check2equiv<T, TO, NPAD><<<nblocks, 256, 0, st>>>(a, ops, X, Y); break;
+        default:                             // FP32 only: FP64 solves by k_box_pairs64
+            if constexpr (std::is_same<T, float>::value)
+                k_check2equiv<T, TO, NPAD><<<nblocks, 256, 0, st>>>(a, ops, X, Y);
+            break;
     }
     PB_CHECK_LAUNCH();
 }
@@ -1823,34 +1826,27 @@ static void far_dc2de_x(fmm_tree* Tr, const Operators& O, Work<T>& W, const XFar
 template <typename T>
 static void far_m2l(fmm_tree* Tr, const Operators& O, Work<T>& W) {
     pb_ctx* ctx = Tr->ctx;
-    bool tc_done = false;
-    if constexpr (std::is_same<T, float>::value) {
-        if (!ctx->deterministic)
-            tc_done = m2l_h_launch(Tr, O, nullptr, W.Qu.p, W.Qd.p, W.tmp.p, nullptr, nullptr, nullptr, ctx->dev_err,
-                                   ctx->stream);
-    }
-    if constexpr (std::is_same<T, double>::value) {
-        if (!ctx->deterministic) {
-            const auto& P = Tr->m2l_pairs;
+    const auto& P = Tr->m2l_pairs;
+    if (Tr->n_v == 0) return;
+    if (!ctx->deterministic) {
+        if constexpr (std::is_same<T, double>::value) {
             box_pairs64(O.npad, O.ne, P.items32.p, P.nitems32, 32, P.tgt.p, P.src.p, O.m2l_d.p, W.Qu.p, W.Qd.p,
                         ctx->stream);
-            return;
+        } else if (!m2l_h_launch(Tr, O, nullptr, W.Qu.p, W.Qd.p, W.tmp.p, nullptr, nullptr, nullptr, ctx->dev_err,
+                                 ctx->stream)) {
+            // one CTA per at most 32 V-list pairs of one (level, offset) group:
+            // parallel over pairs, so small trees fill the GPU too
+            GemmArgs ga = tree_gemm_args<T>(Tr);
+            ga.mode = G_PAIRS;
+            ga.pitems = P.items32.p;
+            ga.ptgt = P.tgt.p;
+            ga.psrc = P.src.p;
+            gemm_dispatch<T, T>(O.npad, ctx->stream, P.nitems32, ga, O.m2l.p, W.Qu.p, W.Qd.p);
         }
+        return;
     }
-    if (!tc_done && !ctx->deterministic && Tr->m2l_pairs.nitems32 > 0) {
-        // one CTA per at most 32 V-list pairs of one (level, offset) group:
-        // parallel over pairs, so small trees fill the GPU too
-        GemmArgs ga = tree_gemm_args<T>(Tr);
-        ga.mode = G_PAIRS;
-        ga.pitems = Tr->m2l_pairs.items32.p;
-        ga.ptgt = Tr->m2l_pairs.tgt.p;
-        ga.psrc = Tr->m2l_pairs.src.p;
-        gemm_dispatch<T, T>(O.npad, ctx->stream, Tr->m2l_pairs.nitems32, ga, opsel<T>(O, O.m2l, O.m2l_d), W.Qu.p,
-                            W.Qd.p);
-        tc_done = true;
-    }
-    if (!tc_done && Tr->n_v > 0) build_m2l_schedule(Tr);
-    if (!tc_done && Tr->m2l.ntile > 0) {
+    build_m2l_schedule(Tr);
+    if (Tr->m2l.ntile > 0) {
         GemmArgs ga = tree_gemm_args<T>(Tr);
         ga.mode = G_M2L;
         ga.tile_box = Tr->m2l.tile_box.p;

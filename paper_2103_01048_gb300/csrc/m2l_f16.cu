@@ -220,7 +220,7 @@ struct HArgs {
 
 template <int STAGES>
 struct HSmem {
-    uint64_t barB, bdone, full[STAGES], empty[STAGES], accf[2], acce[2];
+    uint64_t barB, full[STAGES], empty[STAGES], accf[2], acce[2];
     uint32_t tmem_slot;
     int failed;
 };
@@ -328,7 +328,6 @@ __global__ void __launch_bounds__(kHThreads, 1) k_m2l_f16(const HArgs A) {
 
     if (tid == 0) {
         mbar_init(&S->barB, 1);
-        mbar_init(&S->bdone, 1);
         for (int q = 0; q < STAGES; ++q) {
             mbar_init(&S->full[q], kHProdWarps);
             mbar_init(&S->empty[q], 1);

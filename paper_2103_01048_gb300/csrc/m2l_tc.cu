@@ -66,7 +66,7 @@ __device__ __forceinline__ float tf32_hi(float x) {
 // swizzled (nh = npad / NS output rows, KB = npad / KS / 32 blocks of 32
 // inner columns); the part a CTA owns is one contiguous block
 // ---------------------------------------------------------------------------
-__global__ void k_pack_m2l_tc(int npad, int NS, int KS, long long nmat, const float* __restrict__ m2l,
+__global__ void k_pack_box_ops(int npad, int NS, int KS, long long nmat, const float* __restrict__ m2l,
                               float* __restrict__ out) {
     long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const long long m2 = (long long)npad * npad;
@@ -89,7 +89,7 @@ static void pack_tc(int npad, long long nmat, const float* src, DBuf<float>& dst
     if (!tc_split(npad, ns, ks)) throw Error(PB_EINVAL, "no tensor-core split for this operator size");
     const long long m2 = (long long)npad * npad;
     dst.alloc(nmat * m2 * 2, st);
-    k_pack_m2l_tc<<<div_up(nmat * m2, 256), 256, 0, st>>>(npad, ns, ks, nmat, src, dst.p);
+    k_pack_box_ops<<<div_up(nmat * m2, 256), 256, 0, st>>>(npad, ns, ks, nmat, src, dst.p);
     PB_CHECK_LAUNCH();
 }
 
@@ -364,7 +364,7 @@ struct TcSets {
 };
 
 template <int NPAD>
-__global__ void __launch_bounds__(kTcThreads, 1) k_m2l_tc(const int4* __restrict__ items, const int* __restrict__ ptgt,
+__global__ void __launch_bounds__(kTcThreads, 1) k_box_ops_tc(const int4* __restrict__ items, const int* __restrict__ ptgt,
                                                           const int* __restrict__ psrc, const TcSets sets,
                                                           int* __restrict__ err) {
     // Generic tensor-core box-operator product: for every pair p of the
@@ -624,8 +624,8 @@ static void launch_tc_items(const int4* items, int nitems, const int* tgt, const
     dim3 grid(nitems * s2.sub, TcCfg<NPAD>::NS * TcCfg<NPAD>::KS, nsets);
     static bool done[64] = {false};
     const size_t sm = tc_smem_bytes<NPAD>();
-    smem_optin(k_m2l_tc<NPAD>, sm, done);
-    k_m2l_tc<NPAD><<<grid, kTcThreads, sm, st>>>(items, tgt, src, s2, err);
+    smem_optin(k_box_ops_tc<NPAD>, sm, done);
+    k_box_ops_tc<NPAD><<<grid, kTcThreads, sm, st>>>(items, tgt, src, s2, err);
     PB_CHECK_LAUNCH();
 }
 
