@@ -1147,8 +1147,11 @@ __device__ __forceinline__ void put_src_x2(ulonglong2* sA, ulonglong2* sB, ulong
 // and pair of thresholds, one warp per leaf; in the leaf kernel the lists
 // were seven dependent loads and a scan over every entry, 0.76 of 4.0 ms at
 // 4M points, p = 6.  Kept until the tree goes: captured graphs point to them.
+// Offsets: U + W below 2^32 in the record, the room for X entries by the leaf's
+// number in 64 bits (together past 2^31 from 74 million leaves on a curve; a
+// 64-bit offset in the record cost the apply 0.6% at 240,000 points).
 // ---------------------------------------------------------------------------
-static_assert(sizeof(LeafStream::Rec::near_off) == 8, "kXCap entries a leaf pass 2^31 at 74 million leaves on a curve");
+static_assert(std::is_unsigned<decltype(LeafStream::Rec::near_off)>::value, "U + W offset: up to 2^32");
 __global__ void __launch_bounds__(128) k_leaf_stream(
     int nleaf, const int* __restrict__ leaves, const int* __restrict__ tb, const int* __restrict__ te,
     const int* __restrict__ sb, const int* __restrict__ se, const int* __restrict__ U_off, const int* __restrict__ U_ids,
@@ -1231,8 +1234,9 @@ __global__ void __launch_bounds__(128) k_leaf_stream(
     if (lane == 0) {
         LeafStream::Rec r;
         r.t0 = t0; r.t1 = t1; r.nself = nself;
-        r.near_off = near_off; r.near_n = n;
+        r.near_off = (unsigned)u0 + (unsigned)w0; r.near_n = n;
         r.far_off = far_off; r.far_n = nf;
+        r.pad = 0;
         r.cx = cb.x; r.cy = cb.y; r.cz = cb.z;
         recs[li] = r;
     }
@@ -1335,7 +1339,8 @@ __global__ void __launch_bounds__(128, 5) k_leaf_pair_x2(const LeafStream::Rec* 
     const float kl2s = -kappa * float(kLog2E);
     const f32x2 kap = x2_pack(kappa, kappa), kl2 = x2_pack(kl2s, kl2s);
     auto load_near = [&](int v0) {
-        for (int v = threadIdx.x; v < min(nvirt - v0, VC); v += CH) s_v[v] = near_l[rec.near_off + v0 + v];
+        for (int v = threadIdx.x; v < min(nvirt - v0, VC); v += CH)
+            s_v[v] = near_l[(size_t)kXCap * blockIdx.x + (rec.near_off + (unsigned)(v0 + v))];
     };
     auto load_far = [&](int f0) {
         const int i = threadIdx.x;

@@ -67,9 +67,10 @@ struct LeafStream {
     struct Rec {
         int t0, t1;                // targets
         int nself;                 // the leaf's own sources (its first near range; 0: no such range)
-        int near_n;                // near: (first source, count)
-        long long near_off;        // (room for kXCap X entries a leaf: past 2^31 before the box count is)
+        unsigned near_off;         // U + W offset; the leaf's ranges start kXCap entries a leaf before it further
+        int near_n;                // near ranges (first source, count)
         int far_off, far_n;
+        int pad;
         double cx, cy, cz;         // centre of the leaf
     };
     DBuf<Rec> rec;
