@@ -34,8 +34,8 @@ METRIC = "FMM apply points/s (4M-point surface, Laplace+Yukawa SL+DL, p=6)"
 UNIT = "points/s"
 # dram__bytes_read.sum + dram__bytes_write.sum of one leaf launch
 # (k_leaf_pair_x2) on this workload (4M points, p = 6, ncrit = 128), from one
-# ncu capture of the current kernel; None where the current one has none
-LEAF_TRAFFIC_BYTES = None
+# ncu capture of the current kernel (509.3 + 28.8 MB); None once the kernel changes
+LEAF_TRAFFIC_BYTES = 538.1e6
 # Arithmetic of one source-target pair in the paired (Laplace + Yukawa)
 # evaluation, FMA = 2 FLOPs, MUFU counted apart: SL+DL of both kernels
 # 30 FLOPs + 2 MUFU (rsqrt, ex2); monopole-only pairs of equivalent
@@ -730,8 +730,8 @@ def main():
                     "note": "achieved = 2 n_e^2 x V-list pairs x 2 kernels / M2L phase time; issued_frac counts "
                             "the 3 half-precision products (hi*hi, hi*lo, lo*hi) at the padded size n_pad actually issued; "
                             "frac_of_fp32_accurate_roof divides by that rate / 3, the rate of a contraction that "
-                            "keeps FP32 accuracy with three products of 11-bit halves; the kernel is bound by "
-                            "the L2's reductions into the target rows"}
+                            "keeps FP32 accuracy with three products of 11-bit halves; the kernel waits for its "
+                            "producers' gathers of source rows from L2, beside the reductions into the target rows"}
 
     clocks = clk.summary()
 

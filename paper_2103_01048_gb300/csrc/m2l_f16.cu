@@ -17,17 +17,20 @@
 // significant bits at twice its rate and half its bytes; its range is no
 // limit because every source row and every operator is scaled by a power of
 // two to a largest entry in [2^14, 2^15) first (undone exactly in the
-// epilogue).  hi + lo then hold an entry to 2^-23 relative, or 2^-40 of the
-// row's largest where lo leaves the normal range; the TF32 split that this
-// replaces kept 2^-21 (lo truncated to 11 bits).
+// epilogue).  hi + lo then hold an entry to 2^-23 relative, or 2^-39 of the
+// row's largest where lo leaves the normal range (spacing 2^-24, largest
+// entry at least 2^14); the TF32 split that this replaces kept 2^-21 (lo
+// truncated to 11 bits) of every entry.
 //
 // Layout: a K block is 32 columns; its row is 128 B = [32 hi halves | 32 lo
 // halves], 128B-swizzled in shared memory.
 //
-// Bound: the reductions into Qd.  They cost n_e * 4 B per pair at the L2's
-// rate for them (measured on random rows: 5.9 TB/s for 64-byte pieces of
-// red.v4; 16-byte pieces 3.3, 32-byte 4.2).  At p = 8 and 10 the MMAs (three
-// products) take as long.  Before (TF32, one operator per offset, CTA pairs)
+// Floor: the reductions into Qd, n_e * 4 B per pair at the L2's rate for them
+// (measured on random rows: 5.9 TB/s for 64-byte pieces of red.v4; 16-byte
+// pieces 3.3, 32-byte 4.2); at p = 8 and 10 the MMAs (three products) take as
+// long.  What bounds it: the producers' gathers of source rows from L2, two K
+// blocks in flight (at 1M points, p = 6, long-scoreboard stalls lead, the
+// tensor pipe is active 33% of the time and the L2 is 45% busy).  Before (TF32, one operator per offset, CTA pairs)
 // -> now, both kernels: p = 4, 3M points 1.35 -> 0.62 ms; p = 6, 15,000 0.18
 // -> 0.03, 240,000 0.40 -> 0.14, 4M 2.74 -> 1.62; p = 8, 500,000 1.98 -> 0.85;
 // p = 10, 197,000 3.19 -> 1.01.

@@ -7,7 +7,8 @@
 // quantisation with correctly rounded operations -> stable radix sort of
 // (key, index) -> level-synchronous box splitting -> box centres ->
 // colleague / V / X lists top-down -> U / W lists of leaves by a bounded
-// depth-first search -> per-tile M2L schedule.
+// depth-first search -> pair lists (the fixed-order M2L takes a schedule, built
+// on its first use).
 #include "tree.cuh"
 #include <cub/cub.cuh>
 #include <algorithm>
