@@ -29,7 +29,7 @@ bool c2e_tc_launch2(const fmm_tree* T, const Operators& O, const Operators* O2, 
                     float* tmp, const float* X2, float* Y2, float* tmp2, int* err, cudaStream_t st,
                     const XFar* far = nullptr);
 // X-list boxes that keep P2L when small leaves sum their X lists directly
-bool c2e_tc_ok(const Operators& O);
+bool c2e_tc_ok(const fmm_tree* T, const Operators& O);
 const XFar* build_xbox_far(fmm_tree* T, int thrX);
 void build_m2l_schedule(fmm_tree* T);
 
@@ -2003,7 +2003,7 @@ static void apply_t(fmm_tree* Tr, const Operators& O, double kappa_d, const In* 
     // P2L: X-list sources -> downward check -> DC2DE, per level
     if (Tr->n_xbox > 0) {
         const XFar* far = nullptr;
-        if (std::is_same<T, float>::value && thrX >= 0 && c2e_tc_ok(O)) far = build_xbox_far(Tr, thrX);
+        if (std::is_same<T, float>::value && thrX >= 0 && c2e_tc_ok(Tr, O)) far = build_xbox_far(Tr, thrX);
         const int nx = far ? far->n : Tr->n_xbox;
         const int* xids = far ? far->ids.p : Tr->xbox_ids.p;
         if (DL) launch_p2check<T, YUK, true>(st, nx, xids, 1, Tr, W, O, kappa, thrX);
@@ -2210,7 +2210,7 @@ static void apply_pair_t(fmm_tree* Tr, const Operators& OL, const Operators& OY,
         // with the small leaves' X lists summed in the leaf kernel, P2L and its
         // solve run on the other X-list boxes only (tensor-core solve path)
         const XFar* far = nullptr;
-        if (std::is_same<T, float>::value && thrX >= 0 && c2e_tc_ok(OL) && c2e_tc_ok(OY))
+        if (std::is_same<T, float>::value && thrX >= 0 && c2e_tc_ok(Tr, OL) && c2e_tc_ok(Tr, OY))
             far = build_xbox_far(Tr, thrX);
         const int nx = far ? far->n : Tr->n_xbox;
         const int* xids = far ? far->ids.p : Tr->xbox_ids.p;

@@ -677,7 +677,12 @@ bool pc_tc_launch(const fmm_tree* T, const Operators& O, int child_level, bool u
 // 10 the operator's inner parts add into tmp (zeroed first) and into Y, whose
 // rows of those boxes must be zero on entry. One operator set, or two (O2, X2, Y2, tmp2)
 // in the same launches. False when the tensor-core path does not apply.
-bool c2e_tc_ok(const Operators& O) { return tc_ok(O) && O.uc2ue_w1_tc.p; }
+// In the fixed-order mode not with more than two inner parts (p = 10): two
+// added to zero give the same bits in either order, four do not.
+bool c2e_tc_ok(const fmm_tree* T, const Operators& O) {
+    int parts = 0, ks = 0;
+    return tc_ok(O) && O.uc2ue_w1_tc.p && tc_split(O.npad, parts, ks) && !(T->ctx->deterministic && ks > 2);
+}
 
 // The X-list boxes that keep P2L at a direct-list threshold (see the
 // field comment in fmm_tree), with their check -> equivalent items; once per
@@ -715,8 +720,8 @@ const XFar* build_xbox_far(fmm_tree* T, int thrX) {
 bool c2e_tc_launch2(const fmm_tree* T, const Operators& O, const Operators* O2, bool up, const float* X, float* Y,
                     float* tmp, const float* X2, float* Y2, float* tmp2, int* err, cudaStream_t st,
                     const XFar* far) {
-    if (!tc_ok(O) || !O.uc2ue_w1_tc.p) return false;
-    if (O2 && (!tc_ok(*O2) || !O2->uc2ue_w1_tc.p || O2->npad != O.npad)) return false;
+    if (!c2e_tc_ok(T, O)) return false;
+    if (O2 && (!c2e_tc_ok(T, *O2) || O2->npad != O.npad)) return false;
     const int nitems = up ? T->n_c2e_up : (far ? far->nitems : T->n_c2e_dn);
     if (nitems == 0) return true;
     const int4* items = up ? T->c2e_items_up.p : (far ? far->items.p : T->c2e_items_dn.p);
